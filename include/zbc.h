@@ -74,9 +74,16 @@ typedef enum { ZBC_C64 = 0, ZBC_C128 = 1 } zbc_dtype;
  *             (M = 128 voxels, N = 2 x 16 .. 2 x 128 right-hand sides, 3 products, FP32
  *             accumulation folded into an FP32 sum in tensor memory every 64 columns).
  * AUTO      : the form (and CTA shape) zbc_tune measured fastest for this handle and this
- *             right-hand-side class; before any tuning, BF16X3 for the forward product when
- *             p >= 8 and FP32_SIMT otherwise.  Every form meets the same 1e-5 relative accuracy,
- *             but their last bits differ, so AUTO results depend on the tuning. */
+ *             right-hand-side class; before any tuning, the joint form where the handle has it,
+ *             else BF16X3 for the forward product when p >= 8 and FP32_SIMT.  Every form meets the
+ *             same 1e-5 relative accuracy, but their last bits differ, so AUTO results depend on
+ *             the tuning.
+ * The joint form (AUTO only): where the factors of all stored columns share small orthonormal bases
+ *             B_1, B_2, B_3 per component (each tensor represented to 1e-7 of its norm, below the
+ *             rounding of its complex64 factors), Z_j = K_j x1 B_1 x2 B_2 x3 B_3 with cores K_j in
+ *             the bases, and the products sum over the columns' cores and pass between the cores
+ *             and the grid once per right-hand side.  The bases and cores are built on the first
+ *             AUTO or zbc_tune call (not during a stream capture) and kept with the handle. */
 typedef enum {
   ZBC_FP32_SIMT = 0,
   ZBC_TF32X3 = 1,
@@ -435,6 +442,7 @@ int zbc_rmatvec_noalloc(const zbc_handle* h, const void* Phi, int64_t ldphi, int
  * handle with p right-hand sides (zero-filled scratch operands), every variant of
  *   zbc_matvec : FP32_SIMT with 6 and with 9 compute warps per CTA, TF32X3, BF16X3, TC2, TC_MODE1, TC_DC
  *   zbc_rmatvec: FP32_SIMT with 6 and with 9 compute warps per CTA, TC_MODE1
+ * (and the joint form of both where the handle has it; its times are not returned)
  * and records the fastest of each for p's right-hand-side class (p = 1, 2, 3-4, 5-8, 9-16,
  * 17-32, 33-64, 65+), which ZBC_AUTO then uses (zbc_rmatvec_noalloc uses the faster SIMT shape).
  * Each variant runs once untimed, then is timed over two calls, or over one when that call took

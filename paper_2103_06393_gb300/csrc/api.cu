@@ -45,6 +45,7 @@ Handle::~Handle() {
   if (d_desc) cudaFree(d_desc);
   if (d_v) cudaFree(d_v);
   if (cache) cache_release(cache);
+  if (joint) joint_release(joint);
 }
 
 int Handle::upload() {
@@ -129,6 +130,10 @@ int handle_append(Handle* h, const std::vector<int32_t>& ranks, const float2* d_
     cache_release(h->cache);
     h->cache = nullptr;
   }
+  if (h->joint) {
+    joint_release(h->joint);
+    h->joint = nullptr;
+  }
   return finish_desc(h);
 }
 
@@ -184,10 +189,10 @@ extern "C" int zbc_device_bytes(const zbc_handle* hh, int64_t* pool, int64_t* ca
   if (pool)
     *pool = (int64_t)(sizeof(float2) * h.pool_elems + sizeof(TensorDesc) * h.desc.size() +
                       (h.has_v ? sizeof(float2) * (size_t)h.m * h.M : 0));
-  if (caches) *caches = cache_bytes(h.cache);
+  if (caches) *caches = cache_bytes(h.cache) + joint_bytes(h.joint);
   if (work)
     *work = (int64_t)(h.work_partial.bytes + h.work_x.bytes + h.work_misc.bytes + h.work_xt.bytes +
-                      h.work_err.bytes + h.work_phi.bytes);
+                      h.work_err.bytes + h.work_phi.bytes + h.work_joint.bytes);
   return ZBC_OK;
 }
 

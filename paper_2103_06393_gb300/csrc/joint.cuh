@@ -1,0 +1,52 @@
+// Joint-subspace form of the products (joint_build.cu, products_joint.cu).
+//
+// Every stored column of component k is Z^{kj} = G x1 U1 x2 U2 x3 U3 with factors of its own, but
+// the factors of all columns are fields of the same domain and span few directions together (the
+// 96^3 head-coil workload: 47-52 directions per axis for 1024 columns of rank 11; the 1 mm grid:
+// 23-25 of 320).  With an orthonormal basis B_g (n_g x R_g) of that span per component and mode,
+//   Z^{kj} = K^{kj} x1 B1 x2 B2 x3 B3,   K^{kj} = G x1 (B1^H U1) x2 (B2^H U2) x3 (B3^H U3),
+// so  Y^k = (sum_j K^{kj} X[j, :]) x1 B1 x2 B2 x3 B3  and the adjoint is its transpose: the sum
+// over the columns runs over R1 R2 R3 entries instead of n1 n2 n3 voxels, and the expansion to the
+// grid is done once per right-hand side instead of once per column.  This is the same operator to
+// the tolerance kJointEps, which is below the rounding of the complex64 tensors.
+#pragma once
+
+#include "zbc_internal.cuh"
+
+namespace zbc {
+
+constexpr int kJointQ = 12;      // components of a handle (q <= 12)
+constexpr int kJointRmax = 64;   // largest R_g
+// largest residual of a tensor's weighted factor outside the basis, relative to its norm.  The
+// complex64 rounding of the factors is 6e-8 of their norm; at 1e-7 the products' error against
+// 64 bits is that of their FP32 sums.
+constexpr double kJointEps = 1e-7;
+
+struct JointGeo {
+  int n1, n2, n3, q, M;
+  int R[kJointQ][3];
+  int Cs[kJointQ];        // R1 R2 R3 rounded up to 4 (row stride of K)
+  int64_t koff[kJointQ];  // component k's rows [j][Cs] in K
+  int64_t boff[kJointQ][3];  // B_g in the basis array: column r at boff + r n_g
+  int64_t toff[kJointQ];  // component k's entries in one right-hand side of T / F
+  int64_t qoff[kJointQ];  // component k's planes [i3][R1 R2] in one right-hand side of Q
+  int64_t Ct, Qt;         // entries of one right-hand side of T / F and of Q
+};
+
+struct JointCache {
+  bool usable = false;    // false: the factors share no small basis (the other forms are used)
+  bool large = false;     // the products decompress more than 1e8 voxel ranks
+  JointGeo geo;
+  float2* basis = nullptr;
+  float2* K = nullptr;
+  int64_t bytes = 0;
+};
+
+// Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
+int build_joint(Handle& h, cudaStream_t st);
+// bytes of h.work_joint that one product of p right-hand sides uses (h.joint usable)
+size_t joint_work_bytes(const Handle& h, int p, bool fwd);
+int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st);
+int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* out, int64_t ldo, cudaStream_t st);
+
+}  // namespace zbc

@@ -4,6 +4,7 @@
 #include <cmath>
 
 #include "decomp.cuh"
+#include "joint.cuh"
 #include "zbc_internal.cuh"
 
 namespace zbc {
@@ -15,6 +16,35 @@ int matvec_dc(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t
 int aca_pre(const Handle& h, const float2* X, int64_t ldx, int p, float2* Xp, cudaStream_t st);
 int aca_post(const Handle& h, const float2* Psip, int p, float2* Psi, int64_t ldpsi, cudaStream_t st);
 
+// The joint-subspace form (joint.cuh): chosen by ZBC_AUTO only, so it has no zbc_precision of its own.
+constexpr zbc_precision kFormJoint = (zbc_precision)7;
+
+// Whether ZBC_AUTO can run the joint form: the basis is built on the first call that asks for it.
+// During a stream capture nothing is built or grown; the other forms then run as they did.
+static bool joint_ready(Handle& h, int p, bool fwd, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cap != cudaStreamCaptureStatusNone)
+    return h.joint && h.joint->usable && h.work_joint.bytes >= joint_work_bytes(h, p, fwd);
+  if (!h.joint && build_joint(h, st) != ZBC_OK) {
+    clear_error();
+    cudaGetLastError();
+  }
+  return h.joint && h.joint->usable;
+}
+
+// The form of ZBC_AUTO: the tuned one; untuned, the joint form where the handle has it, else BF16X3
+// for a forward product of p >= 8 and FP32_SIMT.
+static zbc_precision auto_form(Handle& h, int p, bool fwd, cudaStream_t st) {
+  const int tuned = fwd ? h.tune_fwd_prec[rhs_class(p)] : h.tune_adj_prec[rhs_class(p)];
+  if (tuned >= 0 && tuned != kFormJoint) return (zbc_precision)tuned;
+  if (joint_ready(h, p, fwd, st)) return kFormJoint;
+  return fwd && p >= 8 ? ZBC_BF16X3 : ZBC_FP32_SIMT;
+}
+
 // Y = Z X with an explicit form (prec != AUTO) and SIMT CTA shape
 static int matvec_impl(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, zbc_precision prec,
                        int warps, cudaStream_t st) {
@@ -25,6 +55,10 @@ static int matvec_impl(Handle& h, const float2* X, int64_t ldx, int p, float2* Y
     ZBC_TRY(aca_pre(h, X, ldx, p, (float2*)h.work_x.ptr, st));
     Xe = (const float2*)h.work_x.ptr;
     ldxe = h.M;
+  }
+  if (prec == kFormJoint) {
+    ZBC_TRY(build_decomp_cache(h, st));  // the error word, and the cache zbc_rmatvec_noalloc needs
+    return matvec_joint(h, Xe, ldxe, p, Y, ldy, st);
   }
   if (prec == ZBC_FP32_SIMT) return matvec_simt(h, Xe, ldxe, p, Y, ldy, warps, st);
   if (prec == ZBC_TC2) return matvec_tc2(h, Xe, ldxe, p, Y, ldy, st);
@@ -43,7 +77,10 @@ static int rmatvec_impl(Handle& h, const float2* Phi, int64_t ldphi, int p, floa
     out = (float2*)h.work_x.ptr;
     ldo = h.M;
   }
-  if (prec == ZBC_TC_MODE1)
+  if (prec == kFormJoint) {
+    ZBC_TRY(build_decomp_cache(h, st));
+    ZBC_TRY(rmatvec_joint(h, Phi, ldphi, p, out, ldo, st));
+  } else if (prec == ZBC_TC_MODE1)
     ZBC_TRY(rmatvec_mode1(h, Phi, ldphi, p, out, ldo, st));
   else
     ZBC_TRY(rmatvec_simt(h, Phi, ldphi, p, out, ldo, warps, st));
@@ -67,8 +104,7 @@ extern "C" int zbc_matvec(const zbc_handle* hh, const void* X, int64_t ldx, int 
                 "unknown precision %d", (int)prec);
   const int cls = rhs_class(p);
   int warps = h.tune_fwd_warps[cls];
-  if (prec == ZBC_AUTO)
-    prec = h.tune_fwd_prec[cls] >= 0 ? (zbc_precision)h.tune_fwd_prec[cls] : (p >= 8 ? ZBC_BF16X3 : ZBC_FP32_SIMT);
+  if (prec == ZBC_AUTO) prec = auto_form(h, p, true, (cudaStream_t)stream);
   return matvec_impl(h, (const float2*)X, ldx, p, (float2*)Y, ldy, prec, warps, (cudaStream_t)stream);
 }
 
@@ -86,7 +122,7 @@ extern "C" int zbc_rmatvec(const zbc_handle* hh, const void* Phi, int64_t ldphi,
   ZBC_CHECK_ARG(prec == ZBC_FP32_SIMT || prec == ZBC_AUTO || prec == ZBC_TC_MODE1,
                 "the adjoint product's forms are ZBC_FP32_SIMT, ZBC_TC_MODE1 and ZBC_AUTO");
   const int cls = rhs_class(p);
-  if (prec == ZBC_AUTO) prec = h.tune_adj_prec[cls] >= 0 ? (zbc_precision)h.tune_adj_prec[cls] : ZBC_FP32_SIMT;
+  if (prec == ZBC_AUTO) prec = auto_form(h, p, false, (cudaStream_t)stream);
   return rmatvec_impl(h, (const float2*)Phi, ldphi, p, (float2*)Psi, ldpsi, prec, h.tune_adj_warps[cls],
                       (cudaStream_t)stream);
 }
@@ -97,11 +133,12 @@ extern "C" int zbc_rmatvec(const zbc_handle* hh, const void* Phi, int64_t ldphi,
 static void release_unused_operands(Handle& h) {
   DecompCache* c = h.cache;
   if (!c) return;
-  bool m1f = false, m1a = false, dc = false, tc2 = false;
+  bool m1f = false, m1a = false, dc = false, tc2 = false, joint = false;
   for (int i = 0; i < Handle::kPClasses; ++i) {
     m1f = m1f || h.tune_fwd_prec[i] == ZBC_TC_MODE1;
     dc = dc || h.tune_fwd_prec[i] == ZBC_TC_DC;
     tc2 = tc2 || h.tune_fwd_prec[i] == ZBC_TC2;
+    joint = joint || h.tune_fwd_prec[i] == kFormJoint || h.tune_adj_prec[i] == kFormJoint;
     m1a = m1a || h.tune_adj_prec[i] == ZBC_TC_MODE1;
   }
   if (c->mode1 && !m1f) mode1_fwd_release(c->mode1);
@@ -114,6 +151,10 @@ static void release_unused_operands(Handle& h) {
     c->dc = nullptr;
   }
   if (!tc2) half_release(c);
+  if (!joint && h.joint && h.joint->usable) {
+    joint_release(h.joint);
+    h.joint = nullptr;
+  }
 }
 
 extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_ms_host) {
@@ -139,17 +180,18 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
     int warps;
   };
   constexpr int NV = 10, NF = 7;  // the first NF variants are forward forms
-  const Variant vars[NV] = {{true, ZBC_FP32_SIMT, 6},  {true, ZBC_FP32_SIMT, 9},  {true, ZBC_TF32X3, 0},
+  constexpr int NT = NV + 2;      // and the joint form of both directions, whose times are not returned
+  const Variant vars[NT] = {{true, ZBC_FP32_SIMT, 6},  {true, ZBC_FP32_SIMT, 9},  {true, ZBC_TF32X3, 0},
                             {true, ZBC_BF16X3, 0},     {true, ZBC_TC2, 0},        {true, ZBC_TC_MODE1, 0},
                             {true, ZBC_TC_DC, 0},      {false, ZBC_FP32_SIMT, 6}, {false, ZBC_FP32_SIMT, 9},
-                            {false, ZBC_TC_MODE1, 0}};
-  // timing order: the tensor-core forms first, so that a slower form can be dropped after one
-  // timed call once it is 1.5 times slower than the best of its direction so far
-  const int order[NV] = {5, 6, 2, 3, 4, 0, 1, 9, 8, 7};
-  float t[NV];
+                            {false, ZBC_TC_MODE1, 0}, {true, kFormJoint, 0},      {false, kFormJoint, 0}};
+  // timing order: the joint and the tensor-core forms first, so that a slower form can be dropped
+  // after one timed call once it is 1.5 times slower than the best of its direction so far
+  const int order[NT] = {10, 5, 6, 2, 3, 4, 0, 1, 11, 9, 8, 7};
+  float t[NT];
   float best[2] = {INFINITY, INFINITY};
   int status = ZBC_OK;
-  for (int oi = 0; oi < NV && status == ZBC_OK; ++oi) {
+  for (int oi = 0; oi < NT && status == ZBC_OK; ++oi) {
     const int i = order[oi];
     const Variant& v = vars[i];
     auto run = [&]() {
@@ -157,7 +199,7 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
                    : rmatvec_impl(h, (const float2*)Phi.ptr, rows, p, (float2*)Psi.ptr, h.m, v.prec, v.warps, st);
     };
     t[i] = INFINITY;
-    if (run() != ZBC_OK) {  // a form that does not fit this handle is skipped
+    if ((v.prec == kFormJoint && !joint_ready(h, p, v.fwd, st)) || run() != ZBC_OK) {  // a form that does not fit this handle is skipped
       clear_error();
       continue;
     }
@@ -193,6 +235,13 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
     if (t[i] < t[bf]) bf = i;
   for (int i = NF + 1; i < NV; ++i)
     if (t[i] < t[ba]) ba = i;
+  // a small handle takes the joint form for both directions or for none, so that it does not keep
+  // the reduced cores beside another form's operands
+  const bool jf = t[NV] < t[bf], ja = t[NV + 1] < t[ba];
+  if (h.joint && (h.joint->large || (jf && ja))) {
+    if (jf) bf = NV;
+    if (ja) ba = NV + 1;
+  }
   if (!(t[bf] < INFINITY) || !(t[ba] < INFINITY)) {
     set_error("zbc_tune: no product form fits this handle");
     return ZBC_EINVAL;

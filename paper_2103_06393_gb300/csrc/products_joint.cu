@@ -1,0 +1,644 @@
+// The products through a joint basis of the columns' factors (joint.cuh), FP32 on CUDA cores.
+//
+// Forward:  T = sum_j K_j X[j, :]        joint_core_fwd_kernel    (R1 R2 R3 entries per component)
+//           Q[i3] = T x3 B3              joint_mode3_fwd_kernel
+//           Y[:, :, i3] = B1 Q[i3] B2^T  joint_plane_fwd_kernel   (one write of Y)
+// Adjoint:  Q[i3] = B1^H Phi[:, :, i3] conj(B2)   joint_plane_adj_kernel   (one read of Phi)
+//           F = Q x3 B3^H                         joint_mode3_adj_kernel
+//           Psi[j, :] = sum conj(K_j) F           joint_core_adj_kernel, joint_sum_kernel
+#include <algorithm>
+
+#include "decomp.cuh"
+#include "joint.cuh"
+
+namespace zbc {
+namespace {
+
+constexpr int kJc = 64;  // columns of X per shared-memory chunk of the forward core sum
+
+__device__ __forceinline__ bool finite2(float2 v) { return isfinite(v.x) && isfinite(v.y); }
+
+// T[js][s][toff + c] = sum over columns j of slice js of K[j][c] X[j, s]; two c per thread.
+// Grid (c blocks of 256, slices, q * passes of P right-hand sides).
+template <int P>
+__global__ void __launch_bounds__(128) joint_core_fwd_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ K,
+                                                             const float2* __restrict__ X, int64_t ldx, int p, int JS,
+                                                             float2* __restrict__ T, int* __restrict__ err) {
+  __shared__ __align__(16) float2 xs[kJc][P];
+  const int k = blockIdx.z % G.q, s0 = blockIdx.z / G.q * P;
+  const int c = 2 * (blockIdx.x * 128 + threadIdx.x);
+  if (2 * blockIdx.x * 128 >= G.Cs[k]) return;
+  const bool live = c < G.Cs[k];
+  const int per = (G.M + JS - 1) / JS;
+  const int j0 = blockIdx.y * per, j1 = min(G.M, j0 + per);
+  const int64_t cs = G.Cs[k];
+  const float2* Kp = K + G.koff[k] + (live ? c : 0);
+  float2 acc[2][P];
+#pragma unroll
+  for (int s = 0; s < P; ++s) acc[0][s] = acc[1][s] = make_float2(0.f, 0.f);
+  bool bad = false;
+  for (int jb = j0; jb < j1; jb += kJc) {
+    const int nj = min(kJc, j1 - jb);
+    __syncthreads();
+    for (int e = threadIdx.x; e < kJc * P; e += 128) {
+      const int jj = e % kJc, s = e / kJc;
+      float2 v = make_float2(0.f, 0.f);
+      if (jj < nj && s0 + s < p) v = X[jb + jj + ldx * (s0 + s)];
+      bad = bad || !finite2(v);
+      xs[jj][s] = v;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int jj = 0; jj < nj; ++jj) {
+      const float4 kv = __ldcs((const float4*)(Kp + (jb + jj) * cs));
+#pragma unroll
+      for (int s = 0; s < P; ++s) {
+        const float2 x = xs[jj][s];
+        acc[0][s] = cfma(make_float2(kv.x, kv.y), x, acc[0][s]);
+        acc[1][s] = cfma(make_float2(kv.z, kv.w), x, acc[1][s]);
+      }
+    }
+  }
+  if (bad) atomicOr(err, kErrNonFinite);
+  if (!live) return;
+#pragma unroll
+  for (int s = 0; s < P; ++s)
+    if (s0 + s < p) {
+      float2* o = T + ((int64_t)blockIdx.y * p + s0 + s) * G.Ct + G.toff[k] + c;
+      *(float4*)o = make_float4(acc[0][s].x, acc[0][s].y, acc[1][s].x, acc[1][s].y);
+    }
+}
+
+constexpr int kZ = 16;  // values of i3 (forward) or of the third core index (adjoint) per thread
+
+// Q[s][qoff + i3 RR + xy] = sum_z B3[i3, z] sum_js T[js][s][toff + xy + RR z]
+__global__ void __launch_bounds__(128) joint_mode3_fwd_kernel(const __grid_constant__ JointGeo G,
+                                                              const float2* __restrict__ basis, const float2* __restrict__ T,
+                                                              int p, int JS, float2* __restrict__ Q) {
+  __shared__ float2 b3[kJointRmax][kZ];
+  const int k = blockIdx.z % G.q, s = blockIdx.z / G.q, R3 = G.R[k][2];
+  const int RR = G.R[k][0] * G.R[k][1];
+  if ((int)blockIdx.x * 128 >= RR) return;
+  const int z0 = blockIdx.y * kZ, xy = blockIdx.x * 128 + threadIdx.x;
+  for (int e = threadIdx.x; e < R3 * kZ; e += 128) {
+    const int zz = e % kZ, r = e / kZ;
+    b3[r][zz] = z0 + zz < G.n3 ? basis[G.boff[k][2] + (int64_t)r * G.n3 + z0 + zz] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  if (xy >= RR) return;
+  float2 acc[kZ];
+#pragma unroll
+  for (int z = 0; z < kZ; ++z) acc[z] = make_float2(0.f, 0.f);
+  const float2* Ts = T + (int64_t)s * G.Ct + G.toff[k] + xy;
+#pragma unroll 2
+  for (int r = 0; r < R3; ++r) {
+    float2 t = Ts[(int64_t)r * RR];
+    for (int js = 1; js < JS; ++js) {
+      const float2 u = Ts[(int64_t)js * p * G.Ct + (int64_t)r * RR];
+      t.x += u.x;
+      t.y += u.y;
+    }
+#pragma unroll
+    for (int z = 0; z < kZ; ++z) acc[z] = cfma(t, b3[r][z], acc[z]);
+  }
+  float2* o = Q + (int64_t)s * G.Qt + G.qoff[k] + xy;
+#pragma unroll
+  for (int z = 0; z < kZ; ++z)
+    if (z0 + z < G.n3) o[(int64_t)(z0 + z) * RR] = acc[z];
+}
+
+constexpr int kI2 = 32;  // i2 values of a plane tile (forward)
+
+inline size_t plane_fwd_smem(int R1, int R2, int NI) {
+  return sizeof(float2) * ((size_t)R1 * 32 * NI + (size_t)R1 * kI2 + (size_t)R1 * R2 + (size_t)R2 * kI2);
+}
+
+// Y[i1, i2, i3, s] = sum_xy B1[i1, x] Q[s][i3][x, y] B2[i2, y]: a CTA keeps B1 of its block of
+// 32 NI rows in shared memory and walks (s, i3, tile of 32 i2): S = Q B2^T of the tile (R1 x 32),
+// then B1 S, one thread NI i1 (stride 32) x 4 i2.  Grid (walkers, i1 blocks, q).
+template <int NI>
+__global__ void __launch_bounds__(256) joint_plane_fwd_kernel(const __grid_constant__ JointGeo G,
+                                                              const float2* __restrict__ basis, const float2* __restrict__ Q,
+                                                              int p, float2* __restrict__ Y, int64_t ldy) {
+  extern __shared__ __align__(16) float2 sm[];
+  const int k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1], RR = R1 * R2;
+  constexpr int BW = 32 * NI;
+  float2* b1 = sm;                // [R1][BW]
+  float2* ss = b1 + R1 * BW;      // [R1][kI2]
+  float2* b2 = ss + R1 * kI2;     // [R2][kI2]
+  float2* qs = b2 + R2 * kI2;     // [R2][R1]
+  const int i10 = blockIdx.y * BW, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int e = threadIdx.x; e < R1 * BW; e += 256) {
+    const int il = e % BW, x = e / BW;
+    b1[e] = i10 + il < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i10 + il] : make_float2(0.f, 0.f);
+  }
+  const int nt2 = (G.n2 + kI2 - 1) / kI2;
+  const int64_t items = (int64_t)p * G.n3 * nt2;
+  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const int i20 = (int)(it % nt2) * kI2;
+    const int i3 = (int)(it / nt2 % G.n3), s = (int)(it / nt2 / G.n3);
+    const float2* Qp = Q + (int64_t)s * G.Qt + G.qoff[k] + (int64_t)i3 * RR;
+    __syncthreads();
+    for (int e = threadIdx.x; e < RR; e += 256) qs[e] = Qp[e];
+    for (int e = threadIdx.x; e < R2 * kI2; e += 256) {
+      const int il = e % kI2, y = e / kI2;
+      b2[e] = i20 + il < G.n2 ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i20 + il] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < R1 * (kI2 / 4); e += 256) {
+      const int x = e % R1, i4 = e / R1 * 4;
+      float2 a[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[u] = make_float2(0.f, 0.f);
+      for (int y = 0; y < R2; ++y) {
+        const float2 v = qs[x + R1 * y];
+        const float4 c0 = *(const float4*)&b2[y * kI2 + i4], c1 = *(const float4*)&b2[y * kI2 + i4 + 2];
+        a[0] = cfma(v, make_float2(c0.x, c0.y), a[0]);
+        a[1] = cfma(v, make_float2(c0.z, c0.w), a[1]);
+        a[2] = cfma(v, make_float2(c1.x, c1.y), a[2]);
+        a[3] = cfma(v, make_float2(c1.z, c1.w), a[3]);
+      }
+      *(float4*)&ss[x * kI2 + i4] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+      *(float4*)&ss[x * kI2 + i4 + 2] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+    }
+    __syncthreads();
+    float2 acc[NI][4];
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[i][u] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int x = 0; x < R1; ++x) {
+      const float4 c0 = *(const float4*)&ss[x * kI2 + 4 * warp], c1 = *(const float4*)&ss[x * kI2 + 4 * warp + 2];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const float2 b = b1[x * BW + lane + 32 * i];
+        acc[i][0] = cfma(b, make_float2(c0.x, c0.y), acc[i][0]);
+        acc[i][1] = cfma(b, make_float2(c0.z, c0.w), acc[i][1]);
+        acc[i][2] = cfma(b, make_float2(c1.x, c1.y), acc[i][2]);
+        acc[i][3] = cfma(b, make_float2(c1.z, c1.w), acc[i][3]);
+      }
+    }
+    float2* Yp = Y + ldy * s + (int64_t)k * nv + (int64_t)G.n1 * (i20 + 4 * warp + (int64_t)G.n2 * i3) + i10 + lane;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i20 + 4 * warp + u < G.n2)
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+          if (i10 + lane + 32 * i < G.n1) __stcs(Yp + (int64_t)G.n1 * u + 32 * i, acc[i][u]);
+  }
+}
+
+constexpr int kA2 = 64;       // i2 values of a plane tile (adjoint)
+constexpr int kA1 = 32;       // i1 values per chunk
+constexpr int kPs = kA2 + 2;  // row strides: 16-byte aligned rows, stores over i1 spread over the banks
+
+// Q[s][i3][x, y] = sum over i1, i2 of conj(B1[i1, x]) conj(B2[i2, y]) Phi[i1, i2, i3, s]: one CTA per
+// plane (i3, s, k).  Per tile of 64 i2: V = B1^H Phi over i1 chunks of 32 (a thread holds RA x by
+// 4 i2), then Q += V conj(B2) (RA x by RB y, kept in registers over the tiles).  Grid (n3, p, q).
+template <int RA, int RB>
+__global__ void __launch_bounds__(128) joint_plane_adj_kernel(const __grid_constant__ JointGeo G,
+                                                              const float2* __restrict__ basis,
+                                                              const float2* __restrict__ Phi, int64_t ldphi,
+                                                              float2* __restrict__ Q, int* __restrict__ err) {
+  extern __shared__ __align__(16) float2 sm[];
+  const int i3 = blockIdx.x, s = blockIdx.y, k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1];
+  float2* ph = sm;                     // [kA1][kPs]
+  float2* b1 = ph + kA1 * kPs;         // [kA1][8 RA]
+  float2* vs = b1 + kA1 * 8 * RA;      // [8 RA][kA2 + 1]
+  float2* b2 = vs + 8 * RA * (kA2 + 1);  // [kA2][16 RB]
+  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
+  const float2* P0 = Phi + ldphi * s + (int64_t)k * nv + (int64_t)G.n1 * G.n2 * i3;
+  const float2* B1 = basis + G.boff[k][0];
+  const float2* B2 = basis + G.boff[k][1];
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // i2 group or y group; x group
+  const int il = threadIdx.x % 32, w4 = threadIdx.x / 32;
+  float2 qa[RA][RB];
+#pragma unroll
+  for (int a = 0; a < RA; ++a)
+#pragma unroll
+    for (int b = 0; b < RB; ++b) qa[a][b] = make_float2(0.f, 0.f);
+  bool bad = false;
+  for (int i20 = 0; i20 < G.n2; i20 += kA2) {
+    float2 va[RA][4];
+#pragma unroll
+    for (int a = 0; a < RA; ++a)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) va[a][u] = make_float2(0.f, 0.f);
+    for (int i10 = 0; i10 < G.n1; i10 += kA1) {
+      float2 t[kA2 / 4];
+#pragma unroll
+      for (int u = 0; u < kA2 / 4; ++u) {
+        const int i2 = i20 + w4 + 4 * u;
+        t[u] = i10 + il < G.n1 && i2 < G.n2 ? __ldcs(P0 + (int64_t)G.n1 * i2 + i10 + il) : make_float2(0.f, 0.f);
+      }
+      __syncthreads();  // the previous chunk has been read
+#pragma unroll
+      for (int u = 0; u < kA2 / 4; ++u) {
+        bad = bad || !finite2(t[u]);
+        ph[il * kPs + w4 + 4 * u] = t[u];
+      }
+      for (int e = threadIdx.x; e < kA1 * 8 * RA; e += 128) {
+        const int i = e % kA1, x = e / kA1;
+        b1[i * 8 * RA + x] = x < R1 && i10 + i < G.n1 ? B1[(int64_t)x * G.n1 + i10 + i] : make_float2(0.f, 0.f);
+      }
+      __syncthreads();
+#pragma unroll 4
+      for (int i = 0; i < kA1; ++i) {
+        const float4 p0 = *(const float4*)&ph[i * kPs + 4 * tx], p1 = *(const float4*)&ph[i * kPs + 4 * tx + 2];
+#pragma unroll
+        for (int a = 0; a < RA; ++a) {
+          const float2 b = b1[i * 8 * RA + ty * RA + a];
+          va[a][0] = cfma_conj(b, make_float2(p0.x, p0.y), va[a][0]);
+          va[a][1] = cfma_conj(b, make_float2(p0.z, p0.w), va[a][1]);
+          va[a][2] = cfma_conj(b, make_float2(p1.x, p1.y), va[a][2]);
+          va[a][3] = cfma_conj(b, make_float2(p1.z, p1.w), va[a][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < RA; ++a)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) vs[(ty * RA + a) * (kA2 + 1) + 4 * tx + u] = va[a][u];
+    for (int e = threadIdx.x; e < kA2 * 16 * RB; e += 128) {
+      const int i = e % kA2, y = e / kA2;
+      b2[i * 16 * RB + y] = y < R2 && i20 + i < G.n2 ? B2[(int64_t)y * G.n2 + i20 + i] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int i = 0; i < kA2; ++i) {
+      float2 c[RB];
+#pragma unroll
+      for (int b = 0; b < RB; ++b) c[b] = b2[i * 16 * RB + tx + 16 * b];
+#pragma unroll
+      for (int a = 0; a < RA; ++a) {
+        const float2 v = vs[(ty * RA + a) * (kA2 + 1) + i];
+#pragma unroll
+        for (int b = 0; b < RB; ++b) qa[a][b] = cfma_conj(c[b], v, qa[a][b]);
+      }
+    }
+    // vs and b2 are written again only after the next tile's first barriers
+  }
+  if (bad) atomicOr(err, kErrNonFinite);
+  float2* Qp = Q + (int64_t)s * G.Qt + G.qoff[k] + (int64_t)i3 * R1 * R2;
+#pragma unroll
+  for (int a = 0; a < RA; ++a)
+#pragma unroll
+    for (int b = 0; b < RB; ++b) {
+      const int x = ty * RA + a, y = tx + 16 * b;
+      if (x < R1 && y < R2) Qp[x + R1 * y] = qa[a][b];
+    }
+}
+
+// F[s][toff + xy + RR z] = sum_i3 conj(B3[i3, z]) Q[s][qoff + i3 RR + xy]; entries up to Cs are zero
+__global__ void __launch_bounds__(128) joint_mode3_adj_kernel(const __grid_constant__ JointGeo G,
+                                                              const float2* __restrict__ basis, const float2* __restrict__ Q,
+                                                              float2* __restrict__ F) {
+  constexpr int NZ = 8, NC = 64;
+  __shared__ float2 b3[NC][NZ];
+  const int k = blockIdx.z % G.q, s = blockIdx.z / G.q, R3 = G.R[k][2];
+  const int RR = G.R[k][0] * G.R[k][1], z0 = blockIdx.y * NZ;
+  if ((int)blockIdx.x * 128 >= RR || z0 >= R3) return;
+  const int xy = blockIdx.x * 128 + threadIdx.x;
+  const float2* Qs = Q + (int64_t)s * G.Qt + G.qoff[k] + (xy < RR ? xy : 0);
+  float2 acc[NZ];
+#pragma unroll
+  for (int z = 0; z < NZ; ++z) acc[z] = make_float2(0.f, 0.f);
+  for (int i0 = 0; i0 < G.n3; i0 += NC) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < NC * NZ; e += 128) {
+      const int i = e % NC, z = e / NC;
+      b3[i][z] = z0 + z < R3 && i0 + i < G.n3 ? basis[G.boff[k][2] + (int64_t)(z0 + z) * G.n3 + i0 + i] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const int ni = min(NC, G.n3 - i0);
+#pragma unroll 8
+    for (int i = 0; i < ni; ++i) {
+      const float2 v = Qs[(int64_t)(i0 + i) * RR];
+#pragma unroll
+      for (int z = 0; z < NZ; ++z) acc[z] = cfma_conj(b3[i][z], v, acc[z]);
+    }
+  }
+  float2* o = F + (int64_t)s * G.Ct + G.toff[k];
+  if (xy < RR)
+#pragma unroll
+    for (int z = 0; z < NZ; ++z)
+      if (z0 + z < R3) o[xy + (int64_t)RR * (z0 + z)] = acc[z];
+  if (blockIdx.x == 0 && blockIdx.y == 0)
+    for (int e = RR * R3 + threadIdx.x; e < G.Cs[k]; e += 128) o[e] = make_float2(0.f, 0.f);
+}
+
+constexpr int kCj = 64;  // columns per CTA of the adjoint core sum
+constexpr int kCc = 32;  // core entries per chunk
+
+// part[split][s][j] = sum over the split's core entries c of conj(K[j][c]) F[s][c].  128 threads:
+// 16 groups of 4 columns, P / TS groups of TS right-hand sides, and KS interleaved slices of the
+// chunk where P is small.  Grid (column tiles, splits of all components' entries, passes of P).
+template <int P>
+__global__ void __launch_bounds__(128) joint_core_adj_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ K,
+                                                             const float2* __restrict__ F, int p, int chunk,
+                                                             float2* __restrict__ part) {
+  constexpr int TS = P >= 16 ? 2 : 1, SG = P / TS, KS = 8 / SG;
+  __shared__ __align__(16) float2 ks[kCc][kCj + 2];
+  __shared__ __align__(16) float2 fs[kCc][P];
+  __shared__ float2 red[KS > 1 ? KS : 1][KS > 1 ? kCj : 1][KS > 1 ? P : 1];
+  int sp = blockIdx.y, k = 0;
+  for (; k < G.q; ++k) {
+    const int ns = (G.Cs[k] + chunk - 1) / chunk;
+    if (sp < ns) break;
+    sp -= ns;
+  }
+  const int c0 = sp * chunk, c1 = min(G.Cs[k], c0 + chunk);
+  const int jb = blockIdx.x * kCj, s0 = blockIdx.z * P;
+  const int jg = threadIdx.x % 16, sg = threadIdx.x / 16 % SG, kq = threadIdx.x / (16 * SG);
+  const int cl = threadIdx.x % 32, w4 = threadIdx.x / 32;
+  const float2* Kp = K + G.koff[k];
+  const float2* Fp = F + G.toff[k];
+  float2 acc[4][TS], sum[4][TS];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < TS; ++b) acc[a][b] = sum[a][b] = make_float2(0.f, 0.f);
+  // the running sums go into the totals every 8 chunks: one FP32 sum over a split's several thousand
+  // entries made the 96^3 adjoint's error 1.5e-6, against 9.7e-7 of the mode-1 form
+  auto fold = [&]() {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < TS; ++b) {
+        sum[a][b].x += acc[a][b].x;
+        sum[a][b].y += acc[a][b].y;
+        acc[a][b] = make_float2(0.f, 0.f);
+      }
+  };
+  float2 kr[kCj / 4];
+  auto fetch = [&](int c) {
+#pragma unroll
+    for (int u = 0; u < kCj / 4; ++u) {
+      const int j = jb + w4 + 4 * u;
+      kr[u] = c + cl < c1 && j < G.M ? __ldcs(Kp + (int64_t)j * G.Cs[k] + c + cl) : make_float2(0.f, 0.f);
+    }
+  };
+  fetch(c0);
+  for (int c = c0; c < c1; c += kCc) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kCj / 4; ++u) ks[cl][w4 + 4 * u] = kr[u];
+    for (int e = threadIdx.x; e < kCc * P; e += 128) {
+      const int i = e % kCc, s = e / kCc;
+      fs[i][s] = c + i < c1 && s0 + s < p ? Fp[(int64_t)(s0 + s) * G.Ct + c + i] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    if (c + kCc < c1) fetch(c + kCc);
+#pragma unroll 4
+    for (int i = kq; i < kCc; i += KS) {
+      const float4 k0 = *(const float4*)&ks[i][4 * jg], k1 = *(const float4*)&ks[i][4 * jg + 2];
+#pragma unroll
+      for (int b = 0; b < TS; ++b) {
+        const float2 f = fs[i][sg * TS + b];
+        acc[0][b] = cfma_conj(make_float2(k0.x, k0.y), f, acc[0][b]);
+        acc[1][b] = cfma_conj(make_float2(k0.z, k0.w), f, acc[1][b]);
+        acc[2][b] = cfma_conj(make_float2(k1.x, k1.y), f, acc[2][b]);
+        acc[3][b] = cfma_conj(make_float2(k1.z, k1.w), f, acc[3][b]);
+      }
+    }
+    if ((c - c0) / kCc % 8 == 7) fold();
+  }
+  fold();
+  if constexpr (KS > 1) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) red[kq][4 * jg + a][sg] = sum[a][0];
+    __syncthreads();
+    if (kq == 0)
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        for (int w = 1; w < KS; ++w) {
+          sum[a][0].x += red[w][4 * jg + a][sg].x;
+          sum[a][0].y += red[w][4 * jg + a][sg].y;
+        }
+  }
+  if (kq == 0)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < TS; ++b) {
+        const int j = jb + 4 * jg + a, s = s0 + sg * TS + b;
+        if (j < G.M && s < p) part[((int64_t)blockIdx.y * p + s) * G.M + j] = sum[a][b];
+      }
+}
+
+// out[j, s] = sum over the splits, in order; one warp per 32 columns, the splits over 8 warps
+__global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict__ part, int M, int p, int splits,
+                                                        float2* __restrict__ out, int64_t ldo) {
+  __shared__ float2 red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 32 + lane, s = blockIdx.y;
+  float2 a = make_float2(0.f, 0.f);
+  if (j < M)
+    for (int i = w; i < splits; i += 8) {
+      const float2 v = part[((int64_t)i * p + s) * M + j];
+      a.x += v.x;
+      a.y += v.y;
+    }
+  red[w][lane] = a;
+  __syncthreads();
+  if (w == 0 && j < M) {
+    for (int i = 1; i < 8; ++i) {
+      a.x += red[i][lane].x;
+      a.y += red[i][lane].y;
+    }
+    out[j + ldo * s] = a;
+  }
+}
+
+constexpr int kPassRhs = 64;  // right-hand sides per round of the workspaces
+
+int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : p <= 4 ? 4 : p <= 8 ? 8 : 16; }
+
+template <int NI>
+int launch_plane_fwd(const JointGeo& G, const float2* basis, const float2* Q, int p, float2* Y, int64_t ldy,
+                     cudaStream_t st) {
+  ZBC_TRY(set_smem_limit<joint_plane_fwd_kernel<NI>>((int)plane_fwd_smem(kJointRmax, kJointRmax, NI)));
+  size_t sm = 0;
+  for (int k = 0; k < G.q; ++k) sm = std::max(sm, plane_fwd_smem(G.R[k][0], G.R[k][1], NI));
+  const int nb = ceil_div(G.n1, 32 * NI);
+  int occ = 0;
+  ZBC_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, joint_plane_fwd_kernel<NI>, 256, sm));
+  const int64_t items = (int64_t)p * G.n3 * ceil_div(G.n2, kI2);
+  const int walkers = (int)std::min<int64_t>(items, std::max(1, std::max(1, occ) * sm_count() / (nb * G.q)));
+  joint_plane_fwd_kernel<NI><<<dim3(walkers, nb, G.q), 256, sm, st>>>(G, basis, Q, p, Y, ldy);
+  count_launch();
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
+}
+
+template <int RA, int RB>
+int launch_plane_adj(const JointGeo& G, const float2* basis, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
+                     cudaStream_t st) {
+  constexpr size_t sm = sizeof(float2) * ((size_t)kA1 * kPs + (size_t)kA1 * 8 * RA + (size_t)8 * RA * (kA2 + 1) +
+                                          (size_t)kA2 * 16 * RB);
+  ZBC_TRY((set_smem_limit<joint_plane_adj_kernel<RA, RB>>((int)sm)));
+  joint_plane_adj_kernel<RA, RB><<<dim3(G.n3, p, G.q), 128, sm, st>>>(G, basis, Phi, ldphi, Q, err);
+  count_launch();
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
+}
+
+template <int RA>
+int plane_adj_rb(int RB, const JointGeo& G, const float2* basis, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
+                 cudaStream_t st) {
+  switch (RB) {
+    case 1: return launch_plane_adj<RA, 1>(G, basis, Phi, ldphi, p, Q, err, st);
+    case 2: return launch_plane_adj<RA, 2>(G, basis, Phi, ldphi, p, Q, err, st);
+    case 3: return launch_plane_adj<RA, 3>(G, basis, Phi, ldphi, p, Q, err, st);
+    default: return launch_plane_adj<RA, 4>(G, basis, Phi, ldphi, p, Q, err, st);
+  }
+}
+
+template <int P>
+void launch_core_fwd(const JointGeo& G, const float2* K, const float2* X, int64_t ldx, int p, int JS, float2* T, int* err,
+                     int csmax, cudaStream_t st) {
+  joint_core_fwd_kernel<P><<<dim3(ceil_div(csmax, 256), JS, G.q * ceil_div(p, P)), 128, 0, st>>>(G, K, X, ldx, p, JS, T, err);
+}
+template <int P>
+void launch_core_adj(const JointGeo& G, const float2* K, const float2* F, int p, int chunk, int splits, float2* part,
+                     cudaStream_t st) {
+  joint_core_adj_kernel<P><<<dim3(ceil_div(G.M, kCj), splits, ceil_div(p, P)), 128, 0, st>>>(G, K, F, p, chunk, part);
+}
+
+// work split of one round of ps <= kPassRhs right-hand sides
+struct FwdPlan {
+  int P, JS;              // right-hand sides per CTA, slices of the column sum
+  int64_t telems, qelems;
+  FwdPlan(const JointGeo& G, int ps) {
+    int cblocks = 0;
+    for (int k = 0; k < G.q; ++k) cblocks += ceil_div(G.Cs[k], 256);
+    P = rhs_per_cta(ps);
+    // enough CTAs for 6 per SM, at least 32 columns a slice
+    JS = std::max(1, std::min({16, G.M / 32, ceil_div(6 * sm_count(), cblocks * ceil_div(ps, P))}));
+    telems = (int64_t)JS * ps * G.Ct;
+    qelems = (int64_t)ps * G.Qt;
+  }
+  size_t bytes() const { return sizeof(float2) * (telems + qelems); }
+};
+struct AdjPlan {
+  int P, chunk, splits;   // core entries per split, number of splits
+  int64_t felems, qelems, pelems;
+  AdjPlan(const JointGeo& G, int ps) {
+    P = rhs_per_cta(ps);
+    // about 6 CTAs per SM, at least 256 entries a split
+    const int want = std::max(1, 6 * sm_count() / (ceil_div(G.M, kCj) * ceil_div(ps, P)));
+    chunk = (int)std::max<int64_t>(256, (G.Ct / want + kCc - 1) / kCc * kCc);
+    splits = 0;
+    for (int k = 0; k < G.q; ++k) splits += ceil_div(G.Cs[k], chunk);
+    felems = (int64_t)ps * G.Ct;
+    qelems = (int64_t)ps * G.Qt;
+    pelems = (int64_t)splits * ps * G.M;
+  }
+  size_t bytes() const { return sizeof(float2) * (felems + qelems + pelems); }
+};
+
+}  // namespace
+
+size_t joint_work_bytes(const Handle& h, int p, bool fwd) {
+  const JointGeo& G = h.joint->geo;
+  size_t b = 0;  // the last round holds the rest of p
+  for (int ps : {std::min(p, kPassRhs), p % kPassRhs})
+    if (ps > 0) b = std::max(b, fwd ? FwdPlan(G, ps).bytes() : AdjPlan(G, ps).bytes());
+  return b;
+}
+
+int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st) {
+  const JointCache& jc = *h.joint;
+  const JointGeo& G = jc.geo;
+  int* err = (int*)h.work_err.ptr;
+  ZBC_TRY(h.work_joint.ensure(joint_work_bytes(h, p, true)));
+  int csmax = 0, rrmax = 0;
+  for (int k = 0; k < G.q; ++k) {
+    csmax = std::max(csmax, G.Cs[k]);
+    rrmax = std::max(rrmax, G.R[k][0] * G.R[k][1]);
+  }
+  for (int s0 = 0; s0 < p; s0 += kPassRhs) {
+    const int ps = std::min(kPassRhs, p - s0);
+    const FwdPlan pl(G, ps);
+    const int JS = pl.JS;
+    float2* T = (float2*)h.work_joint.ptr;
+    float2* Q = T + pl.telems;
+    const float2* Xs = X + ldx * s0;
+    switch (pl.P) {
+      case 1: launch_core_fwd<1>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+      case 2: launch_core_fwd<2>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+      case 4: launch_core_fwd<4>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+      case 8: launch_core_fwd<8>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+      default: launch_core_fwd<16>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+    }
+    joint_mode3_fwd_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(G.n3, kZ), ps * G.q), 128, 0, st>>>(G, jc.basis, T, ps, JS, Q);
+    count_launch(2);
+    // i1 block of 32 NI rows: the fewest padded rows, then the largest block
+    int NI = 1, pad = 1 << 30;
+    for (int ni = 1; ni <= 5; ++ni) {
+      const int rows = ceil_div(G.n1, 32 * ni) * 32 * ni;
+      if (rows <= pad) {
+        pad = rows;
+        NI = ni;
+      }
+    }
+    float2* Ys = Y + ldy * s0;
+    switch (NI) {
+      case 1: ZBC_TRY(launch_plane_fwd<1>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
+      case 2: ZBC_TRY(launch_plane_fwd<2>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
+      case 3: ZBC_TRY(launch_plane_fwd<3>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
+      case 4: ZBC_TRY(launch_plane_fwd<4>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
+      default: ZBC_TRY(launch_plane_fwd<5>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
+    }
+  }
+  return ZBC_OK;
+}
+
+int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* out, int64_t ldo, cudaStream_t st) {
+  const JointCache& jc = *h.joint;
+  const JointGeo& G = jc.geo;
+  int* err = (int*)h.work_err.ptr;
+  ZBC_TRY(h.work_joint.ensure(joint_work_bytes(h, p, false)));
+  int r1 = 0, r2 = 0, r3 = 0, rrmax = 0;
+  for (int k = 0; k < G.q; ++k) {
+    r1 = std::max(r1, G.R[k][0]);
+    r2 = std::max(r2, G.R[k][1]);
+    r3 = std::max(r3, G.R[k][2]);
+    rrmax = std::max(rrmax, G.R[k][0] * G.R[k][1]);
+  }
+  const int RA = ceil_div(r1, 8), RB = ceil_div(r2, 16);
+  for (int s0 = 0; s0 < p; s0 += kPassRhs) {
+    const int ps = std::min(kPassRhs, p - s0);
+    const AdjPlan pl(G, ps);
+    const int chunk = pl.chunk, splits = pl.splits;
+    float2* Q = (float2*)h.work_joint.ptr;
+    float2* F = Q + pl.qelems;
+    float2* part = F + pl.felems;
+    const float2* Ps = Phi + ldphi * s0;
+    switch (RA) {
+      case 1: ZBC_TRY(plane_adj_rb<1>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 2: ZBC_TRY(plane_adj_rb<2>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 3: ZBC_TRY(plane_adj_rb<3>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 4: ZBC_TRY(plane_adj_rb<4>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 5: ZBC_TRY(plane_adj_rb<5>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 6: ZBC_TRY(plane_adj_rb<6>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      case 7: ZBC_TRY(plane_adj_rb<7>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+      default: ZBC_TRY(plane_adj_rb<8>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
+    }
+    joint_mode3_adj_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(r3, 8), ps * G.q), 128, 0, st>>>(G, jc.basis, Q, F);
+    switch (pl.P) {
+      case 1: launch_core_adj<1>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      case 2: launch_core_adj<2>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      case 4: launch_core_adj<4>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      case 8: launch_core_adj<8>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      default: launch_core_adj<16>(G, jc.K, F, ps, chunk, splits, part, st); break;
+    }
+    joint_sum_kernel<<<dim3(ceil_div(G.M, 32), ps), 256, 0, st>>>(part, G.M, ps, splits, out + ldo * s0, ldo);
+    count_launch(3);
+    ZBC_TRY_CUDA(cudaGetLastError());
+  }
+  return ZBC_OK;
+}
+
+}  // namespace zbc

@@ -78,6 +78,9 @@ constexpr uint32_t kWaitPolls = 40000000u;
 struct DecompCache;  // W = G x2 U2 x3 U3 and tile-blocked U1 per tensor, built lazily (decomp_cache.cu)
 void cache_release(DecompCache* c);
 int64_t cache_bytes(const DecompCache* c);  // device bytes held by a cache (0 for null)
+struct JointCache;  // joint basis of the factors and the reduced cores (joint.cuh), built lazily
+void joint_release(JointCache* c);
+int64_t joint_bytes(const JointCache* c);
 
 struct Handle {
   int n1 = 0, n2 = 0, n3 = 0, q = 0;
@@ -98,7 +101,9 @@ struct Handle {
   DevBuf work_xt;        // X^T of the forward products (s-chunk padded rows)
   DevBuf work_err;       // int: error bits kErrTimeout / kErrNonFinite set by the product kernels
   DevBuf work_phi;       // mode-1 adjoint: fp16 operand blocks of Phi and their exponents
+  DevBuf work_joint;     // joint form: reduced sums, planes and partial sums
   DecompCache* cache = nullptr;
+  JointCache* joint = nullptr;
   int cache_r = 0;                 // largest r1 rounded up to 2 (cache row stride bound)
   // autotuned choices per right-hand-side class (zbc_tune; -1 / 0 = untuned)
   static constexpr int kPClasses = 8;
