@@ -428,10 +428,9 @@ static int cross_batch(const std::vector<XSrc>& src, const GreenGeom& Gg, double
       launch_gram_f64((const GramJob*)w.jobs_a.ptr, gg, st);
       ZBC_TRY_CUDA(cudaGetLastError());
       std::vector<JacJob> jj(NT);
-      for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, V1b + mat * t, ng};
+      for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, V1b + mat * t, ng, kJacPass1, 0.0, nullptr};
       ZBC_TRY(upload_jobs(w.jobs_b, jj, st));
-      jacobi_kernel<<<NT, 512, jacobi_smem(ng), st>>>((const JacJob*)w.jobs_b.ptr, 60, nullptr);
-      ZBC_TRY_CUDA(cudaGetLastError());
+      ZBC_TRY(launch_jacobi((const JacJob*)w.jobs_b.ptr, NT, ng, true, st));
       std::vector<RotJob> rj(NT);
       for (int t = 0; t < NT; ++t)
         rj[t] = RotJob{Fb + foff[t], unf[t], fcnt[t], ng, ng, ng, V1b + mat * t, Bb + foff[t], Unf{1, fcnt[t], ng, 0}};
@@ -442,10 +441,9 @@ static int cross_batch(const std::vector<XSrc>& src, const GreenGeom& Gg, double
       ZBC_TRY(upload_jobs(w.jobs_a, gr, st));
       launch_gram_f64((const GramJob*)w.jobs_a.ptr, gg, st);
       ZBC_TRY_CUDA(cudaGetLastError());
-      for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, Wb + mat * t, ng};
+      for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, Wb + mat * t, ng, jac_floor(0.25 * tol, ng), 0.0, nullptr};
       ZBC_TRY(upload_jobs(w.jobs_b, jj, st));
-      jacobi_kernel<<<NT, 512, jacobi_smem(ng), st>>>((const JacJob*)w.jobs_b.ptr, 60, nullptr);
-      ZBC_TRY_CUDA(cudaGetLastError());
+      ZBC_TRY(launch_jacobi((const JacJob*)w.jobs_b.ptr, NT, ng, false, st));
       diag_kernel<<<NT, 256, 0, st>>>((const JacJob*)w.jobs_b.ptr, (double*)w.lam.ptr, nmax);
       ZBC_TRY_CUDA(cudaGetLastError());
       count_launch(6);

@@ -23,27 +23,36 @@
 namespace zbc {
 
 // ---------------------------------------------------------------------------------------------
-// Gram matrices G = A_(g) A_(g)^H, 32x32 output tiles, lower-triangle tiles only + mirror
+// Gram matrices G = A_(g) A_(g)^H, 32x32 output tiles, lower-triangle tiles only + mirror.
+// The FP64 units bound it; a few tensors have too few tiles to keep them busy (24 tensors of 96^3:
+// 144 CTAs, 19 ms at half the FP64 rate), so the columns can be cut into ksplit ranges of whole
+// 16-column chunks (job z / ksplit, range z % ksplit) whose partial matrices go to
+// part[z * pstride + x + n y] and are summed in order by gram_reduce_kernel.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) gram_kernel(const GramJob* jobs) {
-  const GramJob jb = jobs[blockIdx.z];
+__global__ void __launch_bounds__(256) gram_kernel(const GramJob* jobs, int ksplit, double2* part, int64_t pstride) {
+  const GramJob jb = jobs[blockIdx.z / ksplit];
   const int tx = blockIdx.x * 32, ty = blockIdx.y * 32;
   if (tx >= jb.n || ty >= jb.n || ty > tx) return;
   __shared__ double2 sa[16][33];
   __shared__ double2 sb[16][33];
-  const int lx = threadIdx.x % 16, ly = threadIdx.x / 16;  // each thread: rows tx+2lx.., cols ty+2ly..
+  // each thread: rows tx+2lx.., cols ty+2ly..; a warp holds a block of 16 rows x 8 columns, and in a
+  // tile on the diagonal those wholly above it have nothing to do
+  const int wp = threadIdx.x / 32, lx = (wp & 1) * 8 + threadIdx.x % 8, ly = (wp >> 1) * 4 + threadIdx.x % 32 / 8;
+  const bool above = tx == ty && (wp & 1) * 16 + 15 < (wp >> 1) * 8;
   double2 acc[2][2];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0, 0);
-  for (int64_t c0 = 0; c0 < jb.C; c0 += 16) {
+  const int64_t range = ((jb.C + ksplit - 1) / ksplit + 15) / 16 * 16;
+  const int64_t cbeg = (int64_t)(blockIdx.z % ksplit) * range, cend = min(jb.C, cbeg + range);
+  for (int64_t c0 = cbeg; c0 < cend; c0 += 16) {
     for (int e = threadIdx.x; e < 16 * 32; e += 256) {
       const int cc = e / 32, xx = e % 32;
       const int64_t c = c0 + cc;
       double2 va = make_double2(0, 0), vb = make_double2(0, 0);
-      if (c < jb.C) {
+      if (c < cend) {
         if (tx + xx < jb.n) va = ld_z<T>(jb.A, jb.u.at(tx + xx, c));
         if (ty + xx < jb.n) vb = ld_z<T>(jb.A, jb.u.at(ty + xx, c));
       }
@@ -51,6 +60,7 @@ __global__ void __launch_bounds__(256) gram_kernel(const GramJob* jobs) {
       sb[cc][xx] = vb;
     }
     __syncthreads();
+    if (!above)
 #pragma unroll 4
     for (int cc = 0; cc < 16; ++cc) {
       double2 a0 = sa[cc][2 * lx], a1 = sa[cc][2 * lx + 1];
@@ -68,11 +78,51 @@ __global__ void __launch_bounds__(256) gram_kernel(const GramJob* jobs) {
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int x = tx + 2 * lx + a, y = ty + 2 * ly + b;
-      if (x < jb.n && y < jb.n && y <= x) {
+      if (x < jb.n && y < jb.n && y <= x && ksplit > 1) {
+        part[(int64_t)blockIdx.z * pstride + x + (int64_t)jb.n * y] = acc[a][b];
+      } else if (x < jb.n && y < jb.n && y <= x) {
         jb.G[x + (int64_t)jb.n * y] = acc[a][b];
         jb.G[y + (int64_t)jb.n * x] = make_double2(acc[a][b].x, -acc[a][b].y);
       }
     }
+}
+
+// G = the sum of its ksplit partial matrices, in order, mirrored (grid (x, jobs))
+__global__ void __launch_bounds__(256) gram_reduce_kernel(const GramJob* jobs, int ksplit,
+                                                          const double2* __restrict__ part, int64_t pstride) {
+  const GramJob jb = jobs[blockIdx.y];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < jb.n * jb.n; e += gridDim.x * blockDim.x) {
+    const int x = e % jb.n, y = e / jb.n;
+    if (y > x) continue;
+    double2 s = make_double2(0.0, 0.0);
+    for (int z = 0; z < ksplit; ++z) {
+      const double2 v = part[((int64_t)blockIdx.y * ksplit + z) * pstride + e];
+      s.x += v.x;
+      s.y += v.y;
+    }
+    jb.G[y + (int64_t)jb.n * x] = make_double2(s.x, -s.y);
+    jb.G[e] = s;
+  }
+}
+
+// Gram matrices of `count` jobs of at most n rows and C columns, split over column ranges while
+// they fill fewer than 12 CTAs per SM, which also evens out the shorter diagonal tiles (part grows as
+// needed)
+template <typename T>
+static int launch_gram(const GramJob* jobs, int count, int n, int64_t C, DevBuf& part, cudaStream_t st) {
+  const int tn = ceil_div(n, 32);
+  const int64_t ctas = (int64_t)tn * (tn + 1) / 2 * count;
+  const int ksplit = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(16, C / 64), 12 * sm_count() / ctas));
+  const int64_t pstride = (int64_t)n * n;
+  if (ksplit > 1) ZBC_TRY(part.ensure(sizeof(double2) * pstride * ksplit * count));
+  gram_kernel<T><<<dim3(tn, tn, count * ksplit), 256, 0, st>>>(jobs, ksplit, (double2*)part.ptr, pstride);
+  count_launch();
+  if (ksplit > 1) {
+    gram_reduce_kernel<<<dim3(ceil_div(pstride, 256), count), 256, 0, st>>>(jobs, ksplit, (const double2*)part.ptr, pstride);
+    count_launch();
+  }
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -127,108 +177,304 @@ __global__ void __launch_bounds__(256) rotate_kernel(const RotJob* jobs) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Hermitian Jacobi eigensolver, one CTA per matrix (JacJob, hosvd.cuh)
+// Hermitian Jacobi eigensolver, one CTA per matrix (JacJob, hosvd.cuh), round-robin ordering: n/2
+// disjoint pairs a round, a row pass, then a column pass.  FP64 runs at about 2 FMA per cycle and
+// SM on this part, so the rotations themselves bound the kernel, and what helps is to rotate less:
+//  - only pairs above the floors are rotated, from a compacted list.  Without the floors the sweeps
+//    went on rotating rounding noise (96 x 96, 24 matrices at once: 88 ms for each pass; 33 and
+//    9 ms with the first floor alone);
+//  - in pass 1 the numerical range of H is split off first: a pivoted Cholesky factor L (n x r) until
+//    the largest remaining diagonal is below the floor, Householder QR of L, and Jacobi on the
+//    r x r matrix R R^H, V starting from the full unitary Q.  A column's Gram matrix has 12 to 30
+//    directions of 96 above its rounding, and the sweeps' work goes with r (r + n) instead of 2 n^2.
+// H stays in shared memory up to n = 116; both passes walk down columns, of H and of V.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(512) jacobi_kernel(const JacJob* jobs, int max_sweeps, int* sweeps_out) {
-  const JacJob jb = jobs[blockIdx.x];
-  const int n = jb.n;
-  double2* H = jb.H;
-  double2* V = jb.V;
-  extern __shared__ unsigned char smem_raw[];
-  double* cs = (double*)smem_raw;            // n/2
-  double* sn = cs + n / 2;                   // n/2
-  double2* ph = (double2*)(sn + n / 2);      // n/2 : e^{i phi}
-  int* pp = (int*)(ph + n / 2);              // n/2
-  int* pq = pp + n / 2;                      // n/2
-  __shared__ int nrot;
-  for (int64_t e = threadIdx.x; e < (int64_t)n * n; e += blockDim.x) {
-    const int i = (int)(e % n), j = (int)(e / n);
-    V[e] = make_double2(i == j ? 1.0 : 0.0, 0.0);
+constexpr int kJacSmemN = 116;
+constexpr int kJacThreads = 512;
+
+struct JacRot {
+  double c;
+  double2 s;  // s e^{i phi}
+  int p, q;
+};
+
+inline size_t jacobi_smem(int n, bool resident) {
+  return (size_t)(n / 2) * sizeof(JacRot) + (resident ? (size_t)n * n * sizeof(double2) : 0);
+}
+
+__device__ __forceinline__ double warp_sum_d(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Splits off the numerical range of H (n x n at S in shared memory): V = a unitary n x n matrix whose
+// first r columns span it, S[i + m j] = their r x r block of H (m = r rounded up to even, padded
+// with zeros).  Returns m.  Reflector vectors pass through V's memory.
+__device__ int range_start(double2* S, double2* V, int n, double bound, double* red, int* sel) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int r = 0;
+  for (; r < n; ++r) {
+    if (warp == 0) {  // the largest remaining diagonal
+      double best = -1.0;
+      int at = 0;
+      for (int i = lane; i < n; i += 32)
+        if (S[i + n * i].x > best) {
+          best = S[i + n * i].x;
+          at = i;
+        }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double b2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int a2 = __shfl_xor_sync(0xffffffffu, at, o);
+        if (b2 > best || (b2 == best && a2 < at)) {
+          best = b2;
+          at = a2;
+        }
+      }
+      if (lane == 0) {
+        red[0] = best;
+        *sel = at;
+      }
+    }
+    __syncthreads();
+    const double d = red[0];
+    const int p = *sel;
+    if (!(d > bound)) break;
+    const double inv = 1.0 / sqrt(d);
+    for (int i = tid; i < n; i += kJacThreads) {
+      const double2 h = S[i + n * p];
+      V[i + n * r] = make_double2(h.x * inv, h.y * inv);
+    }
+    __syncthreads();
+    for (int e = tid; e < n * n; e += kJacThreads) {
+      const int i = e % n, j = e / n;
+      const double2 a = V[i + n * r], b = V[j + n * r];
+      double2 h = S[e];
+      h.x -= a.x * b.x + a.y * b.y;
+      h.y -= a.y * b.x - a.x * b.y;
+      S[e] = i == p || j == p ? make_double2(0.0, 0.0) : h;
+    }
+    __syncthreads();
   }
   __syncthreads();
-  const double eps = 2.220446049250313e-16;
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) nrot = 0;
+  // L into shared memory (H is used up), Householder QR in place: v_k from the diagonal down, R above
+  // it, and R's diagonal in V's last column, which is free from here until Q is formed
+  double2* L = S;
+  double2* rv = V + (size_t)n * (n - 1);
+  for (int e = tid; e < n * r; e += kJacThreads) L[e] = V[e];
+  __syncthreads();
+  for (int k = 0; k < r; ++k) {
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = k + lane; i < n; i += 32) s += L[i + n * k].x * L[i + n * k].x + L[i + n * k].y * L[i + n * k].y;
+      s = warp_sum_d(s);
+      if (lane == 0) {
+        const double2 x0 = L[k + n * k];
+        const double ax = sqrt(x0.x * x0.x + x0.y * x0.y), nx = sqrt(s);
+        const double2 ph = ax > 0.0 ? make_double2(x0.x / ax, x0.y / ax) : make_double2(1.0, 0.0);
+        const double2 v0 = make_double2(x0.x + ph.x * nx, x0.y + ph.y * nx);
+        L[k + n * k] = v0;
+        const double v2 = s - ax * ax + v0.x * v0.x + v0.y * v0.y;
+        red[0] = nx > 0.0 ? 2.0 / v2 : 0.0;                                // H_k = I - f v v^H
+        rv[k] = make_double2(-ph.x * nx, -ph.y * nx);                      // R_kk
+      }
+    }
     __syncthreads();
-    for (int rnd = 0; rnd < n - 1; ++rnd) {
-      for (int i = threadIdx.x; i < n / 2; i += blockDim.x) {
+    const double f = red[0];
+    for (int j = k + 1 + warp; j < r; j += kJacThreads / 32) {
+      double2 d = make_double2(0.0, 0.0);
+      for (int i = k + lane; i < n; i += 32) d = zfma_conj(L[i + n * k], L[i + n * j], d);
+      d.x = f * warp_sum_d(d.x);
+      d.y = f * warp_sum_d(d.y);
+      for (int i = k + lane; i < n; i += 32) {
+        const double2 v = L[i + n * k];
+        double2& y = L[i + n * j];
+        y.x -= v.x * d.x - v.y * d.y;
+        y.y -= v.x * d.y + v.y * d.x;
+      }
+    }
+    __syncthreads();
+  }
+  // Q = H_0 ... H_{r-1}, a column per warp in registers (n <= 128)
+  double2 rkk[4];
+  for (int u = 0; u < 4; ++u) rkk[u] = lane + 32 * u < r ? rv[lane + 32 * u] : make_double2(0.0, 0.0);
+  __syncthreads();
+  for (int c = warp; c < n; c += kJacThreads / 32) {
+    double2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = make_double2(lane + 32 * u == c ? 1.0 : 0.0, 0.0);
+    for (int k = r - 1; k >= 0; --k) {
+      double2 d = make_double2(0.0, 0.0);
+      double v2 = 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = lane + 32 * u;
+        if (i >= k && i < n) {
+          const double2 v = L[i + n * k];
+          d = zfma_conj(v, x[u], d);
+          v2 += v.x * v.x + v.y * v.y;
+        }
+      }
+      v2 = warp_sum_d(v2);
+      const double f = v2 > 0.0 ? 2.0 / v2 : 0.0;
+      d.x = f * warp_sum_d(d.x);
+      d.y = f * warp_sum_d(d.y);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = lane + 32 * u;
+        if (i >= k && i < n) {
+          const double2 v = L[i + n * k];
+          x[u].x -= v.x * d.x - v.y * d.y;
+          x[u].y -= v.x * d.y + v.y * d.x;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lane + 32 * u < n) V[lane + 32 * u + n * c] = x[u];
+  }
+  __syncthreads();
+  // T = R R^H, T(i, j) = sum_{k >= max(i, j)} R(i, k) conj(R(j, k)), kept in registers until L is done with
+  const int m = r + (r & 1);
+  for (int u = 0; u < 4; ++u)
+    if (warp == 0 && lane + 32 * u < r) L[(lane + 32 * u) * (n + 1)] = rkk[u];  // R's diagonal over v's
+  __syncthreads();
+  constexpr int kPer = (kJacSmemN * kJacSmemN + kJacThreads - 1) / kJacThreads;
+  double2 t[kPer];
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int e = tid + kJacThreads * u, i = e % max(m, 1), j = e / max(m, 1);
+    double2 s = make_double2(0.0, 0.0);
+    if (e < m * m && i < r && j < r)
+      for (int k = max(i, j); k < r; ++k) s = zfma_conj(L[j + n * k], L[i + n * k], s);
+    t[u] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kPer; ++u)
+    if (tid + kJacThreads * u < m * m) S[tid + kJacThreads * u] = t[u];
+  __syncthreads();
+  return m;
+}
+
+template <bool RESIDENT, bool START>
+__global__ void __launch_bounds__(kJacThreads) jacobi_kernel(const JacJob* jobs, int max_sweeps) {
+  const JacJob jb = jobs[blockIdx.x];
+  const int n = jb.n;
+  double2* V = jb.V;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* H = RESIDENT ? (double2*)smem_raw : jb.H;
+  JacRot* rot = (JacRot*)(smem_raw + (RESIDENT ? (size_t)n * n * sizeof(double2) : 0));
+  __shared__ int nact[2], nrot, sel;
+  __shared__ double red[kJacThreads / 32];
+  double tr = 0.0;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int i = e % n, j = e / n;
+    if (!START) V[e] = make_double2(i == j ? 1.0 : 0.0, 0.0);
+    const double2 h = jb.H[e];
+    if (RESIDENT) H[e] = h;
+    if (i == j) tr += h.x;
+  }
+  tr = warp_sum_d(tr);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = tr;
+  if (threadIdx.x == 0) nact[0] = nact[1] = nrot = 0;
+  __syncthreads();
+  tr = 0.0;
+  for (int w = 0; w < kJacThreads / 32; ++w) tr += red[w];
+  __syncthreads();
+  const double fl = jb.floor * fabs(tr), fl2 = fl * fl, tail = jb.tail * fabs(tr);
+  const double eps2 = 2.220446049250313e-16 * 2.220446049250313e-16;
+  int m = n;  // order of the matrix that is rotated
+  if (START) m = range_start(H, V, n, fl, red, &sel);
+  int rnd_all = 0;
+  for (int sweep = 0; sweep < max_sweeps && m > 1; ++sweep) {
+    for (int rnd = 0; rnd < m - 1; ++rnd, ++rnd_all) {
+      int& na = nact[rnd_all & 1];
+      for (int i = threadIdx.x; i < m / 2; i += blockDim.x) {
         int p, q;
         if (i == 0) {
-          p = n - 1;
+          p = m - 1;
           q = rnd;
         } else {
-          p = (rnd + i) % (n - 1);
-          q = (rnd - i + n - 1) % (n - 1);
+          p = rnd + i;
+          if (p >= m - 1) p -= m - 1;
+          q = rnd - i;
+          if (q < 0) q += m - 1;
         }
-        const double a = H[p + (int64_t)n * p].x, b = H[q + (int64_t)n * q].x;
-        const double2 c = H[p + (int64_t)n * q];
-        const double ac = hypot(c.x, c.y);
-        pp[i] = p;
-        pq[i] = q;
-        if (ac == 0.0 || ac <= eps * sqrt(fabs(a) * fabs(b))) {
-          cs[i] = 1.0;
-          sn[i] = 0.0;
-          ph[i] = make_double2(1.0, 0.0);
-        } else {
+        const double a = H[p + m * p].x, b = H[q + m * q].x;
+        const double2 c = H[p + m * q];
+        const double ac2 = c.x * c.x + c.y * c.y;
+        // entries below 1e-154 square to zero and count as zero
+        if (ac2 > fl2 && ac2 > eps2 * fabs(a * b) && !(a <= tail && b <= tail)) {
+          const double ac = sqrt(ac2);
           const double zeta = (b - a) / (2.0 * ac);
           const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          const double cc = 1.0 / sqrt(1.0 + t * t);
-          cs[i] = cc;
-          sn[i] = t * cc;
-          ph[i] = make_double2(c.x / ac, c.y / ac);
-          atomicAdd(&nrot, 1);
+          const double cc = 1.0 / sqrt(1.0 + t * t), sc = t * cc / ac;
+          const int slot = atomicAdd(&na, 1);
+          rot[slot] = JacRot{cc, make_double2(c.x * sc, c.y * sc), p, q};
         }
       }
+      if (threadIdx.x == 0) nact[~rnd_all & 1] = 0;
       __syncthreads();
-      // row pass: rows p,q <- J^H rows
-      for (int64_t e = threadIdx.x; e < (int64_t)(n / 2) * n; e += blockDim.x) {
-        const int i = (int)(e % (n / 2)), x = (int)(e / (n / 2));
-        if (sn[i] == 0.0) continue;
-        const int p = pp[i], q = pq[i];
-        const double c = cs[i], s = sn[i];
-        const double2 f = ph[i];
-        const double2 hp = H[p + (int64_t)n * x], hq = H[q + (int64_t)n * x];
-        const double2 fq = zmul(f, hq);  // e^{i phi} H[q,x]
-        H[p + (int64_t)n * x] = make_double2(c * hp.x - s * fq.x, c * hp.y - s * fq.y);
-        H[q + (int64_t)n * x] = make_double2(s * hp.x + c * fq.x, s * hp.y + c * fq.y);
+      const int A = na;
+      if (A == 0) {
+        __syncthreads();  // all have read the count before the round after next clears it
+        continue;
+      }
+      if (threadIdx.x == 0) nrot += A;
+      // rows p, q of H:  p <- c p - s e^{i phi} q,  q <- c q + s e^{-i phi} p
+      for (int e = threadIdx.x; e < A * m; e += blockDim.x) {
+        const int x = e / A;
+        const JacRot r = rot[e - x * A];
+        double2 &hp = H[r.p + m * x], &hq = H[r.q + m * x];
+        const double2 u = hp, v = hq;
+        hp = make_double2(r.c * u.x - (r.s.x * v.x - r.s.y * v.y), r.c * u.y - (r.s.x * v.y + r.s.y * v.x));
+        hq = make_double2(r.c * v.x + (r.s.x * u.x + r.s.y * u.y), r.c * v.y + (r.s.x * u.y - r.s.y * u.x));
       }
       __syncthreads();
-      // column pass: columns p,q <- columns J ; same on V
-      for (int64_t e = threadIdx.x; e < (int64_t)(n / 2) * n; e += blockDim.x) {
-        const int i = (int)(e % (n / 2)), x = (int)(e / (n / 2));
-        if (sn[i] == 0.0) continue;
-        const int p = pp[i], q = pq[i];
-        const double c = cs[i], s = sn[i];
-        const double2 fc = make_double2(ph[i].x, -ph[i].y);  // e^{-i phi}
-        {
-          const double2 hp = H[x + (int64_t)n * p], hq = H[x + (int64_t)n * q];
-          const double2 gq = zmul(fc, hq);
-          H[x + (int64_t)n * p] = make_double2(c * hp.x - s * gq.x, c * hp.y - s * gq.y);
-          H[x + (int64_t)n * q] = make_double2(s * hp.x + c * gq.x, s * hp.y + c * gq.y);
-        }
-        {
-          const double2 vp = V[x + (int64_t)n * p], vq = V[x + (int64_t)n * q];
-          const double2 gq = zmul(fc, vq);
-          V[x + (int64_t)n * p] = make_double2(c * vp.x - s * gq.x, c * vp.y - s * gq.y);
-          V[x + (int64_t)n * q] = make_double2(s * vp.x + c * gq.x, s * vp.y + c * gq.y);
-        }
+      // columns p, q of H (m rows) and V (n rows):  p <- c p - s e^{-i phi} q,  q <- c q + s e^{i phi} p
+      for (int e = threadIdx.x; e < A * (m + n); e += blockDim.x) {
+        const int ia = e / (m + n), y = e - ia * (m + n);
+        const JacRot r = rot[ia];
+        double2 &hp = y < m ? H[y + m * r.p] : V[y - m + n * r.p], &hq = y < m ? H[y + m * r.q] : V[y - m + n * r.q];
+        const double2 u = hp, v = hq;
+        hp = make_double2(r.c * u.x - (r.s.x * v.x + r.s.y * v.y), r.c * u.y - (r.s.x * v.y - r.s.y * v.x));
+        hq = make_double2(r.c * v.x + (r.s.x * u.x - r.s.y * u.y), r.c * v.y + (r.s.x * u.y + r.s.y * u.x));
       }
       __syncthreads();
-      for (int i = threadIdx.x; i < n / 2; i += blockDim.x) {
-        if (sn[i] == 0.0) continue;
-        const int p = pp[i], q = pq[i];
-        H[p + (int64_t)n * q] = make_double2(0, 0);
-        H[q + (int64_t)n * p] = make_double2(0, 0);
-        H[p + (int64_t)n * p].y = 0.0;
-        H[q + (int64_t)n * q].y = 0.0;
+      for (int i = threadIdx.x; i < A; i += blockDim.x) {
+        const int p = rot[i].p, q = rot[i].q;
+        H[p + m * q] = H[q + m * p] = make_double2(0, 0);
+        H[p + m * p].y = H[q + m * q].y = 0.0;
       }
       __syncthreads();
     }
-    if (nrot == 0) break;
+    __syncthreads();
+    const int any = nrot;
+    __syncthreads();
+    if (any == 0) break;
+    if (threadIdx.x == 0) nrot = 0;
     __syncthreads();
   }
-  if (threadIdx.x == 0 && sweeps_out) sweeps_out[blockIdx.x] = sweep;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const double2 d = i < m ? H[i + m * i] : make_double2(0.0, 0.0);
+    if (RESIDENT) jb.H[i + (int64_t)n * i] = d;
+    if (jb.lam) jb.lam[i] = d.x;
+  }
+}
+
+int launch_jacobi(const JacJob* jobs, int count, int n_max, bool start, cudaStream_t st) {
+  constexpr int kSweeps = 60;
+  if (n_max > kJacSmemN) {
+    jacobi_kernel<false, false><<<count, kJacThreads, jacobi_smem(n_max, false), st>>>(jobs, kSweeps);
+  } else if (start) {
+    ZBC_TRY((set_smem_limit<jacobi_kernel<true, true>>((int)jacobi_smem(kJacSmemN, true))));
+    jacobi_kernel<true, true><<<count, kJacThreads, jacobi_smem(n_max, true), st>>>(jobs, kSweeps);
+  } else {
+    ZBC_TRY((set_smem_limit<jacobi_kernel<true, false>>((int)jacobi_smem(kJacSmemN, true))));
+    jacobi_kernel<true, false><<<count, kJacThreads, jacobi_smem(n_max, true), st>>>(jobs, kSweeps);
+  }
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
 }
 
 // ||A||_F^2 partial sums: 64 blocks per tensor, deterministic host-side final sum
@@ -272,7 +518,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const CopyJob* jobs) {
 
 // launches of the FP64-operand forms for other translation units (hosvd.cuh)
 void launch_gram_f64(const GramJob* jobs, dim3 grid, cudaStream_t st) {
-  gram_kernel<double2><<<grid, 256, 0, st>>>(jobs);
+  gram_kernel<double2><<<grid, 256, 0, st>>>(jobs, 1, nullptr, 0);
 }
 void launch_rotate_f64(const RotJob* jobs, dim3 grid, cudaStream_t st) {
   rotate_kernel<double2><<<grid, 256, 0, st>>>(jobs);
@@ -283,8 +529,9 @@ void launch_rotate_f64(const RotJob* jobs, dim3 grid, cudaStream_t st) {
 // ---------------------------------------------------------------------------------------------
 struct HosvdWork {
   DevBuf jobs_a, jobs_b, jobs_c, jobs_d;
-  DevBuf H, V1, W, Bbuf, U, C1, C2, G, norm_part, ord, sweeps, base_ptrs;
+  DevBuf H, V1, W, Bbuf, U, C1, C2, G, norm_part, ord, lam, base_ptrs;
   DevBuf skpart;  // partial sketches of the split sketch kernel
+  DevBuf part;    // partial matrices of the split Gram kernel
 };
 
 // Compress tensors t = 0..T-1 (tensor t = column t/q, component t%q) of one batch.
@@ -320,7 +567,7 @@ static int hosvd_batch(const void* cols, int64_t ld, int ncols, int n1, int n2, 
   ZBC_TRY(w.W.ensure(sizeof(double2) * mat * NT));
   ZBC_TRY(w.Bbuf.ensure(sizeof(double2) * (size_t)nv * NT));
   ZBC_TRY(w.U.ensure(sizeof(double2) * (size_t)(n1 + n2 + n3) * nmax * NT));
-  ZBC_TRY(w.sweeps.ensure(sizeof(int) * NT));
+  ZBC_TRY(w.lam.ensure(sizeof(double) * nmax_e * NT));
   double2* Hb = (double2*)w.H.ptr;
   double2* V1b = (double2*)w.V1.ptr;
   double2* Wb = (double2*)w.W.ptr;
@@ -345,19 +592,15 @@ static int hosvd_batch(const void* cols, int64_t ld, int ncols, int n1, int n2, 
     // the Gram kernel writes an ng x ng block with leading dimension ng; pad handled by ld=ne below
     for (int t = 0; t < NT; ++t) gj[t].n = ng;
     ZBC_TRY(upload_jobs(w.jobs_a, gj, st));
-    dim3 gg(ceil_div(ng, 32), ceil_div(ng, 32), NT);
-    gram_kernel<T><<<gg, 256, 0, st>>>((const GramJob*)w.jobs_a.ptr);
-    ZBC_TRY_CUDA(cudaGetLastError());
+    ZBC_TRY(launch_gram<T>((const GramJob*)w.jobs_a.ptr, NT, ng, C[g], w.part, st));
     if (ne != ng) {
       set_error("odd mode sizes are not supported by the GPU HOSVD (n=%d)", ng);
       return ZBC_EINVAL;
     }
     std::vector<JacJob> jj(NT);
-    for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, V1b + mat * t, ne};
+    for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, V1b + mat * t, ne, kJacPass1, 0.0, nullptr};
     ZBC_TRY(upload_jobs(w.jobs_b, jj, st));
-    const size_t jsm = (size_t)(ne / 2) * (2 * sizeof(double) + sizeof(double2) + 2 * sizeof(int));
-    jacobi_kernel<<<NT, 512, jsm, st>>>((const JacJob*)w.jobs_b.ptr, 60, (int*)w.sweeps.ptr);
-    ZBC_TRY_CUDA(cudaGetLastError());
+    ZBC_TRY(launch_jacobi((const JacJob*)w.jobs_b.ptr, NT, ne, true, st));
     // pass 2: B = V1^H A_(g)  (n x C, column-major), H2 = B B^H
     std::vector<RotJob> rj(NT);
     for (int t = 0; t < NT; ++t)
@@ -367,21 +610,20 @@ static int hosvd_batch(const void* cols, int64_t ld, int ncols, int n1, int n2, 
     ZBC_TRY_CUDA(cudaGetLastError());
     for (int t = 0; t < NT; ++t) gj[t] = GramJob{Bb + (size_t)nv * t, Unf{1, C[g], ng, 0}, C[g], ng, Hb + mat * t};
     ZBC_TRY(upload_jobs(w.jobs_a, gj, st));
-    gram_kernel<double2><<<gg, 256, 0, st>>>((const GramJob*)w.jobs_a.ptr);
-    ZBC_TRY_CUDA(cudaGetLastError());
-    for (int t = 0; t < NT; ++t) jj[t] = JacJob{Hb + mat * t, Wb + mat * t, ne};
+    ZBC_TRY(launch_gram<double2>((const GramJob*)w.jobs_a.ptr, NT, ng, C[g], w.part, st));
+    for (int t = 0; t < NT; ++t)
+      jj[t] = JacJob{Hb + mat * t, Wb + mat * t, ne, jac_floor(tol, ne), jac_tail(tol, ne), (double*)w.lam.ptr + (size_t)ne * t};
     ZBC_TRY(upload_jobs(w.jobs_b, jj, st));
-    jacobi_kernel<<<NT, 512, jsm, st>>>((const JacJob*)w.jobs_b.ptr, 60, (int*)w.sweeps.ptr);
-    ZBC_TRY_CUDA(cudaGetLastError());
+    ZBC_TRY(launch_jacobi((const JacJob*)w.jobs_b.ptr, NT, ne, false, st));
     // eigenvalues -> host, rank rule, order
-    std::vector<double2> Hh(mat * NT);
-    ZBC_TRY_CUDA(cudaMemcpyAsync(Hh.data(), Hb, sizeof(double2) * mat * NT, cudaMemcpyDeviceToHost, st));
+    std::vector<double> lamh((size_t)ne * NT);
+    ZBC_TRY_CUDA(cudaMemcpyAsync(lamh.data(), w.lam.ptr, sizeof(double) * lamh.size(), cudaMemcpyDeviceToHost, st));
     ZBC_TRY_CUDA(cudaStreamSynchronize(st));
     std::vector<int> ord_all((size_t)NT * ng);
     std::vector<FacJob> fj(NT);
     for (int t = 0; t < NT; ++t) {
       std::vector<double> lam(ng);
-      for (int i = 0; i < ng; ++i) lam[i] = Hh[mat * t + i + (size_t)ng * i].x;
+      for (int i = 0; i < ng; ++i) lam[i] = lamh[(size_t)ne * t + i];
       std::vector<int> ord(ng);
       std::iota(ord.begin(), ord.end(), 0);
       std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return lam[a] > lam[b]; });
@@ -875,11 +1117,11 @@ static int randomized_batch(const void* cols, int64_t ld, int ncols, int n1, int
   std::vector<NormJob> nj(NT);
   for (int t = 0; t < NT; ++t) nj[t] = NormJob{Cc + csz * t, (int64_t)wd[3 * t] * wd[3 * t + 1] * wd[3 * t + 2]};
   ZBC_TRY(upload_jobs(w.jobs_d, nj, st));
-  ZBC_TRY(w.sweeps.ensure(sizeof(double) * 16 * NT));
-  norm_jobs_kernel<<<dim3(16, NT), 256, 0, st>>>((const NormJob*)w.jobs_d.ptr, (double*)w.sweeps.ptr);
+  ZBC_TRY(w.lam.ensure(sizeof(double) * 16 * NT));
+  norm_jobs_kernel<<<dim3(16, NT), 256, 0, st>>>((const NormJob*)w.jobs_d.ptr, (double*)w.lam.ptr);
   count_launch();
   std::vector<double> cpart(16 * (size_t)NT);
-  ZBC_TRY_CUDA(cudaMemcpyAsync(cpart.data(), w.sweeps.ptr, sizeof(double) * cpart.size(), cudaMemcpyDeviceToHost, st));
+  ZBC_TRY_CUDA(cudaMemcpyAsync(cpart.data(), w.lam.ptr, sizeof(double) * cpart.size(), cudaMemcpyDeviceToHost, st));
   ZBC_TRY_CUDA(cudaStreamSynchronize(st));
   std::vector<double> budget(NT, -1.0);
   std::vector<int> pass;
@@ -902,6 +1144,7 @@ static int randomized_batch(const void* cols, int64_t ld, int ncols, int n1, int
   const int P = (int)pass.size();
   const int wme = kWmax;  // padded Gram size bound
   ZBC_TRY(w.H.ensure(sizeof(double2) * (size_t)wme * wme * P));
+  ZBC_TRY(w.lam.ensure(sizeof(double) * wme * P));
   ZBC_TRY(w.W.ensure(sizeof(double2) * (size_t)wme * wme * P * 3));
   double2* Hb = (double2*)w.H.ptr;
   double2* Wb = (double2*)w.W.ptr;
@@ -923,23 +1166,31 @@ static int randomized_batch(const void* cols, int64_t ld, int ncols, int n1, int
       const Unf cu[3] = {{1, (int64_t)b * c, a, 0}, {a, a, 1, (int64_t)a * b}, {(int64_t)a * b, (int64_t)a * b, 1, 0}};
       const int64_t Cg = (int64_t)a * b * c / wg;
       gj[pi] = GramJob{Cc + csz * t, cu[g], Cg, wg, Hb + (size_t)wme * wme * pi};
-      jj[pi] = JacJob{Hb + (size_t)wme * wme * pi, Wb + (size_t)wme * wme * (3 * pi + g), we[pi]};
+      // what is left alone may move a tail sum by 1e-8 of what the projection left of the budget
+      const double left = std::sqrt(std::max(0.0, budget[t] / norm2[t]));
+      jj[pi] = JacJob{Hb + (size_t)wme * wme * pi, Wb + (size_t)wme * wme * (3 * pi + g), we[pi],
+                      jac_floor(left, we[pi]), jac_tail(left, we[pi]), (double*)w.lam.ptr + (size_t)wme * pi};
     }
     ZBC_TRY(upload_jobs(w.jobs_a, gj, st));
-    gram_kernel<double2><<<dim3(2, 2, P), 256, 0, st>>>((const GramJob*)w.jobs_a.ptr);
+    int wmax = 0;
+    int64_t cmax = 0;
+    for (const GramJob& j : gj) {
+      wmax = std::max(wmax, j.n);
+      cmax = std::max(cmax, j.C);
+    }
+    ZBC_TRY(launch_gram<double2>((const GramJob*)w.jobs_a.ptr, P, wmax, cmax, w.part, st));
     ZBC_TRY(upload_jobs(w.jobs_b, jj, st));
-    const size_t jsm = (size_t)(wme / 2) * (2 * sizeof(double) + sizeof(double2) + 2 * sizeof(int));
-    jacobi_kernel<<<P, 512, jsm, st>>>((const JacJob*)w.jobs_b.ptr, 60, nullptr);
-    count_launch(2);
-    std::vector<double2> Hh((size_t)wme * wme * P);
-    ZBC_TRY_CUDA(cudaMemcpyAsync(Hh.data(), Hb, sizeof(double2) * Hh.size(), cudaMemcpyDeviceToHost, st));
+    ZBC_TRY(launch_jacobi((const JacJob*)w.jobs_b.ptr, P, *std::max_element(we.begin(), we.end()), false, st));
+    count_launch();
+    std::vector<double> lamh((size_t)wme * P);
+    ZBC_TRY_CUDA(cudaMemcpyAsync(lamh.data(), w.lam.ptr, sizeof(double) * lamh.size(), cudaMemcpyDeviceToHost, st));
     ZBC_TRY_CUDA(cudaStreamSynchronize(st));
     for (int pi = 0; pi < P; ++pi) {
       const int t = pass[pi];
       const int dims[3] = {wd[3 * t], wd[3 * t + 1], wd[3 * t + 2]};
       const int wg = dims[g], e = we[pi];
       std::vector<double> lam(e);
-      for (int i = 0; i < e; ++i) lam[i] = Hh[(size_t)wme * wme * pi + i + (size_t)e * i].x;
+      for (int i = 0; i < e; ++i) lam[i] = lamh[(size_t)wme * pi + i];
       std::vector<int> ord(e);
       std::iota(ord.begin(), ord.end(), 0);
       std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return lam[x] > lam[y]; });

@@ -35,13 +35,26 @@ struct RotJob {    // out(x, c) = sum_i conj(V[i + ldv*x]) A(i, c),  x < r, i < 
   Unf o;           // output placement of (x, c)
 };
 
-// Hermitian Jacobi eigensolver, one CTA per matrix (n even, in global memory).  On return H is
-// diagonal (eigenvalues on the diagonal) and V holds the eigenvectors (columns).
+// Hermitian Jacobi eigensolver, one CTA per matrix (n even).  On return the diagonal of H holds the
+// eigenvalues (also at lam, n doubles, unless null) and V the eigenvectors (columns); the rest of H
+// is undefined.  All bounds are relative to trace(H).  Off-diagonal entries of at most `floor` are
+// left as they are, and so are pairs whose diagonals are both at most `tail`: a caller that only
+// sums those eigenvalues does not see how they split among each other.
 struct JacJob {
   double2* H;
   double2* V;
   int n;
+  double floor, tail;
+  double* lam;
 };
+// Pass 1 of a two-pass scheme only has to give a unitary start for the second Gram matrix: below the
+// rounding of H itself there is nothing to resolve.
+constexpr double kJacPass1 = 1e-16;
+// Pass 2 with relative tolerance tol on ||A||_F: the neglected entries of a row together move a
+// tail sum by less than 1e-8 of the budget tol^2 / 3; eigenvalues that together stay below 1e-3 of
+// the budget are in every tail.
+inline double jac_floor(double tol, int n) { return std::min(1e-20, 1e-8 * tol * tol / 3.0 / n); }
+inline double jac_tail(double tol, int n) { return 1e-3 * tol * tol / 3.0 / n; }
 
 // U[:, a] = V1 * W[:, ord[a]]  (n x r), FP64
 struct FacJob {
@@ -73,14 +86,13 @@ __device__ __forceinline__ double2 ld_z(const void* p, int64_t i) {
 void launch_gram_f64(const GramJob* jobs, dim3 grid, cudaStream_t st);
 // out(x, c) = sum_i conj(V[i + ldv x]) A(i, c) for FP64 operands; grid (ceil(C/64), ceil(r/32), jobs)
 void launch_rotate_f64(const RotJob* jobs, dim3 grid, cudaStream_t st);
-// grid (jobs), 512 threads, dynamic smem jacobi_smem(n)
-__global__ void jacobi_kernel(const JacJob* jobs, int max_sweeps, int* sweeps_out);
+// eigensolves of `count` matrices, the largest n_max x n_max; start: pass 1 (the numerical range of
+// H is split off first, floor bounds what it leaves out)
+int launch_jacobi(const JacJob* jobs, int count, int n_max, bool start, cudaStream_t st);
 // grid (x, jobs), 256 threads
 __global__ void factor_kernel(const FacJob* jobs);
 // grid (x, jobs), 256 threads
 __global__ void pack_kernel(const CopyJob* jobs);
-
-inline size_t jacobi_smem(int n) { return (size_t)(n / 2) * (2 * sizeof(double) + sizeof(double2) + 2 * sizeof(int)); }
 
 template <typename J>
 static int upload_jobs(DevBuf& buf, const std::vector<J>& jobs, cudaStream_t st) {
