@@ -813,7 +813,9 @@ struct SketchJob {
 // ksplit ranges of whole 16-column chunks (so one tensor's sketch spreads over many SMs) and each
 // range's partial Y goes to part[(job * ksplit + z) * pstride + x + n l], summed in a fixed order
 // by sketch_reduce_kernel.
-template <typename T>
+// NW: groups of 8 sketch columns (the FP64 units bound the kernel, so columns that were not asked
+// for cost as much as those that were: 64 columns for a width of 32 took 134 ms, 16 x 128^3 columns).
+template <typename T, int NW>
 __global__ void __launch_bounds__(256) sketch_kernel(const SketchJob* jobs, int ksplit, double2* part,
                                                      int64_t pstride) {
   const SketchJob jb = jobs[blockIdx.y];
@@ -822,11 +824,11 @@ __global__ void __launch_bounds__(256) sketch_kernel(const SketchJob* jobs, int 
   const int64_t chunk = ((jb.C + ksplit - 1) / ksplit + 15) / 16 * 16;
   const int64_t cbeg = (int64_t)blockIdx.z * chunk, cend = min(jb.C, cbeg + chunk);
   __shared__ double2 sa[16][33];
-  __shared__ double2 so[16][kWmax + 1];
+  __shared__ double2 so[16][8 * NW + 1];
   const int lx = threadIdx.x % 32, lg = threadIdx.x / 32;
-  double2 acc[kWmax / 8];
+  double2 acc[NW];
 #pragma unroll
-  for (int i = 0; i < kWmax / 8; ++i) acc[i] = make_double2(0.0, 0.0);
+  for (int i = 0; i < NW; ++i) acc[i] = make_double2(0.0, 0.0);
   for (int64_t c0 = cbeg; c0 < cend; c0 += 16) {
     for (int e = threadIdx.x; e < 16 * 32; e += 256) {
       const int cc = e / 32, xx = e % 32;
@@ -835,8 +837,8 @@ __global__ void __launch_bounds__(256) sketch_kernel(const SketchJob* jobs, int 
       if (c < cend && x0 + xx < jb.n) v = ld_z<T>(jb.A, jb.u.at(x0 + xx, c));
       sa[cc][xx] = v;
     }
-    for (int e = threadIdx.x; e < 16 * kWmax; e += 256) {
-      const int cc = e / kWmax, l = e % kWmax;
+    for (int e = threadIdx.x; e < 16 * 8 * NW; e += 256) {
+      const int cc = e / (8 * NW), l = e % (8 * NW);
       const int64_t c = c0 + cc;
       double2 v = make_double2(0.0, 0.0);
       if (c < cend && l < jb.w) {
@@ -850,13 +852,13 @@ __global__ void __launch_bounds__(256) sketch_kernel(const SketchJob* jobs, int 
     for (int cc = 0; cc < 16; ++cc) {
       const double2 a = sa[cc][lx];
 #pragma unroll
-      for (int i = 0; i < kWmax / 8; ++i) acc[i] = zfma(a, so[cc][lg + 8 * i], acc[i]);
+      for (int i = 0; i < NW; ++i) acc[i] = zfma(a, so[cc][lg + 8 * i], acc[i]);
     }
     __syncthreads();
   }
   double2* out = ksplit > 1 ? part + ((int64_t)blockIdx.y * ksplit + blockIdx.z) * pstride : jb.Y;
 #pragma unroll
-  for (int i = 0; i < kWmax / 8; ++i) {
+  for (int i = 0; i < NW; ++i) {
     const int l = lg + 8 * i;
     if (x0 + lx < jb.n && l < jb.w) out[(x0 + lx) + (int64_t)jb.n * l] = acc[i];
   }
@@ -1070,7 +1072,15 @@ static int randomized_batch(const void* cols, int64_t ld, int ncols, int n1, int
   const int ksplit = (int)std::max<int64_t>(1, std::min<int64_t>(32, (4 * sm_count() + tiles - 1) / tiles));
   const int64_t pstride = (int64_t)nmax * kWmax;
   if (ksplit > 1) ZBC_TRY(w.skpart.ensure(sizeof(double2) * pstride * ksplit * sj.size()));
-  sketch_kernel<T><<<dim3(ceil_div(nmax, 32), (unsigned)sj.size(), ksplit), 256, 0, st>>>(
+  const int nw = ceil_div(*std::max_element(wd.begin(), wd.end()), 8);
+  auto* sketch_fn = nw <= 1   ? sketch_kernel<T, 1>
+                    : nw == 2 ? sketch_kernel<T, 2>
+                    : nw == 3 ? sketch_kernel<T, 3>
+                    : nw == 4 ? sketch_kernel<T, 4>
+                    : nw == 5 ? sketch_kernel<T, 5>
+                    : nw == 6 ? sketch_kernel<T, 6>
+                              : sketch_kernel<T, 8>;
+  sketch_fn<<<dim3(ceil_div(nmax, 32), (unsigned)sj.size(), ksplit), 256, 0, st>>>(
       (const SketchJob*)w.jobs_a.ptr, ksplit, (double2*)w.skpart.ptr, pstride);
   count_launch();
   if (ksplit > 1) {
