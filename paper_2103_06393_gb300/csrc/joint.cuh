@@ -39,8 +39,15 @@ struct JointCache {
   JointGeo geo;
   float2* basis = nullptr;
   float2* K = nullptr;
+  unsigned char* bop = nullptr;  // B1 split for the adjoint's plane product (joint_planes.cu)
   int64_t bytes = 0;
 };
+
+// the plane products on the tensor cores (joint_planes.cu): Y from Q, and Q from Phi
+size_t joint_planes_bytes(const JointGeo& G);
+int joint_planes_build(const JointGeo& G, const float2* basis, unsigned char* bop, cudaStream_t st);
+int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st);
+int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err, cudaStream_t st);
 
 // Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
 int build_joint(Handle& h, cudaStream_t st);

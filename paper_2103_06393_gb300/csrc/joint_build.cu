@@ -19,6 +19,7 @@ void joint_release(JointCache* c) {
   if (!c) return;
   if (c->basis) cudaFree(c->basis);
   if (c->K) cudaFree(c->K);
+  if (c->bop) cudaFree(c->bop);
   delete c;
 }
 int64_t joint_bytes(const JointCache* c) { return c ? c->bytes : 0; }
@@ -404,11 +405,12 @@ int build_joint(Handle& h, cudaStream_t st) {
   if (work > 0.5 * direct || 8.0 * kelems > (jc->large ? 2.0 : 0.5) * wbytes) return ZBC_OK;
   cudaError_t e = cudaMalloc(&jc->basis, sizeof(float2) * belems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->K, sizeof(float2) * kelems);
+  if (e == cudaSuccess) e = cudaMalloc(&jc->bop, joint_planes_bytes(g));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return ZBC_OK;  // no room: unusable
   }
-  jc->bytes = (int64_t)sizeof(float2) * (belems + kelems);
+  jc->bytes = (int64_t)(sizeof(float2) * (belems + kelems) + joint_planes_bytes(g));
   for (int k = 0; k < q; ++k)
     for (int m = 0; m < 3; ++m) {
       const int64_t len = (int64_t)n[m] * g.R[k][m];
@@ -416,6 +418,7 @@ int build_joint(Handle& h, cudaStream_t st) {
                                                                              jc->basis + g.boff[k][m], len);
       count_launch();
     }
+  ZBC_TRY(joint_planes_build(g, jc->basis, jc->bop, st));
   coef_kernel<<<nf, 256, 0, st>>>(dj, dp, dr);
   count_launch();
   // reduced cores in batches that keep the FP64 intermediates near 1 GB

@@ -1,0 +1,653 @@
+// The plane products of the joint form (joint.cuh) on the tensor cores: per right-hand side s,
+// component k and plane i3,
+//   forward  Y[:, :, i3] = B1 S,  S = Q[i3] B2^T          (one write of Y)
+//   adjoint  Q[i3] = V conj(B2),  V = B1^H Phi[:, :, i3]  (one read of Phi)
+// The contraction with B1 touches every voxel R1 times and is a tcgen05 GEMM (kind::f16); the one
+// with B2 works on R1 rows and stays in FP32 on the CUDA cores.  Both operands are split into fp16
+// hi + lo (x = hi + lo to 2^-22) after scaling by powers of two and the three products hi hi,
+// hi lo, lo hi are summed in FP32.  In FP32 on the CUDA cores the same planes took 3.1 / 4.7 ms
+// (320 x 320 x 256, 8 right-hand sides, R = 23-25: 57 % of the FP32 rate) against 0.74 ms that
+// writing or reading the 5 GB takes.
+//
+// Operand conventions: a complex row entry is the pair of K elements (Re, Im), so with
+//   A[i1] = (Re, Im) B1[i1, :]  and  B rows (Re S, -Im S), (Im S, Re S)
+// D's column pair is (Re, Im) Y; the adjoint contracts Phi's own (Re, Im) pairs along i1 with rows
+// (Re b, Im b), (-Im b, Re b) of the basis vector b, which gives (Re, Im) of conj(b) Phi.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "joint.cuh"
+#include "stage.cuh"
+
+namespace zbc {
+namespace {
+
+constexpr int kBasisShift = 10;  // basis entries (|b| <= 1) are scaled by 2^10
+constexpr int kDataShift = 10;   // the other operand is brought below 2^10
+
+// fp16 hi / lo of a scaled pair, as words (x low)
+__device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(x, y);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// e with m < 2^e, at least -100 so that 2^(kDataShift - e) and its inverse are normal floats (0 for
+// zero and for values that are not finite, which go through unscaled)
+__device__ __forceinline__ int exp_of(float m) {
+  if (!(m > 0.f) || !(m < INFINITY)) return 0;
+  return max(-100, (int)(__float_as_uint(m) >> 23) - 126);
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+// max(|a|, |b|, |c|), NaN if any is
+__device__ __forceinline__ float absmax_nan(float a, float b, float c) {
+  float r;
+  asm("{\n\t.reg .f32 t, u, v;\n\tabs.f32 t, %2;\n\tabs.f32 u, %3;\n\tmax.NaN.f32 v, t, u;\n\tmax.NaN.f32 %0, %1, v;\n\t}"
+      : "=f"(r)
+      : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
+               "tcgen05.wait::ld.sync.aligned;"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// the adjoint's eight worker warps and a ninth that issues the MMAs: an issue occupies its thread for
+// about 100 cycles, and a worker that did it held the others up at the next barrier (2.34 -> 1.80 ms,
+// 320 x 320 x 256, 8 right-hand sides)
+constexpr int kThreads = 288;
+__device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// a warp's shared-memory writes, visible to the MMAs of whoever waits on `bar`
+__device__ __forceinline__ void warp_publish(uint64_t* bar) {
+  tc::fence_proxy_async();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive1(bar);
+}
+
+__host__ __device__ inline uint32_t tmem_cols(uint32_t need) {
+  uint32_t c = 32;
+  while (c < need) c *= 2;
+  return c;
+}
+
+// ---------------------------------------------------------------------------------------------
+// forward
+// ---------------------------------------------------------------------------------------------
+// A CTA keeps the hi / lo rows of B1 for up to `nb` blocks of 128 i1 and B2's rows of one tile of NT
+// i2 in shared memory and walks the planes (s, i3) of its component.  Per plane: Q[i3] to shared
+// memory (loaded into registers during the plane before), S (R1 x NT) in FP32, its hi / lo rows to
+// shared memory, one MMA chain per i1 block (M = 128, N = 2 NT, K = 2 R1p) into alternating
+// accumulators, the epilogues (tensor memory to Y, 32 consecutive i1 per store) overlapping the next
+// block's MMAs.  Two CTAs share an SM, so one's stores overlap the other's S.  NT = 64 up to
+// R = 32, else 32 (shared memory).  K-major core-matrix layout without swizzle, KB = R1p / 4 chunks of
+// 16 bytes a row; rows of B1 past n1 are not stored: the MMAs read what follows, into rows of the
+// accumulator that nothing reads.  S is scaled by the bound
+// |S| <= sqrt(2 R2) max |Re Q|, |Im Q| < 12 max.
+constexpr int kQRegs = kJointRmax * kJointRmax / 256;
+
+template <int NT>
+__global__ void __launch_bounds__(256, 2)
+    joint_planes_fwd_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ basis,
+                            const float2* __restrict__ Q, int R1p, int R2p, int nb, int p, float2* __restrict__ Y,
+                            int64_t ldy, int* __restrict__ err) {
+  extern __shared__ __align__(128) unsigned char smem_f[];
+  unsigned char* smem = smem_f;
+  __shared__ __align__(8) uint64_t done[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ float wmax[8];
+  __shared__ int abort_flag;
+  constexpr int GR = 256 / NT;  // groups of 4-row chunks of S
+  constexpr int QR = NT == 64 ? kQRegs / 4 : kQRegs;  // entries of Q per thread
+  const int k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1], RR = R1 * R2, KB = R1p / 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt2 = (G.n2 + NT - 1) / NT, i20 = (int)(blockIdx.y % nt2) * NT;
+  const int row0 = (int)(blockIdx.y / nt2) * nb * 128, rows = min(nb * 128, G.n1 - row0), nblk = (rows + 127) / 128;
+  const uint32_t bbytes = 2u * NT * KB * 16u;  // one term of S
+  unsigned char* sb = smem;                    // S before B1: the MMAs may read past B1's last rows
+  float2* qs = (float2*)(sb + 2 * bbytes);     // [R2][R1p]
+  float2* b2 = qs + R2p * R1p;                 // [R2][NT]
+  unsigned char* sa = (unsigned char*)(b2 + R2p * NT);
+  const uint32_t ablk = 128u * KB * 16u;       // one term of a full block; the last block is shorter
+  const uint32_t alast = (uint32_t)((rows - (nblk - 1) * 128 + 7) / 8) * 8u * KB * 16u;
+  const uint32_t ncols = tmem_cols(nblk > 1 ? 4 * NT : 2 * NT);
+  if (tid == 0) {
+    tc::mbar_init(&done[0], 1);
+    tc::mbar_init(&done[1], 1);
+    abort_flag = 0;
+  }
+  if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
+  const int rows8 = (rows + 7) / 8 * 8;
+  for (int e = tid; e < rows8 * KB; e += 256) {
+    const int rr = e % rows8, kc = e / rows8, b = rr / 128, r = rr % 128, i1 = row0 + rr;
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int x = 4 * kc + u;
+      const float2 v = x < R1 && i1 < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i1] : make_float2(0.f, 0.f);
+      split2(v.x * pow2f(kBasisShift), v.y * pow2f(kBasisShift), h[u], l[u]);
+    }
+    unsigned char* d = sa + (size_t)b * 2 * ablk + tc::core_off(r, kc, KB);
+    *(uint4*)d = make_uint4(h[0], h[1], h[2], h[3]);
+    *(uint4*)(d + (b == nblk - 1 ? alast : ablk)) = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+  for (int e = tid; e < R2 * R1p; e += 256) qs[e] = make_float2(0.f, 0.f);  // the pad stays zero
+  for (int e = tid; e < R2 * NT; e += 256) {
+    const int i2 = i20 + e % NT;
+    b2[e] = i2 < G.n2 ? basis[G.boff[k][1] + (int64_t)(e / NT) * G.n2 + i2] : make_float2(0.f, 0.f);
+  }
+  const int planes = p * G.n3;
+  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
+  const float2* Qk = Q + G.qoff[k];
+  float2 qr[QR];
+  auto fetch_q = [&](int pl) {
+    const float2* Qp = Qk + (int64_t)(pl / G.n3) * G.Qt + (int64_t)(pl % G.n3) * RR;
+#pragma unroll
+    for (int u = 0; u < QR; ++u)
+      if (tid + 256 * u < RR) qr[u] = __ldg(Qp + tid + 256 * u);
+  };
+  int qdst[QR];
+#pragma unroll
+  for (int u = 0; u < QR; ++u) qdst[u] = (tid + 256 * u) / R1 * R1p + (tid + 256 * u) % R1;
+  fetch_q(blockIdx.x);  // grid x <= planes
+  __syncthreads();
+  const uint32_t tmem = tmem_base;
+  const int il = tid % NT, grp = tid / NT, q4 = warp & 3, half = warp >> 2;
+  const bool full2 = i20 + NT <= G.n2, has0 = grp < KB, has1 = grp + GR < KB;
+  uint32_t ph[2] = {0, 0};  // parity of the next completion of each accumulator
+  bool ok = true;
+  for (int pl = blockIdx.x; pl < planes; pl += gridDim.x) {
+    float m = 0.f;
+#pragma unroll
+    for (int u = 0; u < QR; ++u)
+      if (tid + 256 * u < RR) {
+        qs[qdst[u]] = qr[u];
+        m = absmax_nan(m, qr[u].x, qr[u].y);
+      }
+    for (int o = 16; o > 0; o >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) wmax[warp] = m;
+    __syncthreads();
+    if (abort_flag) break;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = max_nan(m, wmax[w]);
+    if (pl + gridDim.x < planes) fetch_q(pl + gridDim.x);
+    float2 a[2][4];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a[c][u] = make_float2(0.f, 0.f);
+    if (has1) {
+#pragma unroll 2
+      for (int y = 0; y < R2; ++y) {
+        const float2 b = b2[y * NT + il];
+        const float4* q = (const float4*)(qs + y * R1p);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float4 v0 = q[2 * (grp + c * GR)], v1 = q[2 * (grp + c * GR) + 1];
+          a[c][0] = cfma(make_float2(v0.x, v0.y), b, a[c][0]);
+          a[c][1] = cfma(make_float2(v0.z, v0.w), b, a[c][1]);
+          a[c][2] = cfma(make_float2(v1.x, v1.y), b, a[c][2]);
+          a[c][3] = cfma(make_float2(v1.z, v1.w), b, a[c][3]);
+        }
+      }
+    } else if (has0) {
+#pragma unroll 2
+      for (int y = 0; y < R2; ++y) {
+        const float2 b = b2[y * NT + il];
+        const float4* q = (const float4*)(qs + y * R1p);
+        const float4 v0 = q[2 * grp], v1 = q[2 * grp + 1];
+        a[0][0] = cfma(make_float2(v0.x, v0.y), b, a[0][0]);
+        a[0][1] = cfma(make_float2(v0.z, v0.w), b, a[0][1]);
+        a[0][2] = cfma(make_float2(v1.x, v1.y), b, a[0][2]);
+        a[0][3] = cfma(make_float2(v1.z, v1.w), b, a[0][3]);
+      }
+    }
+    const int e = exp_of(m) - 1;  // |S| < 12 max |Q| < 2^(e + 5): scaled below 2^(kDataShift + 5) = 2^15
+    const float sc = pow2f(kDataShift - e);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int kc = grp + c * GR;
+      if (kc < KB) {
+        uint32_t hr[4], lr[4], hi[4], li[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          // rows (Re, -Im) and (Im, Re) of the same words: swap the halves, flip the sign of Im
+          split2(a[c][u].x * sc, a[c][u].y * sc, hr[u], lr[u]);
+          hi[u] = __byte_perm(hr[u], 0, 0x1032);
+          li[u] = __byte_perm(lr[u], 0, 0x1032);
+          hr[u] ^= 0x80000000u;
+          lr[u] ^= 0x80000000u;
+        }
+        unsigned char* d0 = sb + tc::core_off(2 * il, kc, KB);
+        unsigned char* d1 = sb + tc::core_off(2 * il + 1, kc, KB);
+        *(uint4*)d0 = make_uint4(hr[0], hr[1], hr[2], hr[3]);
+        *(uint4*)(d0 + bbytes) = make_uint4(lr[0], lr[1], lr[2], lr[3]);
+        *(uint4*)d1 = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *(uint4*)(d1 + bbytes) = make_uint4(li[0], li[1], li[2], li[3]);
+      }
+    }
+    tc::fence_proxy_async();
+    __syncthreads();
+    const float us = pow2f(e - kDataShift - kBasisShift);
+    const int s = pl / G.n3, i3 = pl - s * G.n3;
+    float2* Yp = Y + ldy * s + (int64_t)k * nv + (int64_t)G.n1 * (i20 + (int64_t)G.n2 * i3) + row0;
+    auto epilogue = [&](int b) {
+      const int d = b & 1;
+      if (ok && !tc::mbar_wait(&done[d], ph[d])) {
+        ok = false;
+        abort_flag = 1;
+        atomicOr(err, kErrTimeout);
+      }
+      ph[d] ^= 1;
+      tc::fence_after();
+      const int i1 = b * 128 + 32 * q4;
+      if (i1 < rows && ok) {
+        const uint32_t t0 = tmem + (uint32_t)(d * 2 * NT + half * NT) + ((uint32_t)(32 * q4) << 16);
+        const int i2h = half * (NT / 2);
+        float2* y0 = Yp + (int64_t)G.n1 * i2h + i1 + lane;
+        const bool live = i1 + lane < rows;
+#pragma unroll
+        for (int c = 0; c < NT / 16; ++c) {
+          float v[16];
+          tc::tmem_ld16(t0 + 16 * c, v);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (live && (full2 || i20 + i2h + 8 * c + u < G.n2))
+              __stcs(y0 + (int64_t)G.n1 * (8 * c + u), make_float2(v[2 * u] * us, v[2 * u + 1] * us));
+        }
+      }
+      tc::fence_before();
+    };
+    for (int b = 0; b < nblk; ++b) {
+      if (tid == 0) {
+        tc::fence_after();
+        const uint32_t a0 = tc::smem_u32(sa) + (uint32_t)b * 2 * ablk, a1 = a0 + (b == nblk - 1 ? alast : ablk);
+        const uint32_t b0 = tc::smem_u32(sb), b1 = b0 + bbytes, sbo = KB * 128u;
+        const uint32_t d = tmem + (uint32_t)((b & 1) * 2 * NT), id = tc::instr_desc(128, 2 * NT, 0);
+        for (int ks = 0; ks < KB / 2; ++ks) {
+          const uint64_t ah = tc::smem_desc(a0 + ks * 256u, 128, sbo), al = tc::smem_desc(a1 + ks * 256u, 128, sbo);
+          const uint64_t bh = tc::smem_desc(b0 + ks * 256u, 128, sbo), bl = tc::smem_desc(b1 + ks * 256u, 128, sbo);
+          tc::mma<0>(d, al, bh, id, ks > 0);
+          tc::mma<0>(d, ah, bl, id, 1);
+          tc::mma<0>(d, ah, bh, id, 1);
+        }
+        tc::commit(&done[b & 1]);
+      }
+      if (b > 0) {
+        epilogue(b - 1);
+        __syncthreads();  // accumulator (b - 1) & 1 is free for block b + 1
+      }
+    }
+    // all threads pass the next plane's two barriers after this before anything is reused
+    epilogue(nblk - 1);
+  }
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+}
+
+// ---------------------------------------------------------------------------------------------
+// adjoint
+// ---------------------------------------------------------------------------------------------
+// Walks planes (k, s, i3).  Per tile of 128 i2 (the rows of D) Phi streams through registers in
+// chunks of 32 i1: 8 lanes hold a row's 32 entries, take the row's exponent, and write its scaled
+// hi / lo words (one 128-byte swizzled row per term) to one of two buffers; the basis rows of the
+// chunk (N = 2 NC, split once per handle) arrive by bulk copy.  12 MMAs a chunk (K = 64); the
+// accumulator is added into FP32 registers with the row's scale while the next chunk's MMAs run, so
+// each tensor-core sum has only 64 terms.  Then V (registers -> shared) is contracted with B2 on the
+// CUDA cores into Q, which stays in registers over the plane's tiles.
+constexpr int kTile2 = 128;   // i2 rows of a tile
+constexpr int kChunk1 = 32;   // i1 per chunk
+constexpr int kStage2 = 32;   // i2 per stage of B2
+constexpr uint32_t kATerm = kTile2 * 128u;
+
+inline size_t planes_adj_smem(int NC) {
+  return 4 * (size_t)kATerm + 2 * 2 * 2 * (size_t)NC * 128 + sizeof(float2) * kStage2 * ((NC + 15) / 16 * 16);
+}
+
+template <int I>  // NC = 8 I >= R1, R2 of every component
+__global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
+    joint_planes_adj_kernel(const __grid_constant__ JointGeo G, const unsigned char* __restrict__ bop,
+                            const float2* __restrict__ b2t, const float2* __restrict__ Phi, int64_t ldphi, int p,
+                            float2* __restrict__ Q, int* __restrict__ err) {
+  constexpr int NC = 8 * I, N = 2 * NC, RC = (NC + 15) / 16;  // Q: RC x RC entries a thread
+  constexpr int R2p = 16 * RC;
+  constexpr uint32_t kBTerm = N * 128u;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t done[2], full[2], ready[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ int rexp[4][kTile2];
+  unsigned char* sa = smem;                       // [2 buffers][2 terms][128 rows][128 B]; V after a tile
+  unsigned char* sb = sa + 4 * kATerm;            // [2 buffers][2 terms][N rows][128 B]
+  float2* b2s = (float2*)(sb + 4 * kBTerm);       // [kStage2][R2p]
+  float2* vs = (float2*)sa;                       // [NC][128]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr uint32_t ncols = N <= 16 ? 32 : N <= 32 ? 64 : N <= 64 ? 128 : 256;
+  if (tid == 0)
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&done[i], 1);
+      tc::mbar_init(&full[i], 1);
+      tc::mbar_init(&ready[i], 8);
+    }
+  if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
+  __syncthreads();
+  const uint32_t tmem = tmem_base;
+  const int nch = (G.n1 + kChunk1 - 1) / kChunk1, nt2 = (G.n2 + kTile2 - 1) / kTile2;
+  const int planes = G.n3 * p * G.q;  // plane = k + q (i3 + n3 s); a CTA's planes are blockIdx.x + g gridDim.x
+  const int mine = (planes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;  // grid <= planes
+  bool ok = true;  // false after a wait gave up: no further waits, the barriers are still passed
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (ok && !tc::mbar_wait_idle(bar, parity)) {
+      ok = false;
+      atomicOr(err, kErrTimeout);
+    }
+  };
+  if (warp == 8) {
+    if (lane == 0) {
+      // chunk c of this CTA (all tiles of all its planes in order): its B block is copied once the MMAs
+      // of chunk c - 2 have read the buffer
+      const int per = nch * nt2, total = mine * per;
+      int issued = 0;
+      auto copy_b = [&](int c) {
+        const int k = ((int)blockIdx.x + c / per * (int)gridDim.x) % G.q, ch = c % nch;
+        mbar_arrive_expect_tx(&full[c & 1], 2 * kBTerm);
+        bulk_g2s(sb + (size_t)(c & 1) * 2 * kBTerm, bop + ((size_t)k * nch + ch) * 2 * kBTerm, 2 * kBTerm, &full[c & 1]);
+        ++issued;
+      };
+      copy_b(0);
+      int c = 0;
+      for (; c < total; ++c) {
+        const int d = c & 1;
+        const uint32_t par = (c >> 1) & 1;
+        if (c > 0) wait(&done[d ^ 1], ((c - 1) >> 1) & 1);
+        if (!ok) break;
+        if (c + 1 < total) copy_b(c + 1);
+        wait(&full[d], par);
+        wait(&ready[d], par);
+        if (!ok) break;
+        tc::fence_after();
+        const uint32_t a0 = tc::smem_u32(sa) + d * 2 * kATerm, b0 = tc::smem_u32(sb) + d * 2 * kBTerm;
+        constexpr uint32_t id = tc::instr_desc(128, N, 0);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          const uint64_t ah = tc::smem_desc_sw128(a0 + ks * 32), al = tc::smem_desc_sw128(a0 + kATerm + ks * 32);
+          const uint64_t bh = tc::smem_desc_sw128(b0 + ks * 32), bl = tc::smem_desc_sw128(b0 + kBTerm + ks * 32);
+          tc::mma<0>(tmem + d * N, al, bh, id, ks > 0);
+          tc::mma<0>(tmem + d * N, ah, bl, id, 1);
+          tc::mma<0>(tmem + d * N, ah, bh, id, 1);
+        }
+        tc::commit(&done[d]);
+      }
+      // after giving up: the copies in flight land before the buffers are left
+      for (int i = c; i < issued; ++i) tc::mbar_wait_idle(&full[i & 1], (i >> 1) & 1);
+    }
+    __syncwarp();
+  } else {
+    const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
+    const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // loader: rows row0 + 32 u, i1 = c8 + 8 w
+    const int q4 = warp & 3, half = warp >> 2;            // accumulator rows and columns
+    const int tx = tid % 16, ty = tid / 16;
+    bool bad = false;
+    // a work item is one tile of one plane: Phi at the loader's first row and i1, and the tile's rows
+    const float2* src = nullptr;
+    int rows = 0;
+    auto locate = [&](int plane, int t2) {
+      const int k = plane % G.q, i3 = plane / G.q % G.n3, s = plane / G.q / G.n3;
+      rows = min(kTile2, G.n2 - t2 * kTile2);
+      src = Phi + ldphi * s + (int64_t)k * nv + (int64_t)G.n1 * ((int64_t)G.n2 * i3 + t2 * kTile2 + row0) + c8;
+    };
+    float2 x[4][4];
+    auto fetch = [&](int ch) {
+      const int left = G.n1 - ch * kChunk1 - c8;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float2* g = src + (int64_t)G.n1 * (32 * u) + ch * kChunk1;
+        const bool live = row0 + 32 * u < rows;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) x[u][w] = live && 8 * w < left ? __ldcs(g + 8 * w) : make_float2(0.f, 0.f);
+      }
+    };
+    float2 qa[RC][RC];
+    int c0 = 0;  // the CTA's chunk number of this item's first chunk
+    locate(blockIdx.x, 0);
+    fetch(0);
+    for (int item = 0; item < mine * nt2; ++item, c0 += nch) {
+      const int plane = (int)blockIdx.x + item / nt2 * (int)gridDim.x, t2 = item % nt2, k = plane % G.q;
+      if (t2 == 0)
+#pragma unroll
+        for (int a = 0; a < RC; ++a)
+#pragma unroll
+          for (int b = 0; b < RC; ++b) qa[a][b] = make_float2(0.f, 0.f);
+      float acc[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = 0.f;
+      auto fold = [&](int c) {  // also: the MMAs have read chunk c's buffer
+        const int d = c & 1;
+        wait(&done[d], (c >> 1) & 1);
+        tc::fence_after();
+        if (32 * q4 < rows) {
+          const float us = pow2f(rexp[c & 3][32 * q4 + lane] - kDataShift - kBasisShift);
+          const uint32_t t0 = tmem + (uint32_t)(d * N + half * NC) + ((uint32_t)(32 * q4) << 16);
+#pragma unroll
+          for (int i = 0; i < I; ++i) {
+            uint32_t r[8];
+            tmem_ld8(t0 + 8 * i, r);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc[8 * i + u] = fmaf(__uint_as_float(r[u]), us, acc[8 * i + u]);
+          }
+        }
+        tc::fence_before();
+      };
+      for (int ch = 0; ch < nch; ++ch) {
+        const int c = c0 + ch, d = c & 1;
+        if (ch >= 2) fold(c - 2);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (warp * 4 + 32 * u >= rows) continue;  // rows past the grid: their D rows are not used
+          float m = 0.f;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) m = absmax_nan(m, x[u][w].x, x[u][w].y);
+          m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 1));
+          m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
+          m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
+          bad = bad || !(m < INFINITY);
+          const int e = exp_of(m), r = row0 + 32 * u;
+          if (c8 == 0) rexp[c & 3][r] = e;
+          const float sc = pow2f(kDataShift - e);
+          uint32_t h[4], l[4];
+#pragma unroll
+          for (int w = 0; w < 4; ++w) split2(x[u][w].x * sc, x[u][w].y * sc, h[w], l[w]);
+          unsigned char* o = sa + (size_t)d * 2 * kATerm + tc::sw128_off(r, c8);
+          *(uint4*)o = make_uint4(h[0], h[1], h[2], h[3]);
+          *(uint4*)(o + kATerm) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+        if (ch + 1 < nch) fetch(ch + 1);
+        warp_publish(&ready[d]);
+      }
+      if (nch > 1) fold(c0 + nch - 2);
+      fold(c0 + nch - 1);
+      // the next item's first chunk is on its way during the contraction with B2
+      const int done_rows = rows;
+      if (item + 1 < mine * nt2) {
+        locate(t2 + 1 < nt2 ? plane : plane + (int)gridDim.x, t2 + 1 < nt2 ? t2 + 1 : 0);
+        fetch(0);
+      }
+      // V: row i2 = 32 q4 + lane, columns (Re, Im) of x = half NC / 2 + c
+#pragma unroll
+      for (int c = 0; c < NC / 2; ++c)
+        vs[(half * (NC / 2) + c) * kTile2 + 32 * q4 + lane] =
+            32 * q4 + lane < done_rows ? make_float2(acc[2 * c], acc[2 * c + 1]) : make_float2(0.f, 0.f);
+      const float4* bsrc = (const float4*)(b2t + ((int64_t)k * nt2 + t2) * kTile2 * R2p);
+      for (int j0 = 0; j0 < done_rows; j0 += kStage2) {
+        if (j0 > 0) worker_barrier();
+#pragma unroll
+        for (int e = 0; e < kStage2 * R2p / 512; ++e)
+          ((float4*)b2s)[tid + 256 * e] = __ldg(bsrc + j0 * R2p / 2 + tid + 256 * e);
+        worker_barrier();
+#pragma unroll 2
+        for (int j = 0; j < kStage2; j += 2) {
+          float4 v[RC];
+#pragma unroll
+          for (int a = 0; a < RC; ++a) {
+            const int xx = ty + 16 * a;
+            v[a] = NC % 16 == 0 || xx < NC ? *(const float4*)&vs[xx * kTile2 + j0 + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+#pragma unroll
+          for (int b = 0; b < RC; ++b) {
+            const float2 e0 = b2s[j * R2p + tx + 16 * b], e1 = b2s[(j + 1) * R2p + tx + 16 * b];
+#pragma unroll
+            for (int a = 0; a < RC; ++a) {
+              qa[a][b] = cfma_conj(e0, make_float2(v[a].x, v[a].y), qa[a][b]);
+              qa[a][b] = cfma_conj(e1, make_float2(v[a].z, v[a].w), qa[a][b]);
+            }
+          }
+        }
+      }
+      worker_barrier();  // V is read before the next item overwrites the buffers
+      if (t2 == nt2 - 1) {
+        const int i3 = plane / G.q % G.n3, s = plane / G.q / G.n3, R1 = G.R[k][0], R2 = G.R[k][1];
+        float2* Qp = Q + (int64_t)s * G.Qt + G.qoff[k] + (int64_t)i3 * R1 * R2;
+#pragma unroll
+        for (int a = 0; a < RC; ++a)
+#pragma unroll
+          for (int b = 0; b < RC; ++b) {
+            const int xx = ty + 16 * a, y = tx + 16 * b;
+            if (xx < R1 && y < R2) Qp[xx + R1 * y] = qa[a][b];
+          }
+      }
+    }
+    if (bad) atomicOr(err, kErrNonFinite);
+  }
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+}
+
+// B1's rows of the adjoint: per component and chunk of 32 i1, [term][2 x + e][64 fp16], 128-byte
+// swizzled, the 16-byte chunk c holding i1 = c, c + 8, c + 16, c + 24 (the order in which 8 lanes read
+// Phi without gaps); one thread per (row pair, 16-byte chunk)
+__global__ void __launch_bounds__(256) split_basis_kernel(const __grid_constant__ JointGeo G,
+                                                          const float2* __restrict__ basis, int NC, int nch,
+                                                          unsigned char* __restrict__ out) {
+  const int k = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
+  const int c8 = e % 8, x = e / 8 % NC, ch = e / (8 * NC);
+  if (ch >= nch) return;
+  uint32_t h0[4], l0[4], h1[4], l1[4];
+  for (int w = 0; w < 4; ++w) {
+    const int i1 = ch * kChunk1 + c8 + 8 * w;
+    const float2 v = x < G.R[k][0] && i1 < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i1] : make_float2(0.f, 0.f);
+    const float re = v.x * pow2f(kBasisShift), im = v.y * pow2f(kBasisShift);
+    split2(re, im, h0[w], l0[w]);
+    split2(-im, re, h1[w], l1[w]);
+  }
+  const size_t term = (size_t)2 * NC * 128;
+  unsigned char* o = out + ((size_t)k * nch + ch) * 2 * term;
+  *(uint4*)(o + tc::sw128_off(2 * x, c8)) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+  *(uint4*)(o + term + tc::sw128_off(2 * x, c8)) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
+  *(uint4*)(o + tc::sw128_off(2 * x + 1, c8)) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+  *(uint4*)(o + term + tc::sw128_off(2 * x + 1, c8)) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
+}
+
+int max_r(const JointGeo& G, int m) {
+  int r = 0;
+  for (int k = 0; k < G.q; ++k) r = std::max(r, G.R[k][m]);
+  return r;
+}
+int adj_rows(const JointGeo& G) { return ceil_div(std::max(max_r(G, 0), max_r(G, 1)), 8) * 8; }
+size_t bop_bytes(const JointGeo& G) { return (size_t)G.q * ceil_div(G.n1, kChunk1) * 2 * 2 * adj_rows(G) * 128; }
+int b2t_rows(const JointGeo& G) { return ceil_div(G.n2, kTile2) * kTile2; }
+int b2t_cols(const JointGeo& G) { return ceil_div(adj_rows(G), 16) * 16; }
+
+template <int NT>
+int launch_planes_fwd(const JointGeo& G, const float2* basis, const float2* Q, int p, float2* Y, int64_t ldy, int* err,
+                      cudaStream_t st) {
+  const int R1p = ceil_div(max_r(G, 0), 8) * 8, R2p = ceil_div(max_r(G, 1), 2) * 2, nblk = ceil_div(G.n1, 128);
+  const size_t arow = (size_t)8 * R1p;  // bytes of one row of B1, both terms
+  const size_t rest = (size_t)16 * NT * R1p + sizeof(float2) * R2p * (R1p + NT);
+  // two CTAs an SM while at least one i1 block of B1 fits beside the rest; the last block's MMAs read
+  // up to 128 rows of one term past the rows that are stored
+  constexpr size_t kLimit = 115456;  // (228 KB / 2 - 1 KB reserved), less the static variables
+  const size_t over = 64 * (size_t)R1p * 8;
+  auto bytes = [&](int nb) { return rest + over + std::min(nb * 128, ceil_div(G.n1, 8) * 8) * arow; };
+  int nb = nblk;
+  while (nb > 1 && bytes(nb) > kLimit) --nb;
+  const size_t sm = bytes(nb);
+  ZBC_TRY(set_smem_limit<joint_planes_fwd_kernel<NT>>(200 * 1024));
+  const int gy = ceil_div(nblk, nb) * ceil_div(G.n2, NT), per_sm = sm <= kLimit ? 2 : 1;
+  const int walkers = std::min(p * G.n3, std::max(1, per_sm * sm_count() / (gy * G.q)));
+  joint_planes_fwd_kernel<NT><<<dim3(walkers, gy, G.q), 256, sm, st>>>(G, basis, Q, R1p, R2p, nb, p, Y, ldy, err);
+  count_launch();
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
+}
+
+// B2 by i2: per component [n2 rounded up to tiles][R2p], zeros past n2 and R2
+__global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_constant__ JointGeo G,
+                                                              const float2* __restrict__ basis, int rows, int R2p,
+                                                              float2* __restrict__ out) {
+  const int k = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x, y = e % R2p, i2 = e / R2p;
+  if (i2 >= rows) return;
+  out[((int64_t)k * rows + i2) * R2p + y] =
+      i2 < G.n2 && y < G.R[k][1] ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i2] : make_float2(0.f, 0.f);
+}
+
+template <int I>
+int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
+                      int* err, cudaStream_t st) {
+  const float2* b2t = (const float2*)(bop + bop_bytes(G));
+  ZBC_TRY(set_smem_limit<joint_planes_adj_kernel<I>>((int)planes_adj_smem(8 * I)));
+  const size_t sm = planes_adj_smem(8 * I);
+  const int64_t planes = (int64_t)G.n3 * p * G.q;
+  const int grid = (int)std::min<int64_t>(planes, (sm <= 112 * 1024 ? 2 : 1) * sm_count());
+  joint_planes_adj_kernel<I><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err);
+  count_launch();
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
+}
+
+}  // namespace
+
+int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st) {
+  if (std::max(max_r(jc.geo, 0), max_r(jc.geo, 1)) <= 32) return launch_planes_fwd<64>(jc.geo, jc.basis, Q, p, Y, ldy, err, st);
+  return launch_planes_fwd<32>(jc.geo, jc.basis, Q, p, Y, ldy, err, st);
+}
+
+int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
+                     cudaStream_t st) {
+  const JointGeo& G = jc.geo;
+  switch (adj_rows(G) / 8) {
+    case 1: return launch_planes_adj<1>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 2: return launch_planes_adj<2>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 3: return launch_planes_adj<3>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 4: return launch_planes_adj<4>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 5: return launch_planes_adj<5>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 6: return launch_planes_adj<6>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 7: return launch_planes_adj<7>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    default: return launch_planes_adj<8>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+  }
+}
+
+size_t joint_planes_bytes(const JointGeo& G) {
+  return bop_bytes(G) + sizeof(float2) * (size_t)G.q * b2t_rows(G) * b2t_cols(G);
+}
+
+int joint_planes_build(const JointGeo& G, const float2* basis, unsigned char* bop, cudaStream_t st) {
+  const int NC = adj_rows(G), nch = ceil_div(G.n1, kChunk1);
+  split_basis_kernel<<<dim3(ceil_div((int64_t)nch * NC * 8, 256), G.q), 256, 0, st>>>(G, basis, NC, nch, bop);
+  const int rows = b2t_rows(G), cols = b2t_cols(G);
+  transpose_basis_kernel<<<dim3(ceil_div((int64_t)rows * cols, 256), G.q), 256, 0, st>>>(G, basis, rows, cols,
+                                                                                         (float2*)(bop + bop_bytes(G)));
+  count_launch(2);
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
+}
+
+}  // namespace zbc

@@ -1,9 +1,9 @@
-// The products through a joint basis of the columns' factors (joint.cuh), FP32 on CUDA cores.
+// The products through a joint basis of the columns' factors (joint.cuh).
 //
 // Forward:  T = sum_j K_j X[j, :]        joint_core_fwd_kernel    (R1 R2 R3 entries per component)
 //           Q[i3] = T x3 B3              joint_mode3_fwd_kernel
-//           Y[:, :, i3] = B1 Q[i3] B2^T  joint_plane_fwd_kernel   (one write of Y)
-// Adjoint:  Q[i3] = B1^H Phi[:, :, i3] conj(B2)   joint_plane_adj_kernel   (one read of Phi)
+//           Y[:, :, i3] = B1 Q[i3] B2^T  joint_planes.cu          (one write of Y)
+// Adjoint:  Q[i3] = B1^H Phi[:, :, i3] conj(B2)   joint_planes.cu          (one read of Phi)
 //           F = Q x3 B3^H                         joint_mode3_adj_kernel
 //           Psi[j, :] = sum conj(K_j) F           joint_core_adj_kernel, joint_sum_kernel
 #include <algorithm>
@@ -105,190 +105,6 @@ __global__ void __launch_bounds__(128) joint_mode3_fwd_kernel(const __grid_const
 #pragma unroll
   for (int z = 0; z < kZ; ++z)
     if (z0 + z < G.n3) o[(int64_t)(z0 + z) * RR] = acc[z];
-}
-
-constexpr int kI2 = 32;  // i2 values of a plane tile (forward)
-
-inline size_t plane_fwd_smem(int R1, int R2, int NI) {
-  return sizeof(float2) * ((size_t)R1 * 32 * NI + (size_t)R1 * kI2 + (size_t)R1 * R2 + (size_t)R2 * kI2);
-}
-
-// Y[i1, i2, i3, s] = sum_xy B1[i1, x] Q[s][i3][x, y] B2[i2, y]: a CTA keeps B1 of its block of
-// 32 NI rows in shared memory and walks (s, i3, tile of 32 i2): S = Q B2^T of the tile (R1 x 32),
-// then B1 S, one thread NI i1 (stride 32) x 4 i2.  Grid (walkers, i1 blocks, q).
-template <int NI>
-__global__ void __launch_bounds__(256) joint_plane_fwd_kernel(const __grid_constant__ JointGeo G,
-                                                              const float2* __restrict__ basis, const float2* __restrict__ Q,
-                                                              int p, float2* __restrict__ Y, int64_t ldy) {
-  extern __shared__ __align__(16) float2 sm[];
-  const int k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1], RR = R1 * R2;
-  constexpr int BW = 32 * NI;
-  float2* b1 = sm;                // [R1][BW]
-  float2* ss = b1 + R1 * BW;      // [R1][kI2]
-  float2* b2 = ss + R1 * kI2;     // [R2][kI2]
-  float2* qs = b2 + R2 * kI2;     // [R2][R1]
-  const int i10 = blockIdx.y * BW, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int e = threadIdx.x; e < R1 * BW; e += 256) {
-    const int il = e % BW, x = e / BW;
-    b1[e] = i10 + il < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i10 + il] : make_float2(0.f, 0.f);
-  }
-  const int nt2 = (G.n2 + kI2 - 1) / kI2;
-  const int64_t items = (int64_t)p * G.n3 * nt2;
-  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
-  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-    const int i20 = (int)(it % nt2) * kI2;
-    const int i3 = (int)(it / nt2 % G.n3), s = (int)(it / nt2 / G.n3);
-    const float2* Qp = Q + (int64_t)s * G.Qt + G.qoff[k] + (int64_t)i3 * RR;
-    __syncthreads();
-    for (int e = threadIdx.x; e < RR; e += 256) qs[e] = Qp[e];
-    for (int e = threadIdx.x; e < R2 * kI2; e += 256) {
-      const int il = e % kI2, y = e / kI2;
-      b2[e] = i20 + il < G.n2 ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i20 + il] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < R1 * (kI2 / 4); e += 256) {
-      const int x = e % R1, i4 = e / R1 * 4;
-      float2 a[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = make_float2(0.f, 0.f);
-      for (int y = 0; y < R2; ++y) {
-        const float2 v = qs[x + R1 * y];
-        const float4 c0 = *(const float4*)&b2[y * kI2 + i4], c1 = *(const float4*)&b2[y * kI2 + i4 + 2];
-        a[0] = cfma(v, make_float2(c0.x, c0.y), a[0]);
-        a[1] = cfma(v, make_float2(c0.z, c0.w), a[1]);
-        a[2] = cfma(v, make_float2(c1.x, c1.y), a[2]);
-        a[3] = cfma(v, make_float2(c1.z, c1.w), a[3]);
-      }
-      *(float4*)&ss[x * kI2 + i4] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-      *(float4*)&ss[x * kI2 + i4 + 2] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
-    }
-    __syncthreads();
-    float2 acc[NI][4];
-#pragma unroll
-    for (int i = 0; i < NI; ++i)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[i][u] = make_float2(0.f, 0.f);
-#pragma unroll 2
-    for (int x = 0; x < R1; ++x) {
-      const float4 c0 = *(const float4*)&ss[x * kI2 + 4 * warp], c1 = *(const float4*)&ss[x * kI2 + 4 * warp + 2];
-#pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        const float2 b = b1[x * BW + lane + 32 * i];
-        acc[i][0] = cfma(b, make_float2(c0.x, c0.y), acc[i][0]);
-        acc[i][1] = cfma(b, make_float2(c0.z, c0.w), acc[i][1]);
-        acc[i][2] = cfma(b, make_float2(c1.x, c1.y), acc[i][2]);
-        acc[i][3] = cfma(b, make_float2(c1.z, c1.w), acc[i][3]);
-      }
-    }
-    float2* Yp = Y + ldy * s + (int64_t)k * nv + (int64_t)G.n1 * (i20 + 4 * warp + (int64_t)G.n2 * i3) + i10 + lane;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (i20 + 4 * warp + u < G.n2)
-#pragma unroll
-        for (int i = 0; i < NI; ++i)
-          if (i10 + lane + 32 * i < G.n1) __stcs(Yp + (int64_t)G.n1 * u + 32 * i, acc[i][u]);
-  }
-}
-
-constexpr int kA2 = 64;       // i2 values of a plane tile (adjoint)
-constexpr int kA1 = 32;       // i1 values per chunk
-constexpr int kPs = kA2 + 2;  // row strides: 16-byte aligned rows, stores over i1 spread over the banks
-
-// Q[s][i3][x, y] = sum over i1, i2 of conj(B1[i1, x]) conj(B2[i2, y]) Phi[i1, i2, i3, s]: one CTA per
-// plane (i3, s, k).  Per tile of 64 i2: V = B1^H Phi over i1 chunks of 32 (a thread holds RA x by
-// 4 i2), then Q += V conj(B2) (RA x by RB y, kept in registers over the tiles).  Grid (n3, p, q).
-template <int RA, int RB>
-__global__ void __launch_bounds__(128) joint_plane_adj_kernel(const __grid_constant__ JointGeo G,
-                                                              const float2* __restrict__ basis,
-                                                              const float2* __restrict__ Phi, int64_t ldphi,
-                                                              float2* __restrict__ Q, int* __restrict__ err) {
-  extern __shared__ __align__(16) float2 sm[];
-  const int i3 = blockIdx.x, s = blockIdx.y, k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1];
-  float2* ph = sm;                     // [kA1][kPs]
-  float2* b1 = ph + kA1 * kPs;         // [kA1][8 RA]
-  float2* vs = b1 + kA1 * 8 * RA;      // [8 RA][kA2 + 1]
-  float2* b2 = vs + 8 * RA * (kA2 + 1);  // [kA2][16 RB]
-  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
-  const float2* P0 = Phi + ldphi * s + (int64_t)k * nv + (int64_t)G.n1 * G.n2 * i3;
-  const float2* B1 = basis + G.boff[k][0];
-  const float2* B2 = basis + G.boff[k][1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // i2 group or y group; x group
-  const int il = threadIdx.x % 32, w4 = threadIdx.x / 32;
-  float2 qa[RA][RB];
-#pragma unroll
-  for (int a = 0; a < RA; ++a)
-#pragma unroll
-    for (int b = 0; b < RB; ++b) qa[a][b] = make_float2(0.f, 0.f);
-  bool bad = false;
-  for (int i20 = 0; i20 < G.n2; i20 += kA2) {
-    float2 va[RA][4];
-#pragma unroll
-    for (int a = 0; a < RA; ++a)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) va[a][u] = make_float2(0.f, 0.f);
-    for (int i10 = 0; i10 < G.n1; i10 += kA1) {
-      float2 t[kA2 / 4];
-#pragma unroll
-      for (int u = 0; u < kA2 / 4; ++u) {
-        const int i2 = i20 + w4 + 4 * u;
-        t[u] = i10 + il < G.n1 && i2 < G.n2 ? __ldcs(P0 + (int64_t)G.n1 * i2 + i10 + il) : make_float2(0.f, 0.f);
-      }
-      __syncthreads();  // the previous chunk has been read
-#pragma unroll
-      for (int u = 0; u < kA2 / 4; ++u) {
-        bad = bad || !finite2(t[u]);
-        ph[il * kPs + w4 + 4 * u] = t[u];
-      }
-      for (int e = threadIdx.x; e < kA1 * 8 * RA; e += 128) {
-        const int i = e % kA1, x = e / kA1;
-        b1[i * 8 * RA + x] = x < R1 && i10 + i < G.n1 ? B1[(int64_t)x * G.n1 + i10 + i] : make_float2(0.f, 0.f);
-      }
-      __syncthreads();
-#pragma unroll 4
-      for (int i = 0; i < kA1; ++i) {
-        const float4 p0 = *(const float4*)&ph[i * kPs + 4 * tx], p1 = *(const float4*)&ph[i * kPs + 4 * tx + 2];
-#pragma unroll
-        for (int a = 0; a < RA; ++a) {
-          const float2 b = b1[i * 8 * RA + ty * RA + a];
-          va[a][0] = cfma_conj(b, make_float2(p0.x, p0.y), va[a][0]);
-          va[a][1] = cfma_conj(b, make_float2(p0.z, p0.w), va[a][1]);
-          va[a][2] = cfma_conj(b, make_float2(p1.x, p1.y), va[a][2]);
-          va[a][3] = cfma_conj(b, make_float2(p1.z, p1.w), va[a][3]);
-        }
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < RA; ++a)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) vs[(ty * RA + a) * (kA2 + 1) + 4 * tx + u] = va[a][u];
-    for (int e = threadIdx.x; e < kA2 * 16 * RB; e += 128) {
-      const int i = e % kA2, y = e / kA2;
-      b2[i * 16 * RB + y] = y < R2 && i20 + i < G.n2 ? B2[(int64_t)y * G.n2 + i20 + i] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int i = 0; i < kA2; ++i) {
-      float2 c[RB];
-#pragma unroll
-      for (int b = 0; b < RB; ++b) c[b] = b2[i * 16 * RB + tx + 16 * b];
-#pragma unroll
-      for (int a = 0; a < RA; ++a) {
-        const float2 v = vs[(ty * RA + a) * (kA2 + 1) + i];
-#pragma unroll
-        for (int b = 0; b < RB; ++b) qa[a][b] = cfma_conj(c[b], v, qa[a][b]);
-      }
-    }
-    // vs and b2 are written again only after the next tile's first barriers
-  }
-  if (bad) atomicOr(err, kErrNonFinite);
-  float2* Qp = Q + (int64_t)s * G.Qt + G.qoff[k] + (int64_t)i3 * R1 * R2;
-#pragma unroll
-  for (int a = 0; a < RA; ++a)
-#pragma unroll
-    for (int b = 0; b < RB; ++b) {
-      const int x = ty * RA + a, y = tx + 16 * b;
-      if (x < R1 && y < R2) Qp[x + R1 * y] = qa[a][b];
-    }
 }
 
 // F[s][toff + xy + RR z] = sum_i3 conj(B3[i3, z]) Q[s][qoff + i3 RR + xy]; entries up to Cs are zero
@@ -455,46 +271,6 @@ constexpr int kPassRhs = 64;  // right-hand sides per round of the workspaces
 
 int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : p <= 4 ? 4 : p <= 8 ? 8 : 16; }
 
-template <int NI>
-int launch_plane_fwd(const JointGeo& G, const float2* basis, const float2* Q, int p, float2* Y, int64_t ldy,
-                     cudaStream_t st) {
-  ZBC_TRY(set_smem_limit<joint_plane_fwd_kernel<NI>>((int)plane_fwd_smem(kJointRmax, kJointRmax, NI)));
-  size_t sm = 0;
-  for (int k = 0; k < G.q; ++k) sm = std::max(sm, plane_fwd_smem(G.R[k][0], G.R[k][1], NI));
-  const int nb = ceil_div(G.n1, 32 * NI);
-  int occ = 0;
-  ZBC_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, joint_plane_fwd_kernel<NI>, 256, sm));
-  const int64_t items = (int64_t)p * G.n3 * ceil_div(G.n2, kI2);
-  const int walkers = (int)std::min<int64_t>(items, std::max(1, std::max(1, occ) * sm_count() / (nb * G.q)));
-  joint_plane_fwd_kernel<NI><<<dim3(walkers, nb, G.q), 256, sm, st>>>(G, basis, Q, p, Y, ldy);
-  count_launch();
-  ZBC_TRY_CUDA(cudaGetLastError());
-  return ZBC_OK;
-}
-
-template <int RA, int RB>
-int launch_plane_adj(const JointGeo& G, const float2* basis, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
-                     cudaStream_t st) {
-  constexpr size_t sm = sizeof(float2) * ((size_t)kA1 * kPs + (size_t)kA1 * 8 * RA + (size_t)8 * RA * (kA2 + 1) +
-                                          (size_t)kA2 * 16 * RB);
-  ZBC_TRY((set_smem_limit<joint_plane_adj_kernel<RA, RB>>((int)sm)));
-  joint_plane_adj_kernel<RA, RB><<<dim3(G.n3, p, G.q), 128, sm, st>>>(G, basis, Phi, ldphi, Q, err);
-  count_launch();
-  ZBC_TRY_CUDA(cudaGetLastError());
-  return ZBC_OK;
-}
-
-template <int RA>
-int plane_adj_rb(int RB, const JointGeo& G, const float2* basis, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
-                 cudaStream_t st) {
-  switch (RB) {
-    case 1: return launch_plane_adj<RA, 1>(G, basis, Phi, ldphi, p, Q, err, st);
-    case 2: return launch_plane_adj<RA, 2>(G, basis, Phi, ldphi, p, Q, err, st);
-    case 3: return launch_plane_adj<RA, 3>(G, basis, Phi, ldphi, p, Q, err, st);
-    default: return launch_plane_adj<RA, 4>(G, basis, Phi, ldphi, p, Q, err, st);
-  }
-}
-
 template <int P>
 void launch_core_fwd(const JointGeo& G, const float2* K, const float2* X, int64_t ldx, int p, int JS, float2* T, int* err,
                      int csmax, cudaStream_t st) {
@@ -574,23 +350,7 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
     }
     joint_mode3_fwd_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(G.n3, kZ), ps * G.q), 128, 0, st>>>(G, jc.basis, T, ps, JS, Q);
     count_launch(2);
-    // i1 block of 32 NI rows: the fewest padded rows, then the largest block
-    int NI = 1, pad = 1 << 30;
-    for (int ni = 1; ni <= 5; ++ni) {
-      const int rows = ceil_div(G.n1, 32 * ni) * 32 * ni;
-      if (rows <= pad) {
-        pad = rows;
-        NI = ni;
-      }
-    }
-    float2* Ys = Y + ldy * s0;
-    switch (NI) {
-      case 1: ZBC_TRY(launch_plane_fwd<1>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
-      case 2: ZBC_TRY(launch_plane_fwd<2>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
-      case 3: ZBC_TRY(launch_plane_fwd<3>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
-      case 4: ZBC_TRY(launch_plane_fwd<4>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
-      default: ZBC_TRY(launch_plane_fwd<5>(G, jc.basis, Q, ps, Ys, ldy, st)); break;
-    }
+    ZBC_TRY(joint_planes_fwd(jc, Q, ps, Y + ldy * s0, ldy, err, st));
   }
   return ZBC_OK;
 }
@@ -600,14 +360,11 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
   const JointGeo& G = jc.geo;
   int* err = (int*)h.work_err.ptr;
   ZBC_TRY(h.work_joint.ensure(joint_work_bytes(h, p, false)));
-  int r1 = 0, r2 = 0, r3 = 0, rrmax = 0;
+  int r3 = 0, rrmax = 0;
   for (int k = 0; k < G.q; ++k) {
-    r1 = std::max(r1, G.R[k][0]);
-    r2 = std::max(r2, G.R[k][1]);
     r3 = std::max(r3, G.R[k][2]);
     rrmax = std::max(rrmax, G.R[k][0] * G.R[k][1]);
   }
-  const int RA = ceil_div(r1, 8), RB = ceil_div(r2, 16);
   for (int s0 = 0; s0 < p; s0 += kPassRhs) {
     const int ps = std::min(kPassRhs, p - s0);
     const AdjPlan pl(G, ps);
@@ -616,16 +373,7 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
     float2* F = Q + pl.qelems;
     float2* part = F + pl.felems;
     const float2* Ps = Phi + ldphi * s0;
-    switch (RA) {
-      case 1: ZBC_TRY(plane_adj_rb<1>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 2: ZBC_TRY(plane_adj_rb<2>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 3: ZBC_TRY(plane_adj_rb<3>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 4: ZBC_TRY(plane_adj_rb<4>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 5: ZBC_TRY(plane_adj_rb<5>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 6: ZBC_TRY(plane_adj_rb<6>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      case 7: ZBC_TRY(plane_adj_rb<7>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-      default: ZBC_TRY(plane_adj_rb<8>(RB, G, jc.basis, Ps, ldphi, ps, Q, err, st)); break;
-    }
+    ZBC_TRY(joint_planes_adj(jc, Ps, ldphi, ps, Q, err, st));
     joint_mode3_adj_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(r3, 8), ps * G.q), 128, 0, st>>>(G, jc.basis, Q, F);
     switch (pl.P) {
       case 1: launch_core_adj<1>(G, jc.K, F, ps, chunk, splits, part, st); break;
