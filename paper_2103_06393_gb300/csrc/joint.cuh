@@ -40,6 +40,7 @@ struct JointCache {
   float2* basis = nullptr;
   float2* K = nullptr;
   unsigned char* bop = nullptr;  // B1 split for the adjoint's plane product (joint_planes.cu)
+  float* kscale = nullptr;       // power-of-two scales of K's columns (joint_core.cu)
   int64_t bytes = 0;
 };
 
@@ -48,6 +49,14 @@ size_t joint_planes_bytes(const JointGeo& G);
 int joint_planes_build(const JointGeo& G, const float2* basis, unsigned char* bop, cudaStream_t st);
 int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st);
 int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err, cudaStream_t st);
+
+// the column sums on the tensor cores (joint_core.cu): T from X, and partial Psi from F in `splits`
+// slices of `split` chunks of core entries
+size_t joint_core_bytes(const JointGeo& G);
+int joint_core_build(const JointGeo& G, const float2* K, float* kscale, cudaStream_t st);
+int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, cudaStream_t st);
+void joint_core_split(const JointGeo& G, int p, int* split, int* splits);
+int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, cudaStream_t st);
 
 // Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
 int build_joint(Handle& h, cudaStream_t st);

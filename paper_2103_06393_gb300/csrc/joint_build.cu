@@ -20,6 +20,7 @@ void joint_release(JointCache* c) {
   if (c->basis) cudaFree(c->basis);
   if (c->K) cudaFree(c->K);
   if (c->bop) cudaFree(c->bop);
+  if (c->kscale) cudaFree(c->kscale);
   delete c;
 }
 int64_t joint_bytes(const JointCache* c) { return c ? c->bytes : 0; }
@@ -406,11 +407,12 @@ int build_joint(Handle& h, cudaStream_t st) {
   cudaError_t e = cudaMalloc(&jc->basis, sizeof(float2) * belems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->K, sizeof(float2) * kelems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->bop, joint_planes_bytes(g));
+  if (e == cudaSuccess) e = cudaMalloc(&jc->kscale, joint_core_bytes(g));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return ZBC_OK;  // no room: unusable
   }
-  jc->bytes = (int64_t)(sizeof(float2) * (belems + kelems) + joint_planes_bytes(g));
+  jc->bytes = (int64_t)(sizeof(float2) * (belems + kelems) + joint_planes_bytes(g) + joint_core_bytes(g));
   for (int k = 0; k < q; ++k)
     for (int m = 0; m < 3; ++m) {
       const int64_t len = (int64_t)n[m] * g.R[k][m];
@@ -454,8 +456,8 @@ int build_joint(Handle& h, cudaStream_t st) {
     core3_kernel<<<dim3(std::min(64, ceil_div(csmax / kCoreZ + 1, 256)), nt), 256, 0, st>>>(p);
     count_launch(3);
   }
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  ZBC_TRY(joint_core_build(g, jc->K, jc->kscale, st));
+  e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e, "reduced cores");
   jc->usable = true;
   return ZBC_OK;

@@ -13,73 +13,12 @@
 //   A[i1] = (Re, Im) B1[i1, :]  and  B rows (Re S, -Im S), (Im S, Re S)
 // D's column pair is (Re, Im) Y; the adjoint contracts Phi's own (Re, Im) pairs along i1 with rows
 // (Re b, Im b), (-Im b, Re b) of the basis vector b, which gives (Re, Im) of conj(b) Phi.
-#include <cuda_fp16.h>
-
 #include <algorithm>
 
-#include "joint.cuh"
-#include "stage.cuh"
+#include "joint_tc.cuh"
 
 namespace zbc {
 namespace {
-
-constexpr int kBasisShift = 10;  // basis entries (|b| <= 1) are scaled by 2^10
-constexpr int kDataShift = 10;   // the other operand is brought below 2^10
-
-// fp16 hi / lo of a scaled pair, as words (x low)
-__device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(x, y);
-  const float2 f = __half22float2(h);
-  const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
-// e with m < 2^e, at least -100 so that 2^(kDataShift - e) and its inverse are normal floats (0 for
-// zero and for values that are not finite, which go through unscaled)
-__device__ __forceinline__ int exp_of(float m) {
-  if (!(m > 0.f) || !(m < INFINITY)) return 0;
-  return max(-100, (int)(__float_as_uint(m) >> 23) - 126);
-}
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
-// max(|a|, |b|, |c|), NaN if any is
-__device__ __forceinline__ float absmax_nan(float a, float b, float c) {
-  float r;
-  asm("{\n\t.reg .f32 t, u, v;\n\tabs.f32 t, %2;\n\tabs.f32 u, %3;\n\tmax.NaN.f32 v, t, u;\n\tmax.NaN.f32 %0, %1, v;\n\t}"
-      : "=f"(r)
-      : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
-               "tcgen05.wait::ld.sync.aligned;"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-
-// the adjoint's eight worker warps and a ninth that issues the MMAs: an issue occupies its thread for
-// about 100 cycles, and a worker that did it held the others up at the next barrier (2.34 -> 1.80 ms,
-// 320 x 320 x 256, 8 right-hand sides)
-constexpr int kThreads = 288;
-__device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-// a warp's shared-memory writes, visible to the MMAs of whoever waits on `bar`
-__device__ __forceinline__ void warp_publish(uint64_t* bar) {
-  tc::fence_proxy_async();
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive1(bar);
-}
-
-__host__ __device__ inline uint32_t tmem_cols(uint32_t need) {
-  uint32_t c = 32;
-  while (c < need) c *= 2;
-  return c;
-}
 
 // ---------------------------------------------------------------------------------------------
 // forward

@@ -155,7 +155,7 @@ template <int P>
 __global__ void __launch_bounds__(128) joint_core_adj_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ K,
                                                              const float2* __restrict__ F, int p, int chunk,
                                                              float2* __restrict__ part) {
-  constexpr int TS = P >= 16 ? 2 : 1, SG = P / TS, KS = 8 / SG;
+  constexpr int TS = 1, SG = P, KS = 8 / SG;
   __shared__ __align__(16) float2 ks[kCc][kCj + 2];
   __shared__ __align__(16) float2 fs[kCc][P];
   __shared__ float2 red[KS > 1 ? KS : 1][KS > 1 ? kCj : 1][KS > 1 ? P : 1];
@@ -269,17 +269,22 @@ __global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict
 
 constexpr int kPassRhs = 64;  // right-hand sides per round of the workspaces
 
-int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : p <= 4 ? 4 : p <= 8 ? 8 : 16; }
+// from this many right-hand sides of a round on, the column sums run on the tensor cores
+constexpr int kTcRhs = 5;
+
+int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : 4; }  // FP32 column sums
 
 template <int P>
 void launch_core_fwd(const JointGeo& G, const float2* K, const float2* X, int64_t ldx, int p, int JS, float2* T, int* err,
                      int csmax, cudaStream_t st) {
   joint_core_fwd_kernel<P><<<dim3(ceil_div(csmax, 256), JS, G.q * ceil_div(p, P)), 128, 0, st>>>(G, K, X, ldx, p, JS, T, err);
+  count_launch();
 }
 template <int P>
 void launch_core_adj(const JointGeo& G, const float2* K, const float2* F, int p, int chunk, int splits, float2* part,
                      cudaStream_t st) {
   joint_core_adj_kernel<P><<<dim3(ceil_div(G.M, kCj), splits, ceil_div(p, P)), 128, 0, st>>>(G, K, F, p, chunk, part);
+  count_launch();
 }
 
 // work split of one round of ps <= kPassRhs right-hand sides
@@ -292,6 +297,7 @@ struct FwdPlan {
     P = rhs_per_cta(ps);
     // enough CTAs for 6 per SM, at least 32 columns a slice
     JS = std::max(1, std::min({16, G.M / 32, ceil_div(6 * sm_count(), cblocks * ceil_div(ps, P))}));
+    if (ps >= kTcRhs) JS = 1;
     telems = (int64_t)JS * ps * G.Ct;
     qelems = (int64_t)ps * G.Qt;
   }
@@ -307,6 +313,7 @@ struct AdjPlan {
     chunk = (int)std::max<int64_t>(256, (G.Ct / want + kCc - 1) / kCc * kCc);
     splits = 0;
     for (int k = 0; k < G.q; ++k) splits += ceil_div(G.Cs[k], chunk);
+    if (ps >= kTcRhs) joint_core_split(G, ps, &chunk, &splits);
     felems = (int64_t)ps * G.Ct;
     qelems = (int64_t)ps * G.Qt;
     pelems = (int64_t)splits * ps * G.M;
@@ -341,15 +348,14 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
     float2* T = (float2*)h.work_joint.ptr;
     float2* Q = T + pl.telems;
     const float2* Xs = X + ldx * s0;
-    switch (pl.P) {
+    switch (ps >= kTcRhs ? 0 : pl.P) {
+      case 0: ZBC_TRY(joint_core_fwd(jc, Xs, ldx, ps, T, err, st)); break;
       case 1: launch_core_fwd<1>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
       case 2: launch_core_fwd<2>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
-      case 4: launch_core_fwd<4>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
-      case 8: launch_core_fwd<8>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
-      default: launch_core_fwd<16>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
+      default: launch_core_fwd<4>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
     }
     joint_mode3_fwd_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(G.n3, kZ), ps * G.q), 128, 0, st>>>(G, jc.basis, T, ps, JS, Q);
-    count_launch(2);
+    count_launch();
     ZBC_TRY(joint_planes_fwd(jc, Q, ps, Y + ldy * s0, ldy, err, st));
   }
   return ZBC_OK;
@@ -375,15 +381,14 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
     const float2* Ps = Phi + ldphi * s0;
     ZBC_TRY(joint_planes_adj(jc, Ps, ldphi, ps, Q, err, st));
     joint_mode3_adj_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(r3, 8), ps * G.q), 128, 0, st>>>(G, jc.basis, Q, F);
-    switch (pl.P) {
+    switch (ps >= kTcRhs ? 0 : pl.P) {
+      case 0: ZBC_TRY(joint_core_adj(jc, F, ps, part, err, st)); break;
       case 1: launch_core_adj<1>(G, jc.K, F, ps, chunk, splits, part, st); break;
       case 2: launch_core_adj<2>(G, jc.K, F, ps, chunk, splits, part, st); break;
-      case 4: launch_core_adj<4>(G, jc.K, F, ps, chunk, splits, part, st); break;
-      case 8: launch_core_adj<8>(G, jc.K, F, ps, chunk, splits, part, st); break;
-      default: launch_core_adj<16>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      default: launch_core_adj<4>(G, jc.K, F, ps, chunk, splits, part, st); break;
     }
     joint_sum_kernel<<<dim3(ceil_div(G.M, 32), ps), 256, 0, st>>>(part, G.M, ps, splits, out + ldo * s0, ldo);
-    count_launch(3);
+    count_launch(2);
     ZBC_TRY_CUDA(cudaGetLastError());
   }
   return ZBC_OK;
