@@ -15,12 +15,20 @@
 
 namespace zbc {
 
-void joint_release(JointCache* c) {
-  if (!c) return;
+static void free_operands(JointCache* c) {
   if (c->basis) cudaFree(c->basis);
   if (c->K) cudaFree(c->K);
   if (c->bop) cudaFree(c->bop);
   if (c->kscale) cudaFree(c->kscale);
+  c->basis = c->K = nullptr;
+  c->bop = nullptr;
+  c->kscale = nullptr;
+  c->bytes = 0;
+}
+
+void joint_release(JointCache* c) {
+  if (!c) return;
+  free_operands(c);
   delete c;
 }
 int64_t joint_bytes(const JointCache* c) { return c ? c->bytes : 0; }
@@ -280,10 +288,7 @@ int cuda_status(cudaError_t e, const char* what) {
 
 }  // namespace
 
-int build_joint(Handle& h, cudaStream_t st) {
-  if (h.joint) return ZBC_OK;
-  auto* jc = new JointCache();
-  h.joint = jc;  // kept also when unusable, so that the search is not repeated
+static int build(Handle& h, JointCache* jc, cudaStream_t st) {
   const int q = h.q, T = (int)h.desc.size(), n[3] = {h.n1, h.n2, h.n3}, NP = 3 * q;
   JointGeo& g = jc->geo;
   g.n1 = h.n1;
@@ -461,6 +466,14 @@ int build_joint(Handle& h, cudaStream_t st) {
   if (e != cudaSuccess) return cuda_status(e, "reduced cores");
   jc->usable = true;
   return ZBC_OK;
+}
+
+int build_joint(Handle& h, cudaStream_t st) {
+  if (h.joint) return ZBC_OK;
+  h.joint = new JointCache();  // kept also when unusable, so that the search is not repeated
+  const int s = build(h, h.joint, st);
+  if (!h.joint->usable) free_operands(h.joint);
+  return s;
 }
 
 }  // namespace zbc

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(288, 2)
     __syncwarp();
   } else {
     const int q4 = warp & 3, half = warp >> 2;           // accumulator rows and columns
-    const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // adjoint loader: rows row0 + 32 u, entries c8 + 8 w
+    const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // adjoint loader: rows row0 + 32 u, entries entry_of(c8, w)
     bool bad = false;
     float2 x[16], b[I];
     // position of the chunk that fetch() reads next: component, first row of the tile (forward) or first
@@ -120,14 +120,18 @@ __global__ void __launch_bounds__(288, 2)
           b[i] = j < G.M && s < p ? __ldg(R + j + ldr * s) : make_float2(0.f, 0.f);
         }
       } else {
-        const int c = fpos + c8;
+        const int c = fpos + 2 * c8;  // rows of K are padded to 4 entries: pairs never cross their end
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int j = blockIdx.y * kRows + row0 + 32 * u;
           const float2* g = K + G.koff[fk] + (int64_t)j * G.Cs[fk] + c;
 #pragma unroll
-          for (int w = 0; w < 4; ++w)
-            x[4 * u + w] = j < G.M && c + 8 * w < G.Cs[fk] ? __ldcs(g + 8 * w) : make_float2(0.f, 0.f);
+          for (int w = 0; w < 2; ++w) {
+            const float4 v = j < G.M && c + 16 * w < G.Cs[fk] ? __ldcs((const float4*)(g + 16 * w))
+                                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[4 * u + 2 * w] = make_float2(v.x, v.y);
+            x[4 * u + 2 * w + 1] = make_float2(v.z, v.w);
+          }
         }
 #pragma unroll
         for (int i = 0; i < I; ++i) {
@@ -220,7 +224,7 @@ __global__ void __launch_bounds__(288, 2)
           }
         }
         // the right-hand sides' rows (two a right-hand side): pair `lane` of the chunk in the rows' order
-        const uint32_t kc = FWD ? lane / 4 : lane % 8, word = FWD ? lane % 4 : lane / 8;
+        const uint32_t kc = FWD ? lane / 4 : lane % 16 / 2, word = FWD ? lane % 4 : lane % 2 + lane / 16 * 2;
         float xs = 1.f;  // 2^(e_j - e)
         if (FWD) xs = __ldg(ks + (G.M + kSum - 1) / kSum * kSum + ch * kSum + lane);
 #pragma unroll

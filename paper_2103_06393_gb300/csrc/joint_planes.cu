@@ -23,212 +23,248 @@ namespace {
 // ---------------------------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------------------------
-// A CTA keeps the hi / lo rows of B1 for up to `nb` blocks of 128 i1 and B2's rows of one tile of NT
-// i2 in shared memory and walks the planes (s, i3) of its component.  Per plane: Q[i3] to shared
-// memory (loaded into registers during the plane before), S (R1 x NT) in FP32, its hi / lo rows to
-// shared memory, one MMA chain per i1 block (M = 128, N = 2 NT, K = 2 R1p) into alternating
-// accumulators, the epilogues (tensor memory to Y, 32 consecutive i1 per store) overlapping the next
-// block's MMAs.  Two CTAs share an SM, so one's stores overlap the other's S.  NT = 64 up to
-// R = 32, else 32 (shared memory).  K-major core-matrix layout without swizzle, KB = R1p / 4 chunks of
-// 16 bytes a row; rows of B1 past n1 are not stored: the MMAs read what follows, into rows of the
-// accumulator that nothing reads.  S is scaled by the bound
-// |S| <= sqrt(2 R2) max |Re Q|, |Im Q| < 12 max.
-constexpr int kQRegs = kJointRmax * kJointRmax / 256;
+// A CTA takes a tile of `T2` i2 (at most 112) and up to `nb` blocks of 128 i1, keeps the hi / lo rows of
+// B2 and B1 for them in shared memory and walks the planes (s, i3) of its component.  Per plane:
+//   workers     Q[i3] (loaded a plane ahead) scaled by its largest entry, split: rows of one MMA operand
+//   MMA 1       D1[i2, (Re, Im) x] = B2 Q^T           M = 128, N = 2 R1p, K = 2 R2p
+//   workers     D1 -> S's rows for the second MMA (a fixed shift: |S| < 12 max |Q|)
+//   MMA 2       D2[i1, (Re, Im) i2] = B1 S            M = 128, N = 2 T2, K = 2 R1p, per i1 block, two
+//                                                     accumulators in turn
+//   workers     D2 -> Y, 32 consecutive i1 per store
+// The ninth warp issues all MMAs.  Where two copies of S fit (ns = 2) the workers make plane t + 1's S
+// before they store plane t, so that the MMAs of one plane overlap the stores of the other; else only
+// the next plane's Q is split ahead.  S on the CUDA cores (R1 R2 multiply-adds per i2 and plane) took two thirds of the
+// issue slots: 0.48 / 1.22 / 1.03 ms for 96^3/16, 160 x 160 x 128/32 and 320 x 320 x 256/8 planes.
+// K-major core-matrix layout without swizzle, KB chunks of 16 bytes a row; rows of B1 past n1 are not
+// stored: MMA 2 reads what follows, into accumulator rows that nothing reads.
+struct FwdShape {
+  int R1p, R2p, T2, nt2, nb, gy, ns;
+  __host__ __device__ size_t b1_bytes(int n1) const { return (size_t)8 * R1p * min(nb * 128, (n1 + 7) / 8 * 8); }
+  __host__ __device__ size_t s_bytes() const { return (size_t)16 * R1p * T2; }
+  __host__ __device__ size_t b2_bytes() const { return (size_t)1024 * R2p; }
+  __host__ __device__ size_t q_bytes() const { return (size_t)16 * R1p * R2p; }
+  __host__ __device__ size_t bytes(int n1) const { return b1_bytes(n1) + ns * s_bytes() + b2_bytes() + q_bytes(); }
+};
+// 16 worker warps: with one CTA an SM, 8 of them left the schedulers two thirds idle
+constexpr int kFwdWorkers = 512, kFwdThreads = kFwdWorkers + 32, kFwdGroups = kFwdWorkers / 128;
+constexpr int kQRegs = kJointRmax * kJointRmax / kFwdWorkers;
 
-template <int NT>
-__global__ void __launch_bounds__(256, 2)
-    joint_planes_fwd_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ basis,
-                            const float2* __restrict__ Q, int R1p, int R2p, int nb, int p, float2* __restrict__ Y,
+__global__ void __launch_bounds__(kFwdThreads, 1)
+    joint_planes_fwd_kernel(const __grid_constant__ JointGeo G, const __grid_constant__ FwdShape F,
+                            const float2* __restrict__ basis, const float2* __restrict__ Q, int p, float2* __restrict__ Y,
                             int64_t ldy, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem_f[];
-  unsigned char* smem = smem_f;
-  __shared__ __align__(8) uint64_t done[2];
+  __shared__ __align__(8) uint64_t done[2], dfree[2], sready, qready, s1done;
   __shared__ uint32_t tmem_base;
-  __shared__ float wmax[8];
-  __shared__ int abort_flag;
-  constexpr int GR = 256 / NT;  // groups of 4-row chunks of S
-  constexpr int QR = NT == 64 ? kQRegs / 4 : kQRegs;  // entries of Q per thread
-  const int k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1], RR = R1 * R2, KB = R1p / 4;
+  __shared__ float wmax[2][kFwdWorkers / 32];
+  const int k = blockIdx.z, R1 = G.R[k][0], R2 = G.R[k][1], RR = R1 * R2;
+  const int R1p = F.R1p, KB = R1p / 4, KB1 = F.R2p / 4, T2 = F.T2;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nt2 = (G.n2 + NT - 1) / NT, i20 = (int)(blockIdx.y % nt2) * NT;
-  const int row0 = (int)(blockIdx.y / nt2) * nb * 128, rows = min(nb * 128, G.n1 - row0), nblk = (rows + 127) / 128;
-  const uint32_t bbytes = 2u * NT * KB * 16u;  // one term of S
-  unsigned char* sb = smem;                    // S before B1: the MMAs may read past B1's last rows
-  float2* qs = (float2*)(sb + 2 * bbytes);     // [R2][R1p]
-  float2* b2 = qs + R2p * R1p;                 // [R2][NT]
-  unsigned char* sa = (unsigned char*)(b2 + R2p * NT);
-  const uint32_t ablk = 128u * KB * 16u;       // one term of a full block; the last block is shorter
+  const int i20 = (int)(blockIdx.y % F.nt2) * T2, row0 = (int)(blockIdx.y / F.nt2) * F.nb * 128;
+  const int rows = min(F.nb * 128, G.n1 - row0), nblk = (rows + 127) / 128;
+  unsigned char* sa = smem_f;                    // B1: [block][term][rows]
+  unsigned char* ss = sa + F.b1_bytes(G.n1);     // S: [ns][term][2 T2 rows]
+  unsigned char* sb2 = ss + F.ns * F.s_bytes();  // B2: [term][128 rows]
+  unsigned char* sq = sb2 + F.b2_bytes();        // Q: [term][2 R1p rows]
+  const uint32_t ablk = 128u * KB * 16u, sterm = 2u * T2 * KB * 16u, b2term = 128u * KB1 * 16u, qterm = 2u * R1p * KB1 * 16u;
   const uint32_t alast = (uint32_t)((rows - (nblk - 1) * 128 + 7) / 8) * 8u * KB * 16u;
-  const uint32_t ncols = tmem_cols(nblk > 1 ? 4 * NT : 2 * NT);
+  constexpr uint32_t ncols = 512;
+  const uint32_t d2 = 2 * R1p;                   // D1 in columns 0 .. 2 R1p - 1, two D2 of 2 T2 columns after it
+  const int lag = F.ns - 1;
   if (tid == 0) {
-    tc::mbar_init(&done[0], 1);
-    tc::mbar_init(&done[1], 1);
-    abort_flag = 0;
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&done[i], 1);
+      tc::mbar_init(&dfree[i], kFwdWorkers / 32);
+    }
+    tc::mbar_init(&sready, kFwdWorkers / 32);
+    tc::mbar_init(&qready, kFwdWorkers / 32);
+    tc::mbar_init(&s1done, 1);
   }
   if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
-  const int rows8 = (rows + 7) / 8 * 8;
-  for (int e = tid; e < rows8 * KB; e += 256) {
-    const int rr = e % rows8, kc = e / rows8, b = rr / 128, r = rr % 128, i1 = row0 + rr;
+  auto rows_of = [&](unsigned char* dst, uint32_t lo, int r, int kc, int kb, const float2* b, int n, int i, bool live, int R) {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int x = 4 * kc + u;
-      const float2 v = x < R1 && i1 < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i1] : make_float2(0.f, 0.f);
+      const float2 v = live && 4 * kc + u < R ? b[(int64_t)(4 * kc + u) * n + i] : make_float2(0.f, 0.f);
       split2(v.x * pow2f(kBasisShift), v.y * pow2f(kBasisShift), h[u], l[u]);
     }
-    unsigned char* d = sa + (size_t)b * 2 * ablk + tc::core_off(r, kc, KB);
+    unsigned char* d = dst + tc::core_off(r, kc, kb);
     *(uint4*)d = make_uint4(h[0], h[1], h[2], h[3]);
-    *(uint4*)(d + (b == nblk - 1 ? alast : ablk)) = make_uint4(l[0], l[1], l[2], l[3]);
-  }
-  for (int e = tid; e < R2 * R1p; e += 256) qs[e] = make_float2(0.f, 0.f);  // the pad stays zero
-  for (int e = tid; e < R2 * NT; e += 256) {
-    const int i2 = i20 + e % NT;
-    b2[e] = i2 < G.n2 ? basis[G.boff[k][1] + (int64_t)(e / NT) * G.n2 + i2] : make_float2(0.f, 0.f);
-  }
-  const int planes = p * G.n3;
-  const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
-  const float2* Qk = Q + G.qoff[k];
-  float2 qr[QR];
-  auto fetch_q = [&](int pl) {
-    const float2* Qp = Qk + (int64_t)(pl / G.n3) * G.Qt + (int64_t)(pl % G.n3) * RR;
-#pragma unroll
-    for (int u = 0; u < QR; ++u)
-      if (tid + 256 * u < RR) qr[u] = __ldg(Qp + tid + 256 * u);
+    *(uint4*)(d + lo) = make_uint4(l[0], l[1], l[2], l[3]);
   };
-  int qdst[QR];
-#pragma unroll
-  for (int u = 0; u < QR; ++u) qdst[u] = (tid + 256 * u) / R1 * R1p + (tid + 256 * u) % R1;
-  fetch_q(blockIdx.x);  // grid x <= planes
+  const int rows8 = (rows + 7) / 8 * 8;
+  for (int e = tid; e < rows8 * KB; e += kFwdThreads) {
+    const int rr = e % rows8, b = rr / 128;
+    rows_of(sa + (size_t)b * 2 * ablk, b == nblk - 1 ? alast : ablk, rr % 128, e / rows8, KB, basis + G.boff[k][0], G.n1,
+            row0 + rr, row0 + rr < G.n1, R1);
+  }
+  for (int e = tid; e < 128 * KB1; e += kFwdThreads) {
+    const int r = e % 128;
+    rows_of(sb2, b2term, r, e / 128, KB1, basis + G.boff[k][1], G.n2, i20 + r, r < T2 && i20 + r < G.n2, R2);
+  }
+  for (uint32_t e = tid; e < qterm / 8; e += kFwdThreads) ((uint4*)sq)[e] = make_uint4(0, 0, 0, 0);  // the pad stays zero
+  tc::fence_proxy_async();
   __syncthreads();
   const uint32_t tmem = tmem_base;
-  const int il = tid % NT, grp = tid / NT, q4 = warp & 3, half = warp >> 2;
-  const bool full2 = i20 + NT <= G.n2, has0 = grp < KB, has1 = grp + GR < KB;
-  uint32_t ph[2] = {0, 0};  // parity of the next completion of each accumulator
-  bool ok = true;
-  for (int pl = blockIdx.x; pl < planes; pl += gridDim.x) {
-    float m = 0.f;
-#pragma unroll
-    for (int u = 0; u < QR; ++u)
-      if (tid + 256 * u < RR) {
-        qs[qdst[u]] = qr[u];
-        m = absmax_nan(m, qr[u].x, qr[u].y);
-      }
-    for (int o = 16; o > 0; o >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) wmax[warp] = m;
-    __syncthreads();
-    if (abort_flag) break;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) m = max_nan(m, wmax[w]);
-    if (pl + gridDim.x < planes) fetch_q(pl + gridDim.x);
-    float2 a[2][4];
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a[c][u] = make_float2(0.f, 0.f);
-    if (has1) {
-#pragma unroll 2
-      for (int y = 0; y < R2; ++y) {
-        const float2 b = b2[y * NT + il];
-        const float4* q = (const float4*)(qs + y * R1p);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const float4 v0 = q[2 * (grp + c * GR)], v1 = q[2 * (grp + c * GR) + 1];
-          a[c][0] = cfma(make_float2(v0.x, v0.y), b, a[c][0]);
-          a[c][1] = cfma(make_float2(v0.z, v0.w), b, a[c][1]);
-          a[c][2] = cfma(make_float2(v1.x, v1.y), b, a[c][2]);
-          a[c][3] = cfma(make_float2(v1.z, v1.w), b, a[c][3]);
-        }
-      }
-    } else if (has0) {
-#pragma unroll 2
-      for (int y = 0; y < R2; ++y) {
-        const float2 b = b2[y * NT + il];
-        const float4* q = (const float4*)(qs + y * R1p);
-        const float4 v0 = q[2 * grp], v1 = q[2 * grp + 1];
-        a[0][0] = cfma(make_float2(v0.x, v0.y), b, a[0][0]);
-        a[0][1] = cfma(make_float2(v0.z, v0.w), b, a[0][1]);
-        a[0][2] = cfma(make_float2(v1.x, v1.y), b, a[0][2]);
-        a[0][3] = cfma(make_float2(v1.z, v1.w), b, a[0][3]);
-      }
+  const int planes = p * G.n3;
+  const int mine = (planes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;  // grid x <= planes
+  bool ok = true;  // false after a wait gave up: no further waits, the barriers are still passed
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (ok && !tc::mbar_wait_idle(bar, parity)) {
+      ok = false;
+      atomicOr(err, kErrTimeout);
     }
-    const int e = exp_of(m) - 1;  // |S| < 12 max |Q| < 2^(e + 5): scaled below 2^(kDataShift + 5) = 2^15
-    const float sc = pow2f(kDataShift - e);
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int kc = grp + c * GR;
-      if (kc < KB) {
-        uint32_t hr[4], lr[4], hi[4], li[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          // rows (Re, -Im) and (Im, Re) of the same words: swap the halves, flip the sign of Im
-          split2(a[c][u].x * sc, a[c][u].y * sc, hr[u], lr[u]);
-          hi[u] = __byte_perm(hr[u], 0, 0x1032);
-          li[u] = __byte_perm(lr[u], 0, 0x1032);
-          hr[u] ^= 0x80000000u;
-          lr[u] ^= 0x80000000u;
-        }
-        unsigned char* d0 = sb + tc::core_off(2 * il, kc, KB);
-        unsigned char* d1 = sb + tc::core_off(2 * il + 1, kc, KB);
-        *(uint4*)d0 = make_uint4(hr[0], hr[1], hr[2], hr[3]);
-        *(uint4*)(d0 + bbytes) = make_uint4(lr[0], lr[1], lr[2], lr[3]);
-        *(uint4*)d1 = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *(uint4*)(d1 + bbytes) = make_uint4(li[0], li[1], li[2], li[3]);
-      }
-    }
-    tc::fence_proxy_async();
-    __syncthreads();
-    const float us = pow2f(e - kDataShift - kBasisShift);
-    const int s = pl / G.n3, i3 = pl - s * G.n3;
-    float2* Yp = Y + ldy * s + (int64_t)k * nv + (int64_t)G.n1 * (i20 + (int64_t)G.n2 * i3) + row0;
-    auto epilogue = [&](int b) {
-      const int d = b & 1;
-      if (ok && !tc::mbar_wait(&done[d], ph[d])) {
-        ok = false;
-        abort_flag = 1;
-        atomicOr(err, kErrTimeout);
-      }
-      ph[d] ^= 1;
-      tc::fence_after();
-      const int i1 = b * 128 + 32 * q4;
-      if (i1 < rows && ok) {
-        const uint32_t t0 = tmem + (uint32_t)(d * 2 * NT + half * NT) + ((uint32_t)(32 * q4) << 16);
-        const int i2h = half * (NT / 2);
-        float2* y0 = Yp + (int64_t)G.n1 * i2h + i1 + lane;
-        const bool live = i1 + lane < rows;
-#pragma unroll
-        for (int c = 0; c < NT / 16; ++c) {
-          float v[16];
-          tc::tmem_ld16(t0 + 16 * c, v);
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (live && (full2 || i20 + i2h + 8 * c + u < G.n2))
-              __stcs(y0 + (int64_t)G.n1 * (8 * c + u), make_float2(v[2 * u] * us, v[2 * u + 1] * us));
-        }
-      }
-      tc::fence_before();
-    };
-    for (int b = 0; b < nblk; ++b) {
-      if (tid == 0) {
-        tc::fence_after();
-        const uint32_t a0 = tc::smem_u32(sa) + (uint32_t)b * 2 * ablk, a1 = a0 + (b == nblk - 1 ? alast : ablk);
-        const uint32_t b0 = tc::smem_u32(sb), b1 = b0 + bbytes, sbo = KB * 128u;
-        const uint32_t d = tmem + (uint32_t)((b & 1) * 2 * NT), id = tc::instr_desc(128, 2 * NT, 0);
-        for (int ks = 0; ks < KB / 2; ++ks) {
-          const uint64_t ah = tc::smem_desc(a0 + ks * 256u, 128, sbo), al = tc::smem_desc(a1 + ks * 256u, 128, sbo);
-          const uint64_t bh = tc::smem_desc(b0 + ks * 256u, 128, sbo), bl = tc::smem_desc(b1 + ks * 256u, 128, sbo);
+  };
+  if (warp == kFwdWorkers / 32) {
+    if (lane == 0) {
+      const uint32_t b1 = tc::smem_u32(sa), s0 = tc::smem_u32(ss), b2 = tc::smem_u32(sb2), q0 = tc::smem_u32(sq);
+      const uint32_t sbo = KB * 128u, sbo1 = KB1 * 128u;
+      auto chain = [&](uint32_t d, uint32_t a, uint32_t alo, uint32_t b, uint32_t blo, uint32_t st, int steps, uint32_t id) {
+        for (int ks = 0; ks < steps; ++ks) {
+          const uint64_t ah = tc::smem_desc(a + ks * 256u, 128, st), al = tc::smem_desc(a + alo + ks * 256u, 128, st);
+          const uint64_t bh = tc::smem_desc(b + ks * 256u, 128, st), bl = tc::smem_desc(b + blo + ks * 256u, 128, st);
           tc::mma<0>(d, al, bh, id, ks > 0);
           tc::mma<0>(d, ah, bl, id, 1);
           tc::mma<0>(d, ah, bh, id, 1);
         }
-        tc::commit(&done[b & 1]);
-      }
-      if (b > 0) {
-        epilogue(b - 1);
-        __syncthreads();  // accumulator (b - 1) & 1 is free for block b + 1
+      };
+      auto mma1 = [&](int t) {
+        wait(&qready, t & 1);
+        if (!ok) return;
+        tc::fence_after();
+        chain(tmem, b2, b2term, q0, qterm, sbo1, KB1 / 2, tc::instr_desc(128, 2 * R1p, 0));
+        tc::commit(&s1done);
+      };
+      mma1(0);
+      int n = 0;  // accumulators used so far
+      for (int t = 0; t < mine && ok; ++t) {
+        wait(&sready, t & 1);
+        if (lag && t + 1 < mine) mma1(t + 1);
+        for (int b = 0; b < nblk && ok; ++b, ++n) {
+          wait(&dfree[n & 1], ((n >> 1) & 1) ^ 1);  // a fresh barrier's preceding phase counts as complete
+          if (!ok) break;
+          tc::fence_after();
+          chain(tmem + d2 + (uint32_t)((n & 1) * 2 * T2), b1 + (uint32_t)b * 2 * ablk, b == nblk - 1 ? alast : ablk,
+                s0 + (uint32_t)(t & lag) * 2 * sterm, sterm, sbo, KB / 2, tc::instr_desc(128, 2 * T2, 0));
+          tc::commit(&done[n & 1]);
+        }
+        if (!lag && t + 1 < mine) mma1(t + 1);
       }
     }
-    // all threads pass the next plane's two barriers after this before anything is reused
-    epilogue(nblk - 1);
+    __syncwarp();
+  } else {
+    const int q4 = warp & 3, grp = warp >> 2;  // accumulator rows; the groups share its columns
+    const float2* Qk = Q + G.qoff[k];
+    float2 qr[kQRegs];
+    uint32_t qoff[kQRegs];  // of the pair (x, y) in row 2 x; row 2 x + 1 lies 16 bytes further
+#pragma unroll
+    for (int u = 0; u < kQRegs; ++u) {
+      const int x = (tid + kFwdWorkers * u) % R1, y = (tid + kFwdWorkers * u) / R1;
+      qoff[u] = tc::core_off(2 * x, y / 4, KB1) + 4 * (y % 4);
+    }
+    auto fetch_q = [&](int t) {
+      const int pl = (int)blockIdx.x + t * (int)gridDim.x;
+      const float2* Qp = Qk + (int64_t)(pl / G.n3) * G.Qt + (int64_t)(pl % G.n3) * RR;
+#pragma unroll
+      for (int u = 0; u < kQRegs; ++u)
+        if (tid + kFwdWorkers * u < RR) qr[u] = __ldg(Qp + tid + kFwdWorkers * u);
+    };
+    auto split_q = [&](int t) {  // returns the plane's exponent; MMA 1 of the plane before has completed
+      float m = 0.f;
+#pragma unroll
+      for (int u = 0; u < kQRegs; ++u)
+        if (tid + kFwdWorkers * u < RR) m = absmax_nan(m, qr[u].x, qr[u].y);
+      for (int o = 16; o > 0; o >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) wmax[t & 1][warp] = m;
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+#pragma unroll
+      for (int w = 0; w < kFwdWorkers / 32; ++w) m = max_nan(m, wmax[t & 1][w]);
+      const int e = exp_of(m, -117);  // 2^(kDataShift - e) stays finite; Y takes 2^-21 and 2^e in turn
+      const float sc = pow2f(kDataShift - e);
+#pragma unroll
+      for (int u = 0; u < kQRegs; ++u)
+        if (tid + kFwdWorkers * u < RR) {
+          uint32_t h, l;
+          split2(qr[u].x * sc, qr[u].y * sc, h, l);
+          unsigned char* d = sq + qoff[u];  // rows (Re, -Im), (Im, Re)
+          *(uint32_t*)d = h ^ 0x80000000u;
+          *(uint32_t*)(d + qterm) = l ^ 0x80000000u;
+          *(uint32_t*)(d + 16) = __byte_perm(h, 0, 0x1032);
+          *(uint32_t*)(d + qterm + 16) = __byte_perm(l, 0, 0x1032);
+        }
+      warp_publish(&qready);
+      return e;
+    };
+    fetch_q(0);
+    int e = split_q(0), elast = 0;
+    if (mine > 1) fetch_q(1);
+    int n = 0;
+    for (int t = 0; t < mine + lag; ++t) {
+      const int eout = lag ? elast : e;  // of the plane that is stored in this round
+      if (t < mine) {
+        // S's rows 2 i2, 2 i2 + 1 from D1's row i2: D1 = 2^(kDataShift + kBasisShift - e) S, so 2^-9 D1 < 2^15,
+        // and D2 = 2^(21 - e) Y
+        wait(&s1done, t & 1);
+        tc::fence_after();
+        const int r = 32 * q4 + lane;
+        if (32 * q4 < T2) {
+          unsigned char* so = ss + (size_t)(t & lag) * 2 * sterm;
+          for (int c = grp; c < R1p / 4; c += kFwdGroups) {
+            uint32_t v[8], hr[4], lr[4], hi[4], li[4];
+            tmem_ld8(tmem + (uint32_t)(8 * c) + ((uint32_t)(32 * q4) << 16), v);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              split2(__uint_as_float(v[2 * u]) * 0x1p-9f, __uint_as_float(v[2 * u + 1]) * 0x1p-9f, hr[u], lr[u]);
+              hi[u] = __byte_perm(hr[u], 0, 0x1032);
+              li[u] = __byte_perm(lr[u], 0, 0x1032);
+              hr[u] ^= 0x80000000u;
+              lr[u] ^= 0x80000000u;
+            }
+            if (r < T2) {
+              unsigned char* d = so + tc::core_off(2 * r, c, KB);
+              *(uint4*)d = make_uint4(hr[0], hr[1], hr[2], hr[3]);
+              *(uint4*)(d + sterm) = make_uint4(lr[0], lr[1], lr[2], lr[3]);
+              *(uint4*)(d + 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              *(uint4*)(d + sterm + 16) = make_uint4(li[0], li[1], li[2], li[3]);
+            }
+          }
+        }
+        tc::fence_before();
+        warp_publish(&sready);
+        elast = e;
+        if (t + 1 < mine) {
+          e = split_q(t + 1);
+          if (t + 2 < mine) fetch_q(t + 2);
+        }
+      }
+      if (t < lag) continue;
+      const float us = pow2f(eout);
+      const int pl = (int)blockIdx.x + (t - lag) * (int)gridDim.x, s = pl / G.n3, i3 = pl - s * G.n3;
+      float2* Yp = Y + ldy * s + (int64_t)k * ((int64_t)G.n1 * G.n2 * G.n3) +
+                   (int64_t)G.n1 * (i20 + (int64_t)G.n2 * i3) + row0;
+      const int left = min(T2, G.n2 - i20);
+      for (int b = 0; b < nblk; ++b, ++n) {
+        const int d = n & 1, i1 = b * 128 + 32 * q4;
+        wait(&done[d], (n >> 1) & 1);
+        tc::fence_after();
+        if (i1 < rows && ok) {
+          const uint32_t t0 = tmem + d2 + (uint32_t)(d * 2 * T2) + ((uint32_t)(32 * q4) << 16);
+          float2* y0 = Yp + i1 + lane;
+          const bool live = i1 + lane < rows;
+          for (int c = grp; c < T2 / 8; c += kFwdGroups) {
+            float v[16];
+            tc::tmem_ld16(t0 + 16 * c, v);
+            float2* y = y0 + (int64_t)G.n1 * 8 * c;
+#pragma unroll
+            for (int w = 0; w < 8; ++w, y += G.n1)
+              if (live && 8 * c + w < left) __stcs(y, make_float2(v[2 * w] * 0x1p-21f * us, v[2 * w + 1] * 0x1p-21f * us));
+          }
+        }
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive1(&dfree[d]);
+      }
+    }
   }
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
@@ -253,7 +289,9 @@ inline size_t planes_adj_smem(int NC) {
   return 4 * (size_t)kATerm + 2 * 2 * 2 * (size_t)NC * 128 + sizeof(float2) * kStage2 * ((NC + 15) / 16 * 16);
 }
 
-template <int I>  // NC = 8 I >= R1, R2 of every component
+// NC = 8 I >= R1, R2 of every component.  VEC: Phi's columns start on 16 bytes, and a lane reads two
+// entries at a time (half the loads; the load unit was the busiest one).
+template <int I, bool VEC>
 __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     joint_planes_adj_kernel(const __grid_constant__ JointGeo G, const unsigned char* __restrict__ bop,
                             const float2* __restrict__ b2t, const float2* __restrict__ Phi, int64_t ldphi, int p,
@@ -332,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     __syncwarp();
   } else {
     const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
-    const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // loader: rows row0 + 32 u, i1 = c8 + 8 w
+    const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // loader: rows row0 + 32 u, i1 = entry_of(c8, w)
     const int q4 = warp & 3, half = warp >> 2;            // accumulator rows and columns
     const int tx = tid % 16, ty = tid / 16;
     bool bad = false;
@@ -342,17 +380,29 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     auto locate = [&](int plane, int t2) {
       const int k = plane % G.q, i3 = plane / G.q % G.n3, s = plane / G.q / G.n3;
       rows = min(kTile2, G.n2 - t2 * kTile2);
-      src = Phi + ldphi * s + (int64_t)k * nv + (int64_t)G.n1 * ((int64_t)G.n2 * i3 + t2 * kTile2 + row0) + c8;
+      src = Phi + ldphi * s + (int64_t)k * nv + (int64_t)G.n1 * ((int64_t)G.n2 * i3 + t2 * kTile2 + row0) + 2 * c8;
     };
     float2 x[4][4];
     auto fetch = [&](int ch) {
-      const int left = G.n1 - ch * kChunk1 - c8;
+      const int left = G.n1 - ch * kChunk1 - 2 * c8;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float2* g = src + (int64_t)G.n1 * (32 * u) + ch * kChunk1;
         const bool live = row0 + 32 * u < rows;
+        if (VEC) {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) x[u][w] = live && 8 * w < left ? __ldcs(g + 8 * w) : make_float2(0.f, 0.f);
+          for (int w = 0; w < 2; ++w) {
+            const float4 v = live && 16 * w < left ? __ldcs((const float4*)(g + 16 * w)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[u][2 * w] = make_float2(v.x, v.y);
+            x[u][2 * w + 1] = make_float2(v.z, v.w);
+          }
+        } else {
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            const int o = (w & 1) + 16 * (w >> 1);
+            x[u][w] = live && o < left ? __ldcs(g + o) : make_float2(0.f, 0.f);
+          }
+        }
       }
     };
     float2 qa[RC][RC];
@@ -471,8 +521,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
 }
 
 // B1's rows of the adjoint: per component and chunk of 32 i1, [term][2 x + e][64 fp16], 128-byte
-// swizzled, the 16-byte chunk c holding i1 = c, c + 8, c + 16, c + 24 (the order in which 8 lanes read
-// Phi without gaps); one thread per (row pair, 16-byte chunk)
+// swizzled, the 16-byte chunk c holding i1 = entry_of(c, 0 .. 3); one thread per (row pair, 16-byte chunk)
 __global__ void __launch_bounds__(256) split_basis_kernel(const __grid_constant__ JointGeo G,
                                                           const float2* __restrict__ basis, int NC, int nch,
                                                           unsigned char* __restrict__ out) {
@@ -481,7 +530,7 @@ __global__ void __launch_bounds__(256) split_basis_kernel(const __grid_constant_
   if (ch >= nch) return;
   uint32_t h0[4], l0[4], h1[4], l1[4];
   for (int w = 0; w < 4; ++w) {
-    const int i1 = ch * kChunk1 + c8 + 8 * w;
+    const int i1 = ch * kChunk1 + entry_of(c8, w);
     const float2 v = x < G.R[k][0] && i1 < G.n1 ? basis[G.boff[k][0] + (int64_t)x * G.n1 + i1] : make_float2(0.f, 0.f);
     const float re = v.x * pow2f(kBasisShift), im = v.y * pow2f(kBasisShift);
     split2(re, im, h0[w], l0[w]);
@@ -505,29 +554,6 @@ size_t bop_bytes(const JointGeo& G) { return (size_t)G.q * ceil_div(G.n1, kChunk
 int b2t_rows(const JointGeo& G) { return ceil_div(G.n2, kTile2) * kTile2; }
 int b2t_cols(const JointGeo& G) { return ceil_div(adj_rows(G), 16) * 16; }
 
-template <int NT>
-int launch_planes_fwd(const JointGeo& G, const float2* basis, const float2* Q, int p, float2* Y, int64_t ldy, int* err,
-                      cudaStream_t st) {
-  const int R1p = ceil_div(max_r(G, 0), 8) * 8, R2p = ceil_div(max_r(G, 1), 2) * 2, nblk = ceil_div(G.n1, 128);
-  const size_t arow = (size_t)8 * R1p;  // bytes of one row of B1, both terms
-  const size_t rest = (size_t)16 * NT * R1p + sizeof(float2) * R2p * (R1p + NT);
-  // two CTAs an SM while at least one i1 block of B1 fits beside the rest; the last block's MMAs read
-  // up to 128 rows of one term past the rows that are stored
-  constexpr size_t kLimit = 115456;  // (228 KB / 2 - 1 KB reserved), less the static variables
-  const size_t over = 64 * (size_t)R1p * 8;
-  auto bytes = [&](int nb) { return rest + over + std::min(nb * 128, ceil_div(G.n1, 8) * 8) * arow; };
-  int nb = nblk;
-  while (nb > 1 && bytes(nb) > kLimit) --nb;
-  const size_t sm = bytes(nb);
-  ZBC_TRY(set_smem_limit<joint_planes_fwd_kernel<NT>>(200 * 1024));
-  const int gy = ceil_div(nblk, nb) * ceil_div(G.n2, NT), per_sm = sm <= kLimit ? 2 : 1;
-  const int walkers = std::min(p * G.n3, std::max(1, per_sm * sm_count() / (gy * G.q)));
-  joint_planes_fwd_kernel<NT><<<dim3(walkers, gy, G.q), 256, sm, st>>>(G, basis, Q, R1p, R2p, nb, p, Y, ldy, err);
-  count_launch();
-  ZBC_TRY_CUDA(cudaGetLastError());
-  return ZBC_OK;
-}
-
 // B2 by i2: per component [n2 rounded up to tiles][R2p], zeros past n2 and R2
 __global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_constant__ JointGeo G,
                                                               const float2* __restrict__ basis, int rows, int R2p,
@@ -538,39 +564,71 @@ __global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_const
       i2 < G.n2 && y < G.R[k][1] ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i2] : make_float2(0.f, 0.f);
 }
 
-template <int I>
+template <int I, bool VEC>
 int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
                       int* err, cudaStream_t st) {
   const float2* b2t = (const float2*)(bop + bop_bytes(G));
-  ZBC_TRY(set_smem_limit<joint_planes_adj_kernel<I>>((int)planes_adj_smem(8 * I)));
+  ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC>>((int)planes_adj_smem(8 * I))));
   const size_t sm = planes_adj_smem(8 * I);
   const int64_t planes = (int64_t)G.n3 * p * G.q;
   const int grid = (int)std::min<int64_t>(planes, (sm <= 112 * 1024 ? 2 : 1) * sm_count());
-  joint_planes_adj_kernel<I><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err);
+  joint_planes_adj_kernel<I, VEC><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err);
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
 }
 
+template <int I>
+int planes_adj_vec(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
+                   int* err, cudaStream_t st) {
+  // every column of every plane on 16 bytes, and no pair of entries across the end of one
+  if (G.n1 % 2 == 0 && (p == 1 || ldphi % 2 == 0) && (uintptr_t)Phi % 16 == 0)
+    return launch_planes_adj<I, true>(G, bop, Phi, ldphi, p, Q, err, st);
+  return launch_planes_adj<I, false>(G, bop, Phi, ldphi, p, Q, err, st);
+}
+
 }  // namespace
 
 int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st) {
-  if (std::max(max_r(jc.geo, 0), max_r(jc.geo, 1)) <= 32) return launch_planes_fwd<64>(jc.geo, jc.basis, Q, p, Y, ldy, err, st);
-  return launch_planes_fwd<32>(jc.geo, jc.basis, Q, p, Y, ldy, err, st);
+  const JointGeo& G = jc.geo;
+  constexpr size_t kLimit = 224 * 1024;
+  // balanced tiles of i2 that leave tensor memory for D1 and two D2; where the operands do not fit
+  // shared memory together, one copy of S, then fewer i1 blocks, then smaller tiles
+  FwdShape F;
+  F.R1p = ceil_div(max_r(G, 0), 8) * 8;
+  F.R2p = ceil_div(max_r(G, 1), 8) * 8;
+  const int nblk = ceil_div(G.n1, 128), t2max = (512 - 2 * F.R1p) / 4 / 16 * 16;
+  for (F.nt2 = ceil_div(G.n2, t2max);; ++F.nt2) {
+    F.T2 = ceil_div(ceil_div(G.n2, F.nt2), 16) * 16;
+    F.nb = nblk;
+    F.ns = 2;
+    if (F.bytes(G.n1) > kLimit) F.ns = 1;
+    while (F.nb > 1 && F.bytes(G.n1) > kLimit) --F.nb;
+    if (F.bytes(G.n1) <= kLimit) break;  // 16 i2, one block, one S: at most 213 KB
+  }
+  F.nt2 = ceil_div(G.n2, F.T2);
+  F.gy = ceil_div(nblk, F.nb);
+  ZBC_TRY(set_smem_limit<joint_planes_fwd_kernel>((int)kLimit));
+  const int walkers = std::min(p * G.n3, std::max(1, sm_count() / (F.gy * F.nt2 * G.q)));
+  joint_planes_fwd_kernel<<<dim3(walkers, F.gy * F.nt2, G.q), kFwdThreads, F.bytes(G.n1), st>>>(G, F, jc.basis, Q, p, Y, ldy,
+                                                                                            err);
+  count_launch();
+  ZBC_TRY_CUDA(cudaGetLastError());
+  return ZBC_OK;
 }
 
 int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
                      cudaStream_t st) {
   const JointGeo& G = jc.geo;
   switch (adj_rows(G) / 8) {
-    case 1: return launch_planes_adj<1>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 2: return launch_planes_adj<2>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 3: return launch_planes_adj<3>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 4: return launch_planes_adj<4>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 5: return launch_planes_adj<5>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 6: return launch_planes_adj<6>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 7: return launch_planes_adj<7>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    default: return launch_planes_adj<8>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 1: return planes_adj_vec<1>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 2: return planes_adj_vec<2>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 3: return planes_adj_vec<3>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 4: return planes_adj_vec<4>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 5: return planes_adj_vec<5>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 6: return planes_adj_vec<6>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 7: return planes_adj_vec<7>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    default: return planes_adj_vec<8>(G, jc.bop, Phi, ldphi, p, Q, err, st);
   }
 }
 

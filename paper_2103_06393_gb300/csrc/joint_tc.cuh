@@ -22,13 +22,16 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t&
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// e with m < 2^e, at least -100 so that 2^(kDataShift - e) and its inverse are normal floats (0 for
-// zero and for values that are not finite, which go through unscaled)
-__device__ __forceinline__ int exp_of(float m) {
+// e with m < 2^e, at least `least` so that the scales made from it are normal floats (0 for zero and for
+// values that are not finite, which go through unscaled)
+__device__ __forceinline__ int exp_of(float m, int least = -106) {
   if (!(m > 0.f) || !(m < INFINITY)) return 0;
-  return max(-100, (int)(__float_as_uint(m) >> 23) - 126);
+  return max(least, (int)(__float_as_uint(m) >> 23) - 126);
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+// order of a chunk's 32 summed entries in a 128-byte row: entry of word w of the 16-byte chunk c, so
+// that lane c's entries are two adjacent pairs and 8 lanes read 128 bytes without a gap
+__host__ __device__ constexpr int entry_of(int c, int w) { return 2 * c + (w & 1) + 16 * (w >> 1); }
 // max(|a|, |b|, |c|), NaN if any is
 __device__ __forceinline__ float absmax_nan(float a, float b, float c) {
   float r;

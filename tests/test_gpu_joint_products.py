@@ -25,9 +25,11 @@ RTOL = 5e-6
 FWD, ADJ = 3, 4  # kernels of one round of the joint form
 
 
-def _tensors(n, m, name="large", tol=1e-6, q=3):
+def _tensors(n, m, name="large", tol=1e-6, q=3, h=None):
     w = inputs.scaled_workload(name, n, m=m)
     g, s = w.grid, w.segments
+    if h is not None:
+        g = inputs.Grid(*n, h)
     Z = greens.assemble_columns(g.shape, g.h, s.centre, s.tangent, s.length, w.freq_hz, np.arange(s.m),
                                 mask_radius=g.mask_radius, mask_box=g.mask_box)
     if q == 12:  # twelve row blocks of the same kind of field
@@ -72,6 +74,39 @@ def test_matches_oracle(n, m, p):
     assert launches == [FWD * rounds, ADJ * rounds]
     assert _rel(Y, products.matvec(tens, g.shape, X)) < RTOL
     assert _rel(Psi, products.rmatvec(tens, g.shape, Phi)) < RTOL
+
+
+@pytest.mark.parametrize("name,n,m,p,h", [("large", (700, 12, 10), 32, 5, 4e-4),      # several groups of i1 blocks
+                                          ("large", (20, 260, 12), 40, 6, 1e-3),      # several tiles of i2
+                                          ("precision", (96, 100, 24), 64, 33, 2e-3)])  # the largest bases
+def test_matches_oracle_at_the_plane_kernels_edges(name, n, m, p, h):
+    g, tens = _tensors(n, m, name=name, h=h)
+    hd = zbc.zbc_create_from_host(g, 3, tens)
+    X, Phi, Y, Psi, launches = _both(hd, g, m, p)
+    assert launches == [FWD, ADJ]
+    assert _rel(Y, products.matvec(tens, g.shape, X)) < RTOL
+    assert _rel(Psi, products.rmatvec(tens, g.shape, Phi)) < RTOL
+
+
+def test_unaligned_vectors():
+    """Columns that start off 16 bytes, and odd leading dimensions, on an even grid."""
+    g, tens = _tensors((40, 36, 20), 40)
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    X, Phi, Y, Psi, _ = _both(h, g, 40, 6)
+    rows = 3 * g.nv
+    buf = torch.zeros((6, rows + 3), dtype=torch.complex64, device="cuda")
+    out = torch.zeros((6, 43), dtype=torch.complex64, device="cuda")
+    P, O = buf[:, 1:1 + rows], out[:, 1:41]
+    P.copy_(zbc.to_colmajor(Phi))
+    zbc.zbc_rmatvec(h, P, O, zbc.AUTO)
+    Xb = torch.zeros((6, 43), dtype=torch.complex64, device="cuda")
+    Xb[:, 1:41].copy_(zbc.to_colmajor(X))
+    P.fill_(float("nan"))
+    zbc.zbc_matvec(h, Xb[:, 1:41], P, zbc.AUTO)
+    zbc.zbc_product_status(h)
+    assert _rel(zbc.from_colmajor(O), products.rmatvec(tens, g.shape, Phi)) < RTOL
+    assert _rel(zbc.from_colmajor(P), products.matvec(tens, g.shape, X)) < RTOL
+    assert not buf[:, 0].any() and not buf[:, 1 + rows:].any()
 
 
 def test_masked_grid_keeps_exact_zeros():
