@@ -381,34 +381,55 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const float2* __re
   out[j + ldo * s] = acc;
 }
 
-// out = op(V) * B:  conj=1 -> V^H B (V is m x M, out M x p); conj=0 -> V B (out m x p)
-__global__ void __launch_bounds__(256) small_gemm_kernel(const float2* __restrict__ V, int m, int Mc, int conj,
-                                                         const float2* __restrict__ B, int64_t ldb, int p,
-                                                         float2* __restrict__ out, int64_t ldo) {
-  const int rows = conj ? Mc : m;
-  const int K = conj ? m : Mc;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)rows * p) return;
-  const int r = (int)(e % rows), s = (int)(e / rows);
+// out = V^H B (V is m x M, out M x p): one warp per entry, its lanes along a column of V.  One thread
+// per entry read V across its columns and walked all m rows alone (m = 512, M = 96, p = 3: two CTAs,
+// most of the product's time).
+__global__ void __launch_bounds__(256) aca_pre_kernel(const float2* __restrict__ V, int m, int M,
+                                                      const float2* __restrict__ B, int64_t ldb,
+                                                      float2* __restrict__ out) {
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), s = blockIdx.y, lane = threadIdx.x & 31;
+  if (r >= M) return;
+  const float2* v = V + (int64_t)m * r;
+  const float2* b = B + ldb * s;
   float2 acc = make_float2(0.f, 0.f);
-  if (conj) {
-    for (int i = 0; i < K; ++i) acc = cfma_conj(V[i + (int64_t)m * r], B[i + ldb * s], acc);
-  } else {
-    for (int i = 0; i < K; ++i) acc = cfma(V[r + (int64_t)m * i], B[i + ldb * s], acc);
+#pragma unroll 4
+  for (int i = lane; i < m; i += 32) acc = cfma_conj(v[i], b[i], acc);
+  for (int o = 16; o > 0; o >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
   }
-  out[r + ldo * s] = acc;
+  if (lane == 0) out[r + (int64_t)M * s] = acc;
+}
+
+// out = V B (out m x p): 32 rows a CTA, the M terms over its 8 warps
+__global__ void __launch_bounds__(256) aca_post_kernel(const float2* __restrict__ V, int m, int M,
+                                                       const float2* __restrict__ B, float2* __restrict__ out,
+                                                       int64_t ldo) {
+  __shared__ float2 red[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane, s = blockIdx.y;
+  float2 acc = make_float2(0.f, 0.f);
+  if (r < m)
+#pragma unroll 4
+    for (int i = w; i < M; i += 8) acc = cfma(V[r + (int64_t)m * i], B[i + (int64_t)M * s], acc);
+  red[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && r < m) {
+    for (int i = 1; i < 8; ++i) {
+      acc.x += red[i][lane].x;
+      acc.y += red[i][lane].y;
+    }
+    out[r + ldo * s] = acc;
+  }
 }
 
 int aca_pre(const Handle& h, const float2* X, int64_t ldx, int p, float2* Xp, cudaStream_t st) {
-  const int64_t n = (int64_t)h.M * p;
-  small_gemm_kernel<<<ceil_div(n, 256), 256, 0, st>>>(h.d_v, h.m, h.M, 1, X, ldx, p, Xp, h.M);
+  aca_pre_kernel<<<dim3(ceil_div(h.M, 8), p), 256, 0, st>>>(h.d_v, h.m, h.M, X, ldx, Xp);
   ZBC_TRY_CUDA(cudaGetLastError());
   count_launch();
   return ZBC_OK;
 }
 int aca_post(const Handle& h, const float2* Psip, int p, float2* Psi, int64_t ldpsi, cudaStream_t st) {
-  const int64_t n = (int64_t)h.m * p;
-  small_gemm_kernel<<<ceil_div(n, 256), 256, 0, st>>>(h.d_v, h.m, h.M, 0, Psip, h.M, p, Psi, ldpsi);
+  aca_post_kernel<<<dim3(ceil_div(h.m, 32), p), 256, 0, st>>>(h.d_v, h.m, h.M, Psip, Psi, ldpsi);
   ZBC_TRY_CUDA(cudaGetLastError());
   count_launch();
   return ZBC_OK;
