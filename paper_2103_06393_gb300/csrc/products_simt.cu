@@ -75,19 +75,26 @@ int transpose_rhs(Handle& h, const float2* X, int64_t ldx, int p, int chunk, con
 }
 
 // ---------------------------------------------------------------------------------------------
-// Algorithm 1: one CTA per (voxel tile, component k, s-chunk); items = the M stored columns
+// Algorithm 1: one CTA per (voxel tile, component k, s-chunk); items = the M stored columns.  A tile
+// takes about 1 us a column whatever its size, so a grid with fewer tiles than SMs is bound by that
+// chain (24^3, 64 columns, 1 right-hand side: 72 CTAs, 66 us); its columns are cut into slices of
+// `jper` (blockIdx.z / schunks), whose sums go to Y + slice * ystride and are added in order by
+// sum_slices_kernel.
 // ---------------------------------------------------------------------------------------------
 template <int PS, int NT>
 __global__ void __launch_bounds__(32 * (NT + 1), 1)
     matvec_simt_kernel(const float2* __restrict__ cache, const CacheDesc* __restrict__ cdesc, Geo g, int q, int M,
                        StageLayout SL, int S, const float2* __restrict__ XT, int pst, int p,
-                       float2* __restrict__ Y, int64_t ldy, int* __restrict__ err) {
+                       float2* __restrict__ Y, int64_t ldy, int schunks, int jper, int64_t ystride,
+                       int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint64_t full[kMaxStages], empty[kMaxStages];
   __shared__ int meta[kMaxStages];
   __shared__ volatile int abort_flag;
   const int k = blockIdx.y;
-  const int s0 = blockIdx.z * PS;
+  const int s0 = (int)(blockIdx.z % schunks) * PS, slice = blockIdx.z / schunks;
+  const int j0 = slice * jper, nj = min(M - j0, jper);
+  Y += slice * ystride;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ncw = g.ntask;
   const int B1p = (g.B1 + 1) / 2 * 2;
@@ -107,15 +114,15 @@ __global__ void __launch_bounds__(32 * (NT + 1), 1)
     if (lane == 0) {
       const uint32_t xb = StageLayout::r16(8u * PS);
       int issued = 0;
-      for (int c = 0; c < M; ++c) {
+      for (int c = 0; c < nj; ++c) {
         const int st = c % S;
         if (c >= S && (abort_flag || !tc::mbar_wait(&empty[st], ((c / S) - 1) & 1))) {
           abort_flag = 1;
           break;
         }
-        const CacheDesc d = cdesc[(int64_t)c * q + k];
+        const CacheDesc d = cdesc[(int64_t)(j0 + c) * q + k];
         issue_item(smem + (size_t)st * SL.stride, SL, &full[st], &meta[st], cache, d, g, B1p, i1_0, i2_0, i3,
-                   XT + (int64_t)c * pst + s0, xb);
+                   XT + (int64_t)(j0 + c) * pst + s0, xb);
         issued = c + 1;
       }
       if (abort_flag)  // let the copies in flight land before the CTA exits
@@ -132,7 +139,7 @@ __global__ void __launch_bounds__(32 * (NT + 1), 1)
     for (int l = 0; l < kUQ; ++l)
 #pragma unroll
       for (int i = 0; i < PS; ++i) acc[l][i] = make_float2(0.f, 0.f);
-    for (int c = 0; c < M; ++c) {
+    for (int c = 0; c < nj; ++c) {
       const int st = c % S;
       // warp-uniform decisions: the warp shuffles below need every lane
       if (__any_sync(0xffffffffu, abort_flag != 0)) break;
@@ -178,6 +185,21 @@ __global__ void __launch_bounds__(32 * (NT + 1), 1)
   }
   __syncthreads();
   if (threadIdx.x == 0 && abort_flag) atomicOr(err, kErrTimeout);
+}
+
+// Y[e, s] = sum over the slices, in order, of part[slice][s][e]
+__global__ void __launch_bounds__(256) sum_slices_kernel(const float2* __restrict__ part, int slices, int64_t rows, int p,
+                                                         float2* __restrict__ Y, int64_t ldy) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= rows) return;
+  const int s = blockIdx.y;
+  float2 acc = part[(int64_t)s * rows + e];
+  for (int i = 1; i < slices; ++i) {
+    const float2 v = part[((int64_t)i * p + s) * rows + e];
+    acc.x += v.x;
+    acc.y += v.y;
+  }
+  Y[e + ldy * s] = acc;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -463,11 +485,32 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   ZBC_CHECK_ARG(S >= 2, "rank %d too large for the FP32 SIMT path", R);
   const size_t sm = (size_t)S * SL.stride;
   ZBC_TRY((set_smem_limit<matvec_simt_kernel<PS, NT>>((int)kSmemBudget)));
-  dim3 grid(g.ntiles(), h.q, schunks);
+  // slices of at least 8 columns while the CTAs are fewer than two waves; not where a stream capture would
+  // have to grow the workspace
+  const int64_t ctas = (int64_t)g.ntiles() * h.q * schunks, rows = (int64_t)h.q * h.nv();
+  int slices = ctas < sm_count() ? (int)std::min<int64_t>({8, h.M / 8, 2 * sm_count() / ctas}) : 1;
+  if (slices > 1) {
+    const size_t bytes = sizeof(float2) * (size_t)slices * rows * p;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (h.work_partial.bytes < bytes) ZBC_TRY_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (cap == cudaStreamCaptureStatusNone)
+      ZBC_TRY(h.work_partial.ensure(bytes));
+    else
+      slices = 1;
+  }
+  const int jper = slices > 1 ? ceil_div(h.M, slices) : h.M;
+  if (slices > 1) slices = ceil_div(h.M, jper);
+  float2* out = slices > 1 ? (float2*)h.work_partial.ptr : Y;
+  dim3 grid(g.ntiles(), h.q, schunks * std::max(1, slices));
   matvec_simt_kernel<PS, NT><<<grid, 32 * (g.ntask + 1), sm, st>>>(h.cache->data, h.cache->d_desc, g, h.q, h.M, SL, S,
-                                                               XT, pst, p, Y, ldy, (int*)h.work_err.ptr);
-  ZBC_TRY_CUDA(cudaGetLastError());
+                                                               XT, pst, p, out, slices > 1 ? rows : ldy, schunks, jper,
+                                                               rows * p, (int*)h.work_err.ptr);
   count_launch();
+  if (slices > 1) {
+    sum_slices_kernel<<<dim3(ceil_div(rows, 256), p), 256, 0, st>>>(out, slices, rows, p, Y, ldy);
+    count_launch();
+  }
+  ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
 }
 
