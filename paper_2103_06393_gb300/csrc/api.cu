@@ -192,7 +192,8 @@ extern "C" int zbc_device_bytes(const zbc_handle* hh, int64_t* pool, int64_t* ca
   if (caches) *caches = cache_bytes(h.cache) + joint_bytes(h.joint);
   if (work)
     *work = (int64_t)(h.work_partial.bytes + h.work_x.bytes + h.work_misc.bytes + h.work_xt.bytes +
-                      h.work_err.bytes + h.work_phi.bytes + h.work_joint.bytes);
+                      h.work_err.bytes + h.work_phi.bytes + h.work_joint_fwd.bytes + h.work_joint_adj.bytes +
+                      h.work_slices.bytes);
   return ZBC_OK;
 }
 

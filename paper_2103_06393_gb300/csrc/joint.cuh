@@ -53,14 +53,14 @@ int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int
 // the column sums on the tensor cores (joint_core.cu): T from X, and partial Psi from F in `splits`
 // slices of `split` chunks of core entries
 size_t joint_core_bytes(const JointGeo& G);
-int joint_core_build(const JointGeo& G, const float2* K, float* kscale, cudaStream_t st);
+int joint_core_build(const JointGeo& G, const float2* K, float* kscale, bool* fits, cudaStream_t st);
 int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, cudaStream_t st);
 void joint_core_split(const JointGeo& G, int p, int* split, int* splits);
 int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, cudaStream_t st);
 
 // Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
 int build_joint(Handle& h, cudaStream_t st);
-// bytes of h.work_joint that one product of p right-hand sides uses (h.joint usable)
+// bytes of h.work_joint_fwd / _adj that one product of p right-hand sides uses (h.joint usable)
 size_t joint_work_bytes(const Handle& h, int p, bool fwd);
 int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st);
 int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* out, int64_t ldo, cudaStream_t st);

@@ -461,10 +461,11 @@ static int build(Handle& h, JointCache* jc, cudaStream_t st) {
     core3_kernel<<<dim3(std::min(64, ceil_div(csmax / kCoreZ + 1, 256)), nt), 256, 0, st>>>(p);
     count_launch(3);
   }
-  ZBC_TRY(joint_core_build(g, jc->K, jc->kscale, st));
+  bool fits = false;
+  ZBC_TRY(joint_core_build(g, jc->K, jc->kscale, &fits, st));
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e, "reduced cores");
-  jc->usable = true;
+  jc->usable = fits;
   return ZBC_OK;
 }
 

@@ -13,9 +13,10 @@
 // registers with the chunk's scales while the next chunk is converted, so that a tensor-core sum has
 // 64 terms.
 //
-// Scales: the adjoint's K per row and chunk.  The forward's rows are shared by the two warps that
-// convert them, so its K is scaled per column j (kscale[j] = 2^(15 - e_j), |K[j]| < 2^e_j, from the
-// build) and X by 2^(e_j - e), e the component's largest e_j.
+// Scales: K per column j (kscale[j] = 2^(15 - e_j), |K[j]| < 2^e_j, from the build; fp16 hi + lo then
+// leave 2^-40 of a column's largest entry); the forward's X by 2^(e_j - e), e the component's largest
+// e_j; the right-hand sides' entries per chunk.  Scales of K's rows taken anew in every chunk of the
+// adjoint cost a fifth of its issue slots (0.61 ms at 96^3, 16 right-hand sides).
 #include <algorithm>
 
 #include "joint_tc.cuh"
@@ -25,6 +26,8 @@ namespace {
 
 constexpr int kRows = 128, kSum = 32;
 constexpr uint32_t kRowTerm = kRows * 128u;  // one term of K's chunk
+
+__host__ __device__ inline int slices_of(int Cs, int split) { return ((Cs + kSum - 1) / kSum + split - 1) / split; }
 
 template <int P>
 constexpr size_t core_smem() {
@@ -41,8 +44,7 @@ __global__ void __launch_bounds__(288, 2)
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t done[2], ready[2];
   __shared__ uint32_t tmem_base;
-  __shared__ int rexp[4][kRows];
-  __shared__ int bexp[4][P];
+  __shared__ float bscale[4][P];            // 2^(e - kDataShift) of a chunk's right-hand sides
   unsigned char* sa = smem;                 // [2 buffers][2 terms][128 rows][128 B]
   unsigned char* sb = sa + 4 * kRowTerm;    // [2 buffers][2 terms][N rows][128 B]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -62,15 +64,16 @@ __global__ void __launch_bounds__(288, 2)
     }
   };
   // forward: items are the 128-row tiles of all components, walked by blockIdx.x; adjoint: one item,
-  // the chunks [split blockIdx.x, + split) of all components in order, for rows 128 blockIdx.y
-  const int s0 = blockIdx.z * P;
-  int tiles = 0, chunks = 0;
-  for (int k = 0; k < G.q; ++k) {
-    tiles += (G.Cs[k] + kRows - 1) / kRows;
-    chunks += (G.Cs[k] + kSum - 1) / kSum;
+  // slice blockIdx.x of `split` chunks of one component (ksplit, first chunk ch0), for rows 128 blockIdx.y
+  const int s0 = blockIdx.z * P, Mp = (G.M + kSum - 1) / kSum * kSum;
+  int tiles = 0, ksplit = 0, ch0 = blockIdx.x;
+  for (int k = 0; k < G.q; ++k) tiles += (G.Cs[k] + kRows - 1) / kRows;
+  if (!FWD) {
+    for (int n; ch0 >= (n = slices_of(G.Cs[ksplit], split)); ++ksplit) ch0 -= n;
+    ch0 *= split;
   }
   const int items = FWD ? (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 1;
-  const int per = FWD ? (G.M + kSum - 1) / kSum : min(split, chunks - (int)blockIdx.x * split);
+  const int per = FWD ? Mp / kSum : min(split, (G.Cs[ksplit] + kSum - 1) / kSum - ch0);
   if (warp == 8) {
     if (lane == 0) {
       constexpr uint32_t id = tc::instr_desc(128, N, 0);
@@ -140,25 +143,23 @@ __global__ void __launch_bounds__(288, 2)
         }
       }
     };
-    auto advance = [&]() {  // adjoint: the next chunk
-      fpos += kSum;
-      if (fpos >= G.Cs[fk]) {
-        ++fk;
-        fpos = 0;
-      }
-    };
+    float kr[4];  // adjoint: scales of the loader's rows
     if (FWD) {
       locate_tile(blockIdx.x);
     } else {
-      int ch = blockIdx.x * split;
-      for (int n; ch >= (n = (G.Cs[fk] + kSum - 1) / kSum); ++fk) ch -= n;
-      fpos = ch * kSum;
+      fk = ksplit;
+      fpos = ch0 * kSum;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = blockIdx.y * kRows + row0 + 32 * u;
+        kr[u] = j < G.M ? __ldg(kscale + (int64_t)fk * 2 * Mp + j) : 1.f;
+      }
     }
     fetch(0);
     int c0 = 0;  // the CTA's number of this item's first chunk
     for (int item = 0; item < items; ++item, c0 += per) {
       const int k = fk, row = fpos;
-      const float* ks = kscale + (int64_t)k * 2 * ((G.M + kSum - 1) / kSum * kSum);
+      const float* ks = kscale + (int64_t)k * 2 * Mp;
       float acc[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) acc[i] = 0.f;
@@ -166,7 +167,6 @@ __global__ void __launch_bounds__(288, 2)
         const int d = c & 1;
         wait(&done[d], (c >> 1) & 1);
         tc::fence_after();
-        const float rf = FWD ? 1.f : pow2f(rexp[c & 3][32 * q4 + lane] - kDataShift);
         const uint32_t t0 = tmem + (uint32_t)(d * N + half * P) + ((uint32_t)(32 * q4) << 16);
 #pragma unroll
         for (int i = 0; i < I; ++i) {
@@ -174,12 +174,10 @@ __global__ void __launch_bounds__(288, 2)
           tmem_ld8(t0 + 8 * i, r);
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const float cf = pow2f(bexp[c & 3][half * (P / 2) + 4 * i + u] - kDataShift);
+            const float cf = bscale[c & 3][half * (P / 2) + 4 * i + u];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float v = __uint_as_float(r[2 * u + e]);
-              acc[8 * i + 2 * u + e] = fmaf(FWD ? v : v * rf, cf, acc[8 * i + 2 * u + e]);
-            }
+            for (int e = 0; e < 2; ++e)
+              acc[8 * i + 2 * u + e] = fmaf(__uint_as_float(r[2 * u + e]), cf, acc[8 * i + 2 * u + e]);
           }
         }
         tc::fence_before();
@@ -206,19 +204,10 @@ __global__ void __launch_bounds__(288, 2)
         } else {
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            float m = 0.f;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) m = absmax_nan(m, x[4 * u + w].x, x[4 * u + w].y);
-            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
-            const int e = exp_of(m), r = row0 + 32 * u;
-            if (c8 == 0) rexp[c & 3][r] = e;
-            const float sc = pow2f(kDataShift - e);
             uint32_t h[4], l[4];
 #pragma unroll
-            for (int w = 0; w < 4; ++w) split2(x[4 * u + w].x * sc, x[4 * u + w].y * sc, h[w], l[w]);
-            unsigned char* o = ad + tc::sw128_off(r, c8);
+            for (int w = 0; w < 4; ++w) split2(x[4 * u + w].x * kr[u], x[4 * u + w].y * kr[u], h[w], l[w]);
+            unsigned char* o = ad + tc::sw128_off(row0 + 32 * u, c8);
             *(uint4*)o = make_uint4(h[0], h[1], h[2], h[3]);
             *(uint4*)(o + kRowTerm) = make_uint4(l[0], l[1], l[2], l[3]);
           }
@@ -226,7 +215,7 @@ __global__ void __launch_bounds__(288, 2)
         // the right-hand sides' rows (two a right-hand side): pair `lane` of the chunk in the rows' order
         const uint32_t kc = FWD ? lane / 4 : lane % 16 / 2, word = FWD ? lane % 4 : lane % 2 + lane / 16 * 2;
         float xs = 1.f;  // 2^(e_j - e)
-        if (FWD) xs = __ldg(ks + (G.M + kSum - 1) / kSum * kSum + ch * kSum + lane);
+        if (FWD) xs = __ldg(ks + Mp + ch * kSum + lane);
 #pragma unroll
         for (int i = 0; i < I; ++i) {
           float2 v = b[i];
@@ -238,7 +227,7 @@ __global__ void __launch_bounds__(288, 2)
           float m = absmax_nan(0.f, v.x, v.y);
           for (int o = 16; o > 0; o >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
           const int e = exp_of(m), n = 2 * (warp + 8 * i);
-          if (lane == 0) bexp[c & 3][warp + 8 * i] = e;
+          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2f(e - kDataShift);
           const float sc = pow2f(kDataShift - e);
           uint32_t h, l;
           split2(v.x * sc, v.y * sc, h, l);
@@ -252,7 +241,7 @@ __global__ void __launch_bounds__(288, 2)
           *(uint32_t*)(o1 + kBTerm) = FWD ? ls : ls ^ 0x80000000u;
         }
         if (ch + 1 < per) {
-          if (!FWD) advance();
+          if (!FWD) fpos += kSum;
           fetch(ch + 1);
         } else if (item + 1 < items) {
           locate_tile((int)blockIdx.x + (item + 1) * (int)gridDim.x);
@@ -264,8 +253,8 @@ __global__ void __launch_bounds__(288, 2)
       fold(c0 + per - 1);
       const int r = 32 * q4 + lane;
       if (FWD) {
-        // K was scaled by 2^(15 - e_j) and X by 2^(e_j - e): what is left is 2^(e - 15)
-        const float ko = __ldg(kscale + (int64_t)G.q * 2 * ((G.M + kSum - 1) / kSum * kSum) + k);
+        // K was scaled by 2^(15 - e_j) and X by 2^(e_j - e): 2^(e - 15) is left
+        const float ko = __ldg(kscale + (int64_t)G.q * 2 * Mp + k);
         if (row + r < G.Cs[k])
 #pragma unroll
           for (int i = 0; i < P / 2; ++i) {
@@ -274,11 +263,12 @@ __global__ void __launch_bounds__(288, 2)
           }
       } else {
         const int j = blockIdx.y * kRows + r;
+        const float kj = j < G.M ? 1.f / __ldg(ks + j) : 0.f;  // 2^(e_j - 15)
         if (j < G.M)
 #pragma unroll
           for (int i = 0; i < P / 2; ++i) {
             const int s = s0 + half * (P / 2) + i;
-            if (s < p) out[((int64_t)blockIdx.x * p + s) * G.M + j] = make_float2(acc[2 * i], acc[2 * i + 1]);
+            if (s < p) out[((int64_t)blockIdx.x * p + s) * G.M + j] = make_float2(acc[2 * i] * kj, acc[2 * i + 1] * kj);
           }
       }
     }
@@ -354,12 +344,19 @@ int rhs_tile(int p) { return p <= 8 ? 8 : p <= 16 ? 16 : 32; }
 
 size_t joint_core_bytes(const JointGeo& G) { return sizeof(float) * ((size_t)G.q * 2 * padded_m(G) + G.q); }
 
-int joint_core_build(const JointGeo& G, const float2* K, float* kscale, cudaStream_t st) {
+int joint_core_build(const JointGeo& G, const float2* K, float* kscale, bool* fits, cudaStream_t st) {
   const int Mp = padded_m(G);
   core_exp_kernel<<<dim3(Mp, G.q), 128, 0, st>>>(G, K, Mp, kscale);
   core_scale_kernel<<<G.q, 256, 0, st>>>(G, Mp, kscale);
   count_launch(2);
   ZBC_TRY_CUDA(cudaGetLastError());
+  // columns further apart than FP32's exponents reach have no common scale
+  std::vector<float> rel((size_t)G.q * 2 * Mp);
+  ZBC_TRY_CUDA(cudaMemcpyAsync(rel.data(), kscale, sizeof(float) * rel.size(), cudaMemcpyDeviceToHost, st));
+  ZBC_TRY_CUDA(cudaStreamSynchronize(st));
+  *fits = true;
+  for (int k = 0; k < G.q; ++k)
+    for (int j = 0; j < G.M; ++j) *fits = *fits && rel[((size_t)2 * k + 1) * Mp + j] > 1e-35f;
   return ZBC_OK;
 }
 
@@ -380,7 +377,8 @@ void joint_core_split(const JointGeo& G, int p, int* split, int* splits) {
   // one wave of two CTAs an SM, at least 4 chunks each
   const int want = std::max(1, 2 * sm_count() / (ceil_div(G.M, kRows) * ceil_div(p, rhs_tile(p))));
   *split = std::max(4, ceil_div(chunks, want));
-  *splits = ceil_div(chunks, *split);
+  *splits = 0;
+  for (int k = 0; k < G.q; ++k) *splits += slices_of(G.Cs[k], *split);
 }
 
 int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, cudaStream_t st) {

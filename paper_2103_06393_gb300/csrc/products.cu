@@ -28,7 +28,7 @@ static bool joint_ready(Handle& h, int p, bool fwd, cudaStream_t st) {
     return false;
   }
   if (cap != cudaStreamCaptureStatusNone)
-    return h.joint && h.joint->usable && h.work_joint.bytes >= joint_work_bytes(h, p, fwd);
+    return h.joint && h.joint->usable && (fwd ? h.work_joint_fwd : h.work_joint_adj).bytes >= joint_work_bytes(h, p, fwd);
   if (!h.joint && build_joint(h, st) != ZBC_OK) {
     clear_error();
     cudaGetLastError();

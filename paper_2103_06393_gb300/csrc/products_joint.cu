@@ -269,8 +269,10 @@ __global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict
 
 constexpr int kPassRhs = 64;  // right-hand sides per round of the workspaces
 
-// from this many right-hand sides of a round on, the column sums run on the tensor cores
-constexpr int kTcRhs = 5;
+// From this many right-hand sides of a round on, the column sums run on the tensor cores (at least 8 a
+// pass).  160 x 160 x 128, 4096 columns: whole forward 0.92 ms in FP32 at 4 against 1.40 ms at 8, whole
+// adjoint 1.35 / 2.05 ms in FP32 at 2 / 4 against 1.37 ms at 8.
+constexpr int kTcFwd = 5, kTcAdj = 3;
 
 int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : 4; }  // FP32 column sums
 
@@ -297,7 +299,7 @@ struct FwdPlan {
     P = rhs_per_cta(ps);
     // enough CTAs for 6 per SM, at least 32 columns a slice
     JS = std::max(1, std::min({16, G.M / 32, ceil_div(6 * sm_count(), cblocks * ceil_div(ps, P))}));
-    if (ps >= kTcRhs) JS = 1;
+    if (ps >= kTcFwd) JS = 1;
     telems = (int64_t)JS * ps * G.Ct;
     qelems = (int64_t)ps * G.Qt;
   }
@@ -313,7 +315,7 @@ struct AdjPlan {
     chunk = (int)std::max<int64_t>(256, (G.Ct / want + kCc - 1) / kCc * kCc);
     splits = 0;
     for (int k = 0; k < G.q; ++k) splits += ceil_div(G.Cs[k], chunk);
-    if (ps >= kTcRhs) joint_core_split(G, ps, &chunk, &splits);
+    if (ps >= kTcAdj) joint_core_split(G, ps, &chunk, &splits);
     felems = (int64_t)ps * G.Ct;
     qelems = (int64_t)ps * G.Qt;
     pelems = (int64_t)splits * ps * G.M;
@@ -335,7 +337,7 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
   const JointCache& jc = *h.joint;
   const JointGeo& G = jc.geo;
   int* err = (int*)h.work_err.ptr;
-  ZBC_TRY(h.work_joint.ensure(joint_work_bytes(h, p, true)));
+  ZBC_TRY(h.work_joint_fwd.ensure(joint_work_bytes(h, p, true)));
   int csmax = 0, rrmax = 0;
   for (int k = 0; k < G.q; ++k) {
     csmax = std::max(csmax, G.Cs[k]);
@@ -345,10 +347,10 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
     const int ps = std::min(kPassRhs, p - s0);
     const FwdPlan pl(G, ps);
     const int JS = pl.JS;
-    float2* T = (float2*)h.work_joint.ptr;
+    float2* T = (float2*)h.work_joint_fwd.ptr;
     float2* Q = T + pl.telems;
     const float2* Xs = X + ldx * s0;
-    switch (ps >= kTcRhs ? 0 : pl.P) {
+    switch (ps >= kTcFwd ? 0 : pl.P) {
       case 0: ZBC_TRY(joint_core_fwd(jc, Xs, ldx, ps, T, err, st)); break;
       case 1: launch_core_fwd<1>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
       case 2: launch_core_fwd<2>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
@@ -365,7 +367,7 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
   const JointCache& jc = *h.joint;
   const JointGeo& G = jc.geo;
   int* err = (int*)h.work_err.ptr;
-  ZBC_TRY(h.work_joint.ensure(joint_work_bytes(h, p, false)));
+  ZBC_TRY(h.work_joint_adj.ensure(joint_work_bytes(h, p, false)));
   int r3 = 0, rrmax = 0;
   for (int k = 0; k < G.q; ++k) {
     r3 = std::max(r3, G.R[k][2]);
@@ -375,17 +377,16 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
     const int ps = std::min(kPassRhs, p - s0);
     const AdjPlan pl(G, ps);
     const int chunk = pl.chunk, splits = pl.splits;
-    float2* Q = (float2*)h.work_joint.ptr;
+    float2* Q = (float2*)h.work_joint_adj.ptr;
     float2* F = Q + pl.qelems;
     float2* part = F + pl.felems;
     const float2* Ps = Phi + ldphi * s0;
     ZBC_TRY(joint_planes_adj(jc, Ps, ldphi, ps, Q, err, st));
     joint_mode3_adj_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(r3, 8), ps * G.q), 128, 0, st>>>(G, jc.basis, Q, F);
-    switch (ps >= kTcRhs ? 0 : pl.P) {
+    switch (ps >= kTcAdj ? 0 : pl.P) {
       case 0: ZBC_TRY(joint_core_adj(jc, F, ps, part, err, st)); break;
       case 1: launch_core_adj<1>(G, jc.K, F, ps, chunk, splits, part, st); break;
-      case 2: launch_core_adj<2>(G, jc.K, F, ps, chunk, splits, part, st); break;
-      default: launch_core_adj<4>(G, jc.K, F, ps, chunk, splits, part, st); break;
+      default: launch_core_adj<2>(G, jc.K, F, ps, chunk, splits, part, st); break;
     }
     joint_sum_kernel<<<dim3(ceil_div(G.M, 32), ps), 256, 0, st>>>(part, G.M, ps, splits, out + ldo * s0, ldo);
     count_launch(2);

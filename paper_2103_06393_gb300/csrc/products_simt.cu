@@ -492,15 +492,15 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   if (slices > 1) {
     const size_t bytes = sizeof(float2) * (size_t)slices * rows * p;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (h.work_partial.bytes < bytes) ZBC_TRY_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (h.work_slices.bytes < bytes) ZBC_TRY_CUDA(cudaStreamIsCapturing(st, &cap));
     if (cap == cudaStreamCaptureStatusNone)
-      ZBC_TRY(h.work_partial.ensure(bytes));
+      ZBC_TRY(h.work_slices.ensure(bytes));
     else
       slices = 1;
   }
   const int jper = slices > 1 ? ceil_div(h.M, slices) : h.M;
   if (slices > 1) slices = ceil_div(h.M, jper);
-  float2* out = slices > 1 ? (float2*)h.work_partial.ptr : Y;
+  float2* out = slices > 1 ? (float2*)h.work_slices.ptr : Y;
   dim3 grid(g.ntiles(), h.q, schunks * std::max(1, slices));
   matvec_simt_kernel<PS, NT><<<grid, 32 * (g.ntask + 1), sm, st>>>(h.cache->data, h.cache->d_desc, g, h.q, h.M, SL, S,
                                                                XT, pst, p, out, slices > 1 ? rows : ldy, schunks, jper,

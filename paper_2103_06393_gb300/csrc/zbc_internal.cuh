@@ -101,7 +101,10 @@ struct Handle {
   DevBuf work_xt;        // X^T of the forward products (s-chunk padded rows)
   DevBuf work_err;       // int: error bits kErrTimeout / kErrNonFinite set by the product kernels
   DevBuf work_phi;       // mode-1 adjoint: fp16 operand blocks of Phi and their exponents
-  DevBuf work_joint;     // joint form: reduced sums, planes and partial sums
+  // a buffer of each direction its own: a call of the other one never moves what a captured graph uses
+  DevBuf work_joint_fwd; // joint form: the columns' sums and the planes before the expansion
+  DevBuf work_joint_adj; // joint form: the projected planes, their cores and partial sums
+  DevBuf work_slices;    // FP32 forward: the column slices' sums
   DecompCache* cache = nullptr;
   JointCache* joint = nullptr;
   int cache_r = 0;                 // largest r1 rounded up to 2 (cache row stride bound)

@@ -232,3 +232,27 @@ def test_capture_without_a_basis_runs_the_form_it_ran():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(Y, Z)
+
+
+@pytest.mark.parametrize("form", ["auto", "fp32"])
+def test_graph_of_one_product_survives_the_other(form):
+    """A captured forward keeps its buffers when the adjoint runs for the first time afterwards."""
+    g, tens = _tensors((40, 36, 20), 40)
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    prec = zbc.AUTO if form == "auto" else zbc.FP32_SIMT
+    X = zbc.to_colmajor(inputs.cn01((40, 6), seed=1).astype(np.complex64))
+    Phi = zbc.to_colmajor(inputs.cn01((3 * g.nv, 6), seed=2).astype(np.complex64))
+    Y, Z = (zbc.colmajor(3 * g.nv, 6, torch.complex64) for _ in range(2))
+    Psi = zbc.colmajor(40, 6, torch.complex64)
+    zbc.zbc_matvec(h, X, Y, prec)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        zbc.zbc_matvec(h, X, Z, prec)
+    work = h.device_bytes()["work"]
+    zbc.zbc_rmatvec(h, Phi, Psi, prec)
+    assert h.device_bytes()["work"] > work  # the adjoint took buffers of its own
+    graph.replay()
+    torch.cuda.synchronize()
+    zbc.zbc_product_status(h)
+    assert torch.equal(Y, Z)
