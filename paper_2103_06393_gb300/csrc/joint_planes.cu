@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     if (mine > 1) fetch_q(1);
     int n = 0;
     for (int t = 0; t < mine + lag; ++t) {
-      const int eout = lag ? elast : e;  // of the plane that is stored in this round
+      const int eout = lag ? elast : e;  // of the plane that is stored in this pass
       if (t < mine) {
         // S's rows 2 i2, 2 i2 + 1 from D1's row i2: D1 = 2^(kDataShift + kBasisShift - e) S, so 2^-9 D1 < 2^15,
         // and D2 = 2^(21 - e) Y

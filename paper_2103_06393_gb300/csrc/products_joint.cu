@@ -267,9 +267,9 @@ __global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict
   }
 }
 
-constexpr int kPassRhs = 64;  // right-hand sides per round of the workspaces
+constexpr int kPassRhs = 64;  // right-hand sides that the workspaces hold at a time
 
-// From this many right-hand sides of a round on, the column sums run on the tensor cores (at least 8 a
+// From this many right-hand sides on, the column sums run on the tensor cores (at least 8 a
 // pass).  160 x 160 x 128, 4096 columns: whole forward 0.92 ms in FP32 at 4 against 1.40 ms at 8, whole
 // adjoint 1.35 / 2.05 ms in FP32 at 2 / 4 against 1.37 ms at 8.
 constexpr int kTcFwd = 5, kTcAdj = 3;
@@ -289,7 +289,7 @@ void launch_core_adj(const JointGeo& G, const float2* K, const float2* F, int p,
   count_launch();
 }
 
-// work split of one round of ps <= kPassRhs right-hand sides
+// work split of ps <= kPassRhs right-hand sides
 struct FwdPlan {
   int P, JS;              // right-hand sides per CTA, slices of the column sum
   int64_t telems, qelems;
@@ -327,7 +327,7 @@ struct AdjPlan {
 
 size_t joint_work_bytes(const Handle& h, int p, bool fwd) {
   const JointGeo& G = h.joint->geo;
-  size_t b = 0;  // the last round holds the rest of p
+  size_t b = 0;  // the last batch holds the rest of p
   for (int ps : {std::min(p, kPassRhs), p % kPassRhs})
     if (ps > 0) b = std::max(b, fwd ? FwdPlan(G, ps).bytes() : AdjPlan(G, ps).bytes());
   return b;

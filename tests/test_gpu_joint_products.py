@@ -1,6 +1,6 @@
 """The joint-subspace form of both products, which ZBC_AUTO runs on an untuned handle whose columns'
 factors share a small basis: against the FP64 oracle at the sizes where its kernels change shape
-(ragged grids and tiles, passes and rounds of right-hand sides, few and many columns, ACA storage,
+(ragged grids and tiles, passes and batches of right-hand sides, few and many columns, ACA storage,
 q = 12, masked voxels), its status word, stream capture, and the handles that must not take it."""
 import numpy as np
 import pytest
@@ -22,7 +22,7 @@ from paper_2103_06393_gb300 import zbc  # noqa: E402
 # FP32 sums of at most a few thousand terms of the same scale: sqrt(4000) 2^-24 = 4e-6, and the
 # basis adds at most sqrt(3) 1e-7
 RTOL = 5e-6
-FWD, ADJ = 3, 4  # kernels of one round of the joint form
+FWD, ADJ = 3, 4  # kernels of the joint form for up to 64 right-hand sides
 
 
 def _tensors(n, m, name="large", tol=1e-6, q=3, h=None):
@@ -70,8 +70,8 @@ def test_matches_oracle(n, m, p):
     g, tens = _tensors(n, m)
     h = zbc.zbc_create_from_host(g, 3, tens)
     X, Phi, Y, Psi, launches = _both(h, g, m, p)
-    rounds = -(-p // 64)
-    assert launches == [FWD * rounds, ADJ * rounds]
+    batches = -(-p // 64)
+    assert launches == [FWD * batches, ADJ * batches]
     assert _rel(Y, products.matvec(tens, g.shape, X)) < RTOL
     assert _rel(Psi, products.rmatvec(tens, g.shape, Phi)) < RTOL
 
