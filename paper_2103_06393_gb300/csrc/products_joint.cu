@@ -1,11 +1,13 @@
 // The products through a joint basis of the columns' factors (joint.cuh).
 //
-// Forward:  T = sum_j K_j X[j, :]        joint_core_fwd_kernel    (R1 R2 R3 entries per component)
+// Forward:  T = sum_j K_j X[j, :]        joint_core_fwd_kernel, joint_core.cu   (R1 R2 R3 entries per component)
 //           Q[i3] = T x3 B3              joint_mode3_fwd_kernel
 //           Y[:, :, i3] = B1 Q[i3] B2^T  joint_planes.cu          (one write of Y)
 // Adjoint:  Q[i3] = B1^H Phi[:, :, i3] conj(B2)   joint_planes.cu          (one read of Phi)
 //           F = Q x3 B3^H                         joint_mode3_adj_kernel
-//           Psi[j, :] = sum conj(K_j) F           joint_core_adj_kernel, joint_sum_kernel
+//           Psi[j, :] = sum conj(K_j) F           joint_core_adj_kernel, joint_core.cu; joint_sum_kernel
+// The column sums here are the FP32 ones of a few right-hand sides, which the read of K bounds;
+// joint_core.cu has those of more on the tensor cores.
 #include <algorithm>
 
 #include "decomp.cuh"
@@ -149,16 +151,15 @@ constexpr int kCj = 64;  // columns per CTA of the adjoint core sum
 constexpr int kCc = 32;  // core entries per chunk
 
 // part[split][s][j] = sum over the split's core entries c of conj(K[j][c]) F[s][c].  128 threads:
-// 16 groups of 4 columns, P / TS groups of TS right-hand sides, and KS interleaved slices of the
-// chunk where P is small.  Grid (column tiles, splits of all components' entries, passes of P).
+// 16 groups of 4 columns, P right-hand sides, and KS interleaved slices of the chunk (P = 1 or 2).  Grid (column tiles, splits of all components' entries, passes of P).
 template <int P>
 __global__ void __launch_bounds__(128) joint_core_adj_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ K,
                                                              const float2* __restrict__ F, int p, int chunk,
                                                              float2* __restrict__ part) {
-  constexpr int TS = 1, SG = P, KS = 8 / SG;
+  constexpr int KS = 8 / P;
   __shared__ __align__(16) float2 ks[kCc][kCj + 2];
   __shared__ __align__(16) float2 fs[kCc][P];
-  __shared__ float2 red[KS > 1 ? KS : 1][KS > 1 ? kCj : 1][KS > 1 ? P : 1];
+  __shared__ float2 red[KS][kCj][P];
   int sp = blockIdx.y, k = 0;
   for (; k < G.q; ++k) {
     const int ns = (G.Cs[k] + chunk - 1) / chunk;
@@ -167,26 +168,22 @@ __global__ void __launch_bounds__(128) joint_core_adj_kernel(const __grid_consta
   }
   const int c0 = sp * chunk, c1 = min(G.Cs[k], c0 + chunk);
   const int jb = blockIdx.x * kCj, s0 = blockIdx.z * P;
-  const int jg = threadIdx.x % 16, sg = threadIdx.x / 16 % SG, kq = threadIdx.x / (16 * SG);
+  const int jg = threadIdx.x % 16, sg = threadIdx.x / 16 % P, kq = threadIdx.x / (16 * P);
   const int cl = threadIdx.x % 32, w4 = threadIdx.x / 32;
   const float2* Kp = K + G.koff[k];
   const float2* Fp = F + G.toff[k];
-  float2 acc[4][TS], sum[4][TS];
+  float2 acc[4], sum[4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < TS; ++b) acc[a][b] = sum[a][b] = make_float2(0.f, 0.f);
+  for (int a = 0; a < 4; ++a) acc[a] = sum[a] = make_float2(0.f, 0.f);
   // the running sums go into the totals every 8 chunks: one FP32 sum over a split's several thousand
   // entries made the 96^3 adjoint's error 1.5e-6, against 9.7e-7 of the mode-1 form
   auto fold = [&]() {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < TS; ++b) {
-        sum[a][b].x += acc[a][b].x;
-        sum[a][b].y += acc[a][b].y;
-        acc[a][b] = make_float2(0.f, 0.f);
-      }
+    for (int a = 0; a < 4; ++a) {
+      sum[a].x += acc[a].x;
+      sum[a].y += acc[a].y;
+      acc[a] = make_float2(0.f, 0.f);
+    }
   };
   float2 kr[kCj / 4];
   auto fetch = [&](int c) {
@@ -210,38 +207,28 @@ __global__ void __launch_bounds__(128) joint_core_adj_kernel(const __grid_consta
 #pragma unroll 4
     for (int i = kq; i < kCc; i += KS) {
       const float4 k0 = *(const float4*)&ks[i][4 * jg], k1 = *(const float4*)&ks[i][4 * jg + 2];
-#pragma unroll
-      for (int b = 0; b < TS; ++b) {
-        const float2 f = fs[i][sg * TS + b];
-        acc[0][b] = cfma_conj(make_float2(k0.x, k0.y), f, acc[0][b]);
-        acc[1][b] = cfma_conj(make_float2(k0.z, k0.w), f, acc[1][b]);
-        acc[2][b] = cfma_conj(make_float2(k1.x, k1.y), f, acc[2][b]);
-        acc[3][b] = cfma_conj(make_float2(k1.z, k1.w), f, acc[3][b]);
-      }
+      const float2 f = fs[i][sg];
+      acc[0] = cfma_conj(make_float2(k0.x, k0.y), f, acc[0]);
+      acc[1] = cfma_conj(make_float2(k0.z, k0.w), f, acc[1]);
+      acc[2] = cfma_conj(make_float2(k1.x, k1.y), f, acc[2]);
+      acc[3] = cfma_conj(make_float2(k1.z, k1.w), f, acc[3]);
     }
     if ((c - c0) / kCc % 8 == 7) fold();
   }
   fold();
-  if constexpr (KS > 1) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a) red[kq][4 * jg + a][sg] = sum[a][0];
-    __syncthreads();
-    if (kq == 0)
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-        for (int w = 1; w < KS; ++w) {
-          sum[a][0].x += red[w][4 * jg + a][sg].x;
-          sum[a][0].y += red[w][4 * jg + a][sg].y;
-        }
-  }
+  for (int a = 0; a < 4; ++a) red[kq][4 * jg + a][sg] = sum[a];
+  __syncthreads();
   if (kq == 0)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < TS; ++b) {
-        const int j = jb + 4 * jg + a, s = s0 + sg * TS + b;
-        if (j < G.M && s < p) part[((int64_t)blockIdx.y * p + s) * G.M + j] = sum[a][b];
+    for (int a = 0; a < 4; ++a) {
+      for (int w = 1; w < KS; ++w) {
+        sum[a].x += red[w][4 * jg + a][sg].x;
+        sum[a].y += red[w][4 * jg + a][sg].y;
       }
+      const int j = jb + 4 * jg + a, s = s0 + sg;
+      if (j < G.M && s < p) part[((int64_t)blockIdx.y * p + s) * G.M + j] = sum[a];
+    }
 }
 
 // out[j, s] = sum over the splits, in order; one warp per 32 columns, the splits over 8 warps
