@@ -61,11 +61,11 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// one CTA per factor: F = U diag(d) / norm, and the first pivot
+// one CTA per factor: F = U diag(d) / norm, and the first pivot (ranks of at most kJointRmax)
 __global__ void __launch_bounds__(128) weight_kernel(const FactorJob* jobs, const Problem* prob, PivotState* state,
                                                      double* resid) {
   const FactorJob jb = jobs[blockIdx.x];
-  __shared__ double w2[kRmax], c2[kRmax];
+  __shared__ double w2[kJointRmax], c2[kJointRmax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ne = (int64_t)jb.r1 * jb.r2 * jb.r3;
   const int64_t per = ne / jb.r;  // entries of one slice along mode g
@@ -296,6 +296,10 @@ static int build(Handle& h, JointCache* jc, cudaStream_t st) {
   g.n3 = h.n3;
   g.q = q;
   g.M = h.M;
+  // A factor of more than kJointRmax columns has no basis of kJointRmax vectors (unless some of its
+  // columns carry less than the tolerance), and the kernels below hold its weights in arrays of that size
+  for (const TensorDesc& d : h.desc)
+    if (std::max({d.r1, d.r2, d.r3}) > kJointRmax) return ZBC_OK;  // unusable
   // factors, grouped by (mode, component) so that a problem's columns are one run
   std::vector<FactorJob> fj;
   std::vector<Problem> prob(NP);

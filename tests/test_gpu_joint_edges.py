@@ -1,0 +1,79 @@
+"""ZBC_AUTO at the edges of the joint form: handles that cannot take it (ranks above its bases' 64
+vectors) keep the forms they had."""
+import numpy as np
+import pytest
+
+from oracle import products
+from paper_2103_06393_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import __graft_entry__  # noqa: E402
+
+__graft_entry__.build()
+from paper_2103_06393_gb300 import zbc  # noqa: E402
+
+RTOL = 1e-5  # what every form meets
+
+
+def _orth(rng, n, r):
+    return np.linalg.qr(rng.standard_normal((n, r)) + 1j * rng.standard_normal((n, r)))[0]
+
+
+def _c64(a):
+    return a.astype(np.complex64).astype(np.complex128)
+
+
+def _shared(n, m, R, r, seed=0, q=3, norm=1.0):
+    """m columns of q tensors of ranks r whose factors lie in common bases of R vectors a mode."""
+    rng = np.random.default_rng(seed)
+    tens = [[None] * q for _ in range(m)]
+    for k in range(q):
+        B = [_orth(rng, n[d], R[d]) for d in range(3)]
+        for j in range(m):
+            G = rng.standard_normal(r) + 1j * rng.standard_normal(r)
+            G *= norm / np.linalg.norm(G)
+            tens[j][k] = _c64(G), [_c64(B[d] @ _orth(rng, R[d], r[d])) for d in range(3)]
+    return inputs.Grid(*n, 0.001), tens
+
+
+def _rel(a, b):
+    a = a.astype(np.complex128)
+    return float(np.max(np.linalg.norm(a - b, axis=0) / np.linalg.norm(b, axis=0)))
+
+
+def _run(h, g, A, fwd, prec=None, q=3):
+    B = zbc.colmajor(q * g.nv if fwd else h.info().m, A.shape[1], torch.complex64)
+    B.fill_(float("nan"))
+    call = zbc.zbc_matvec if fwd else zbc.zbc_rmatvec
+    call(h, zbc.to_colmajor(A.astype(np.complex64)), B, zbc.AUTO if prec is None else prec)
+    zbc.zbc_product_status(h)
+    return zbc.from_colmajor(B)
+
+
+@pytest.mark.parametrize("r", [(8, 70, 6), (8, 6, 70)])
+def test_ranks_above_the_basis_keep_the_other_forms(r):
+    g, tens = _shared((12, 80, 80), 20, (12, 80, 80), r)
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    for tuned in (False, True):
+        if tuned:
+            zbc.zbc_tune(h, 9)
+        for p in (2, 9):
+            X = _c64(inputs.cn01((20, p), seed=1))
+            Phi = _c64(inputs.cn01((3 * g.nv, p), seed=2))
+            assert _rel(_run(h, g, X, True), products.matvec(tens, g.shape, X)) < RTOL
+            assert _rel(_run(h, g, Phi, False), products.rmatvec(tens, g.shape, Phi)) < RTOL
+
+
+def test_rank_above_the_product_kernels_is_refused():
+    g, tens = _shared((80, 12, 12), 4, (80, 12, 12), (70, 6, 6))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    for call in (lambda: _run(h, g, np.ones((4, 2)), True), lambda: _run(h, g, np.ones((3 * g.nv, 2)), False),
+                 lambda: zbc.zbc_tune(h, 2)):
+        with pytest.raises(zbc.ZbcError) as e:
+            call()
+        assert e.value.status == zbc.ZBC_EINVAL
