@@ -8,6 +8,7 @@
 // the bulk-copy stage pipeline of stage.cuh: warps 0 .. ntask-1 compute (one task of 32 i1 x
 // kUQ i2 each), warp ntask copies (and, in Algorithm 2, sums the warps' per-column results).
 #include <algorithm>
+#include <type_traits>
 
 #include "stage.cuh"
 
@@ -79,9 +80,10 @@ int transpose_rhs(Handle& h, const float2* X, int64_t ldx, int p, int chunk, con
 // takes about 1 us a column whatever its size, so a grid with fewer tiles than SMs is bound by that
 // chain (24^3, 64 columns, 1 right-hand side: 72 CTAs, 66 us); its columns are cut into slices of
 // `jper` (blockIdx.z / schunks), whose sums go to Y + slice * ystride and are added in order by
-// sum_slices_kernel.
+// sum_slices_kernel (SLICED: 38 us).  The kernel for whole columns is compiled without the slices: their
+// offsets cost it registers and 0.5 to 2.4 % (96^3, 256 columns, 16 right-hand sides: 6.22 against 6.07 ms).
 // ---------------------------------------------------------------------------------------------
-template <int PS, int NT>
+template <int PS, int NT, bool SLICED>
 __global__ void __launch_bounds__(32 * (NT + 1), 1)
     matvec_simt_kernel(const float2* __restrict__ cache, const CacheDesc* __restrict__ cdesc, Geo g, int q, int M,
                        StageLayout SL, int S, const float2* __restrict__ XT, int pst, int p,
@@ -92,9 +94,10 @@ __global__ void __launch_bounds__(32 * (NT + 1), 1)
   __shared__ int meta[kMaxStages];
   __shared__ volatile int abort_flag;
   const int k = blockIdx.y;
-  const int s0 = (int)(blockIdx.z % schunks) * PS, slice = blockIdx.z / schunks;
-  const int j0 = slice * jper, nj = min(M - j0, jper);
-  Y += slice * ystride;
+  const int slice = SLICED ? blockIdx.z / schunks : 0;
+  const int s0 = (SLICED ? (int)(blockIdx.z % schunks) : blockIdx.z) * PS;
+  const int j0 = SLICED ? slice * jper : 0, nj = SLICED ? min(M - j0, jper) : M;
+  if (SLICED) Y += slice * ystride;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ncw = g.ntask;
   const int B1p = (g.B1 + 1) / 2 * 2;
@@ -484,9 +487,8 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   const int S = (int)std::min<size_t>(kMaxStages, kSmemBudget / SL.stride);
   ZBC_CHECK_ARG(S >= 2, "rank %d too large for the FP32 SIMT path", R);
   const size_t sm = (size_t)S * SL.stride;
-  ZBC_TRY((set_smem_limit<matvec_simt_kernel<PS, NT>>((int)kSmemBudget)));
-  // slices of at least 8 columns while the CTAs are fewer than two waves; not where a stream capture would
-  // have to grow the workspace
+  // slices of at least 8 columns where one wave leaves SMs idle, up to two waves of CTAs; not where a
+  // stream capture would have to grow the workspace
   const int64_t ctas = (int64_t)g.ntiles() * h.q * schunks, rows = (int64_t)h.q * h.nv();
   int slices = ctas < sm_count() ? (int)std::min<int64_t>({8, h.M / 8, 2 * sm_count() / ctas}) : 1;
   if (slices > 1) {
@@ -502,9 +504,15 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   if (slices > 1) slices = ceil_div(h.M, jper);
   float2* out = slices > 1 ? (float2*)h.work_slices.ptr : Y;
   dim3 grid(g.ntiles(), h.q, schunks * std::max(1, slices));
-  matvec_simt_kernel<PS, NT><<<grid, 32 * (g.ntask + 1), sm, st>>>(h.cache->data, h.cache->d_desc, g, h.q, h.M, SL, S,
-                                                               XT, pst, p, out, slices > 1 ? rows : ldy, schunks, jper,
-                                                               rows * p, (int*)h.work_err.ptr);
+  auto launch = [&](auto sliced) -> int {
+    constexpr bool kSliced = decltype(sliced)::value;
+    ZBC_TRY((set_smem_limit<matvec_simt_kernel<PS, NT, kSliced>>((int)kSmemBudget)));
+    matvec_simt_kernel<PS, NT, kSliced><<<grid, 32 * (g.ntask + 1), sm, st>>>(
+        h.cache->data, h.cache->d_desc, g, h.q, h.M, SL, S, XT, pst, p, out, kSliced ? rows : ldy, schunks, jper,
+        rows * p, (int*)h.work_err.ptr);
+    return ZBC_OK;
+  };
+  ZBC_TRY(slices > 1 ? launch(std::true_type{}) : launch(std::false_type{}));
   count_launch();
   if (slices > 1) {
     sum_slices_kernel<<<dim3(ceil_div(rows, 256), p), 256, 0, st>>>(out, slices, rows, p, Y, ldy);
