@@ -33,6 +33,8 @@ struct JointGeo {
   int64_t Ct, Qt;         // entries of one right-hand side of T / F and of Q
 };
 
+constexpr int kJointPass = 64;  // right-hand sides that the products' workspaces hold at a time
+
 struct JointCache {
   bool usable = false;    // false: the factors share no small basis (the other forms are used)
   bool large = false;     // the products decompress more than 1e8 voxel ranks
@@ -42,6 +44,10 @@ struct JointCache {
   unsigned char* bop = nullptr;  // B1 split for the adjoint's plane product (joint_planes.cu)
   float* kscale = nullptr;       // power-of-two scales of K's columns (joint_core.cu)
   int64_t bytes = 0;
+  // workspace bytes of a product (adjoint, forward) of up to p right-hand sides: the largest of every
+  // plan up to p.  The plans of few right-hand sides cut the column sum into more slices and may take
+  // more than those of more, and a buffer that grows for them would leave a captured graph without its own.
+  size_t work[2][kJointPass + 1] = {};
 };
 
 // the plane products on the tensor cores (joint_planes.cu): Y from Q, and Q from Phi
@@ -60,8 +66,11 @@ int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, i
 
 // Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
 int build_joint(Handle& h, cudaStream_t st);
-// bytes of h.work_joint_fwd / _adj that one product of p right-hand sides uses (h.joint usable)
-size_t joint_work_bytes(const Handle& h, int p, bool fwd);
+void joint_plan_work(JointCache* jc);  // fills work from geo
+// bytes of h.work_joint_fwd / _adj that a product of p right-hand sides needs (h.joint usable)
+inline size_t joint_work_bytes(const Handle& h, int p, bool fwd) {
+  return h.joint->work[fwd][p < kJointPass ? p : kJointPass];
+}
 int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st);
 int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* out, int64_t ldo, cudaStream_t st);
 

@@ -469,6 +469,7 @@ static int build(Handle& h, JointCache* jc, cudaStream_t st) {
   ZBC_TRY(joint_core_build(g, jc->K, jc->kscale, &fits, st));
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_status(e, "reduced cores");
+  joint_plan_work(jc);
   jc->usable = fits;
   return ZBC_OK;
 }

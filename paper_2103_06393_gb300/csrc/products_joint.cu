@@ -254,8 +254,6 @@ __global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict
   }
 }
 
-constexpr int kPassRhs = 64;  // right-hand sides that the workspaces hold at a time
-
 // From this many right-hand sides on, the column sums run on the tensor cores (at least 8 a
 // pass).  160 x 160 x 128, 4096 columns: whole forward 0.92 ms in FP32 at 4 against 1.40 ms at 8, whole
 // adjoint 1.35 / 2.05 ms in FP32 at 2 / 4 against 1.37 ms at 8.
@@ -276,7 +274,7 @@ void launch_core_adj(const JointGeo& G, const float2* K, const float2* F, int p,
   count_launch();
 }
 
-// work split of ps <= kPassRhs right-hand sides
+// work split of ps <= kJointPass right-hand sides
 struct FwdPlan {
   int P, JS;              // right-hand sides per CTA, slices of the column sum
   int64_t telems, qelems;
@@ -312,12 +310,12 @@ struct AdjPlan {
 
 }  // namespace
 
-size_t joint_work_bytes(const Handle& h, int p, bool fwd) {
-  const JointGeo& G = h.joint->geo;
-  size_t b = 0;  // the last batch holds the rest of p
-  for (int ps : {std::min(p, kPassRhs), p % kPassRhs})
-    if (ps > 0) b = std::max(b, fwd ? FwdPlan(G, ps).bytes() : AdjPlan(G, ps).bytes());
-  return b;
+void joint_plan_work(JointCache* jc) {
+  jc->work[0][0] = jc->work[1][0] = 0;
+  for (int ps = 1; ps <= kJointPass; ++ps) {
+    jc->work[0][ps] = std::max(jc->work[0][ps - 1], AdjPlan(jc->geo, ps).bytes());
+    jc->work[1][ps] = std::max(jc->work[1][ps - 1], FwdPlan(jc->geo, ps).bytes());
+  }
 }
 
 int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st) {
@@ -330,8 +328,8 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
     csmax = std::max(csmax, G.Cs[k]);
     rrmax = std::max(rrmax, G.R[k][0] * G.R[k][1]);
   }
-  for (int s0 = 0; s0 < p; s0 += kPassRhs) {
-    const int ps = std::min(kPassRhs, p - s0);
+  for (int s0 = 0; s0 < p; s0 += kJointPass) {
+    const int ps = std::min(kJointPass, p - s0);
     const FwdPlan pl(G, ps);
     const int JS = pl.JS;
     float2* T = (float2*)h.work_joint_fwd.ptr;
@@ -360,8 +358,8 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
     r3 = std::max(r3, G.R[k][2]);
     rrmax = std::max(rrmax, G.R[k][0] * G.R[k][1]);
   }
-  for (int s0 = 0; s0 < p; s0 += kPassRhs) {
-    const int ps = std::min(kPassRhs, p - s0);
+  for (int s0 = 0; s0 < p; s0 += kJointPass) {
+    const int ps = std::min(kJointPass, p - s0);
     const AdjPlan pl(G, ps);
     const int chunk = pl.chunk, splits = pl.splits;
     float2* Q = (float2*)h.work_joint_adj.ptr;

@@ -473,6 +473,28 @@ int reduce_partials(const float2* partial, int ng, int M, int p, float2* out, in
 // ---------------------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------------------
+// Slices of a sum over the stored columns: at least 8 columns each, where one wave of the `ctas` whole-column
+// CTAs leaves SMs idle, up to two waves
+static int forward_slices(const Handle& h, int64_t ctas) {
+  return ctas < sm_count() ? (int)std::min<int64_t>({8, h.M / 8, 2 * sm_count() / ctas}) : 1;
+}
+
+// Bytes of h.work_slices: the largest of every forward of up to p right-hand sides, with either CTA shape.
+// Fewer right-hand sides can take more (24^3, 64 columns: 4 slices of 16, but 2 of 17), and a buffer that
+// grows for them would leave a captured graph without its own.
+static size_t slices_bytes(const Handle& h, int p) {
+  size_t most = 0;
+  for (int nt : {6, 9}) {
+    const int64_t ctas = (int64_t)make_geo(h.n1, h.n2, h.n3, 0, nt).ntiles() * h.q;
+    for (int c = 1; c <= ceil_div(p, 16); ++c) {  // chunks of at most 16 right-hand sides share CTAs
+      const int slices = forward_slices(h, ctas * c);
+      if (slices <= 1) break;
+      most = std::max(most, sizeof(float2) * (size_t)slices * h.q * h.nv() * std::min(p, 16 * c));
+    }
+  }
+  return most;
+}
+
 template <int PS, int NT>
 static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st) {
   ZBC_TRY(build_decomp_cache(h, st));
@@ -487,16 +509,14 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   const int S = (int)std::min<size_t>(kMaxStages, kSmemBudget / SL.stride);
   ZBC_CHECK_ARG(S >= 2, "rank %d too large for the FP32 SIMT path", R);
   const size_t sm = (size_t)S * SL.stride;
-  // slices of at least 8 columns where one wave leaves SMs idle, up to two waves of CTAs; not where a
-  // stream capture would have to grow the workspace
-  const int64_t ctas = (int64_t)g.ntiles() * h.q * schunks, rows = (int64_t)h.q * h.nv();
-  int slices = ctas < sm_count() ? (int)std::min<int64_t>({8, h.M / 8, 2 * sm_count() / ctas}) : 1;
-  if (slices > 1) {
+  const int64_t rows = (int64_t)h.q * h.nv();
+  int slices = forward_slices(h, (int64_t)g.ntiles() * h.q * schunks);
+  if (slices > 1) {  // not where a stream capture would have to grow the workspace
     const size_t bytes = sizeof(float2) * (size_t)slices * rows * p;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (h.work_slices.bytes < bytes) ZBC_TRY_CUDA(cudaStreamIsCapturing(st, &cap));
     if (cap == cudaStreamCaptureStatusNone)
-      ZBC_TRY(h.work_slices.ensure(bytes));
+      ZBC_TRY(h.work_slices.ensure(slices_bytes(h, p)));
     else
       slices = 1;
   }

@@ -1,5 +1,5 @@
 """ZBC_AUTO at the edges of the joint form: handles that cannot take it (ranks above its bases' 64
-vectors) keep the forms they had."""
+vectors) keep the forms they had, and its workspaces (and the FP32 forward's) keep their place."""
 import numpy as np
 import pytest
 
@@ -77,3 +77,19 @@ def test_rank_above_the_product_kernels_is_refused():
         with pytest.raises(zbc.ZbcError) as e:
             call()
         assert e.value.status == zbc.ZBC_EINVAL
+
+
+@pytest.mark.parametrize("form,sizes", [("fp32", (17, 32)), ("auto", (5, 17, 33, 64, 66))])
+def test_a_smaller_product_keeps_the_buffers_of_a_larger_one(form, sizes):
+    """A captured graph holds the buffers of its call: no call of fewer right-hand sides moves them."""
+    prec = zbc.FP32_SIMT if form == "fp32" else zbc.AUTO
+    g, tens = _shared((24, 24, 24), 130, (12, 12, 12), (6, 6, 6))
+    for first in sizes:
+        h = zbc.zbc_create_from_host(g, 3, tens)
+        for fwd in (True, False):
+            _run(h, g, np.ones((130 if fwd else 3 * g.nv, first)), fwd, prec)
+        work = h.device_bytes()["work"]
+        for p in range(first, 0, -1):
+            for fwd in (True, False):
+                _run(h, g, np.ones((130 if fwd else 3 * g.nv, p)), fwd, prec)
+            assert h.device_bytes()["work"] == work, (first, p)
