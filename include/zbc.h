@@ -83,7 +83,10 @@ typedef enum { ZBC_C64 = 0, ZBC_C128 = 1 } zbc_dtype;
  *             rounding of its complex64 factors), Z_j = K_j x1 B_1 x2 B_2 x3 B_3 with cores K_j in
  *             the bases, and the products sum over the columns' cores and pass between the cores
  *             and the grid once per right-hand side.  The bases and cores are built on the first
- *             AUTO or zbc_tune call (not during a stream capture) and kept with the handle. */
+ *             AUTO or zbc_tune call (not during a stream capture) and kept with the handle, after the
+ *             decompression cache and if they take at most half of the device memory then free;
+ *             otherwise, and where a call's workspace does not fit, AUTO runs the other forms
+ *             (zbc_tune looks again). */
 typedef enum {
   ZBC_FP32_SIMT = 0,
   ZBC_TF32X3 = 1,

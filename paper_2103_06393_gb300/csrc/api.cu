@@ -26,6 +26,7 @@ int DevBuf::ensure(size_t need) {
   size_t b = need < 256 ? 256 : need;
   cudaError_t e = cudaMalloc(&ptr, b);
   if (e != cudaSuccess) {
+    cudaGetLastError();  // callers that do without the buffer launch next: leave no error behind
     ptr = nullptr;
     bytes = 0;
     set_error("cudaMalloc(%zu) failed: %s", b, cudaGetErrorString(e));

@@ -112,6 +112,7 @@ int build_decomp_cache(Handle& h, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMalloc(&c->d_desc, sizeof(CacheDesc) * T);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_desc, cd.data(), sizeof(CacheDesc) * T, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     cache_release(c);
     set_error("decompression cache allocation failed: %s", cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? ZBC_ENOMEM : ZBC_ECUDA;

@@ -413,13 +413,18 @@ static int build(Handle& h, JointCache* jc, cudaStream_t st) {
   // under half of W, less than the operands that tuning would otherwise leave
   jc->large = direct > 1e8;
   if (work > 0.5 * direct || 8.0 * kelems > (jc->large ? 2.0 : 0.5) * wbytes) return ZBC_OK;
+  // and at most half of what the device has free (W is built): the other forms' operands and the
+  // workspaces of later calls have to fit beside it
+  size_t mem_free = 0, mem_total = 0;
+  ZBC_TRY_CUDA(cudaMemGetInfo(&mem_free, &mem_total));
+  if (sizeof(float2) * (size_t)kelems > mem_free / 2) return ZBC_ENOMEM;
   cudaError_t e = cudaMalloc(&jc->basis, sizeof(float2) * belems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->K, sizeof(float2) * kelems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->bop, joint_planes_bytes(g));
   if (e == cudaSuccess) e = cudaMalloc(&jc->kscale, joint_core_bytes(g));
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return ZBC_OK;  // no room: unusable
+    return cuda_status(e, "allocation");
   }
   jc->bytes = (int64_t)(sizeof(float2) * (belems + kelems) + joint_planes_bytes(g) + joint_core_bytes(g));
   for (int k = 0; k < q; ++k)
@@ -478,6 +483,7 @@ int build_joint(Handle& h, cudaStream_t st) {
   if (h.joint) return ZBC_OK;
   h.joint = new JointCache();  // kept also when unusable, so that the search is not repeated
   const int s = build(h, h.joint, st);
+  h.joint->no_room = s == ZBC_ENOMEM;
   if (!h.joint->usable) free_operands(h.joint);
   return s;
 }

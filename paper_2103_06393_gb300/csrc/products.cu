@@ -19,7 +19,9 @@ int aca_post(const Handle& h, const float2* Psip, int p, float2* Psi, int64_t ld
 // The joint-subspace form (joint.cuh): chosen by ZBC_AUTO only, so it has no zbc_precision of its own.
 constexpr zbc_precision kFormJoint = (zbc_precision)7;
 
-// Whether ZBC_AUTO can run the joint form: the basis is built on the first call that asks for it.
+// Whether ZBC_AUTO can run the joint form: the basis is built on the first call that asks for it, after
+// the decompression cache that every form needs (on a device with room for one of the two, the products
+// stay possible), and its workspace is taken here, so that a call without room for it runs another form.
 // During a stream capture nothing is built or grown; the other forms then run as they did.
 static bool joint_ready(Handle& h, int p, bool fwd, cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -29,11 +31,15 @@ static bool joint_ready(Handle& h, int p, bool fwd, cudaStream_t st) {
   }
   if (cap != cudaStreamCaptureStatusNone)
     return h.joint && h.joint->usable && (fwd ? h.work_joint_fwd : h.work_joint_adj).bytes >= joint_work_bytes(h, p, fwd);
-  if (!h.joint && build_joint(h, st) != ZBC_OK) {
+  int s = build_decomp_cache(h, st);
+  if (s == ZBC_OK) s = build_joint(h, st);
+  if (s == ZBC_OK && h.joint->usable)
+    s = (fwd ? h.work_joint_fwd : h.work_joint_adj).ensure(joint_work_bytes(h, p, fwd));
+  if (s != ZBC_OK) {
     clear_error();
     cudaGetLastError();
   }
-  return h.joint && h.joint->usable;
+  return s == ZBC_OK && h.joint->usable;
 }
 
 // The form of ZBC_AUTO: the tuned one; untuned, the joint form where the handle has it, else BF16X3
@@ -164,6 +170,10 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
   Handle& h = hh->h;
   const cudaStream_t st = (cudaStream_t)stream;
   const int64_t rows = (int64_t)h.q * h.nv();
+  if (h.joint && h.joint->no_room) {
+    joint_release(h.joint);
+    h.joint = nullptr;
+  }
   DevBuf X, Y, Phi, Psi;
   ZBC_TRY(X.ensure(sizeof(float2) * (size_t)h.m * p));
   ZBC_TRY(Psi.ensure(sizeof(float2) * (size_t)h.m * p));
@@ -201,6 +211,7 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
     t[i] = INFINITY;
     if ((v.prec == kFormJoint && !joint_ready(h, p, v.fwd, st)) || run() != ZBC_OK) {  // a form that does not fit this handle is skipped
       clear_error();
+      cudaGetLastError();
       continue;
     }
     float sum = 0.f;

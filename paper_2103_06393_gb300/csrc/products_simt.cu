@@ -511,14 +511,16 @@ static int launch_matvec(Handle& h, const float2* X, int64_t ldx, int p, float2*
   const size_t sm = (size_t)S * SL.stride;
   const int64_t rows = (int64_t)h.q * h.nv();
   int slices = forward_slices(h, (int64_t)g.ntiles() * h.q * schunks);
-  if (slices > 1) {  // not where a stream capture would have to grow the workspace
+  if (slices > 1) {  // not where the workspace does not fit, or a stream capture would have to grow it
     const size_t bytes = sizeof(float2) * (size_t)slices * rows * p;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (h.work_slices.bytes < bytes) ZBC_TRY_CUDA(cudaStreamIsCapturing(st, &cap));
-    if (cap == cudaStreamCaptureStatusNone)
-      ZBC_TRY(h.work_slices.ensure(slices_bytes(h, p)));
-    else
+    if (cap != cudaStreamCaptureStatusNone) {
       slices = 1;
+    } else if (h.work_slices.ensure(slices_bytes(h, p)) != ZBC_OK) {
+      clear_error();
+      slices = 1;
+    }
   }
   const int jper = slices > 1 ? ceil_div(h.M, slices) : h.M;
   if (slices > 1) slices = ceil_div(h.M, jper);

@@ -1,5 +1,6 @@
 """ZBC_AUTO at the edges of the joint form: handles that cannot take it (ranks above its bases' 64
-vectors) keep the forms they had, and its workspaces (and the FP32 forward's) keep their place."""
+vectors) keep the forms they had, its workspaces (and the FP32 forward's) keep their place, and a device
+without room for it still runs the products."""
 import numpy as np
 import pytest
 
@@ -93,3 +94,62 @@ def test_a_smaller_product_keeps_the_buffers_of_a_larger_one(form, sizes):
             for fwd in (True, False):
                 _run(h, g, np.ones((130 if fwd else 3 * g.nv, p)), fwd, prec)
             assert h.device_bytes()["work"] == work, (first, p)
+
+
+def _filled(leave):
+    """All but `leave` bytes of the free device memory."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("first", ["matvec", "rmatvec", "tune"])
+def test_products_without_room_for_the_reduced_cores(first):
+    """Room for the decompression cache, but not for it and the joint form's cores (0.5 GB each)."""
+    g, tens = _shared((96, 96, 96), 256, (44, 44, 44), (8, 8, 8))
+    h, free = (zbc.zbc_create_from_host(g, 3, tens) for _ in range(2))
+    X = zbc.to_colmajor(inputs.cn01((256, 2), seed=1).astype(np.complex64))
+    Phi = zbc.to_colmajor(inputs.cn01((3 * g.nv, 2), seed=2).astype(np.complex64))
+    Y, Psi = zbc.colmajor(3 * g.nv, 2, torch.complex64), zbc.colmajor(256, 2, torch.complex64)
+    zbc.zbc_matvec(free, X, Y, zbc.FP32_SIMT)
+    zbc.zbc_rmatvec(free, Phi, Psi, zbc.FP32_SIMT)
+    want = Y.clone(), Psi.clone()
+    W = free.device_bytes()["caches"]
+    del free
+    fill = _filled(W + (400 << 20))
+    try:
+        if first == "matvec":
+            zbc.zbc_matvec(h, X, Y, zbc.AUTO)
+        elif first == "rmatvec":
+            zbc.zbc_rmatvec(h, Phi, Psi, zbc.AUTO)
+        else:
+            zbc.zbc_tune(h, 2)
+        for prec in (zbc.AUTO, zbc.FP32_SIMT):
+            zbc.zbc_matvec(h, X, Y, prec)
+            zbc.zbc_rmatvec(h, Phi, Psi, prec)
+            zbc.zbc_product_status(h)
+            for got, ref in ((Y, want[0]), (Psi, want[1])):
+                assert torch.linalg.norm(got - ref) < RTOL * torch.linalg.norm(ref)
+        assert torch.equal(Y, want[0])
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    zbc.zbc_tune(h, 2)  # with the memory back, the joint form gets its cores
+    assert h.device_bytes()["caches"] > W + (400 << 20)
+
+
+def test_products_without_room_for_the_joint_workspace():
+    g, tens = _shared((96, 96, 96), 256, (44, 44, 44), (8, 8, 8))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    A = [zbc.to_colmajor(inputs.cn01((256, p), seed=p).astype(np.complex64)) for p in (1, 2)]
+    Y = [zbc.colmajor(3 * g.nv, p, torch.complex64) for p in (1, 2, 2)]
+    zbc.zbc_matvec(h, A[1], Y[2], zbc.FP32_SIMT)
+    zbc.zbc_matvec(h, A[0], Y[0], zbc.AUTO)  # the basis, and a workspace for one right-hand side
+    fill = _filled(6 << 20)
+    try:
+        zbc.zbc_matvec(h, A[1], Y[1], zbc.AUTO)
+        zbc.zbc_product_status(h)
+        assert torch.equal(Y[1], Y[2])
+    finally:
+        del fill
+        torch.cuda.empty_cache()
