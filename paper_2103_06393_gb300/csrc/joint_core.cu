@@ -13,10 +13,13 @@
 // registers with the chunk's scales while the next chunk is converted, so that a tensor-core sum has
 // 64 terms.
 //
-// Scales: K per column j (kscale[j] = 2^(15 - e_j), |K[j]| < 2^e_j, from the build; fp16 hi + lo then
-// leave 2^-40 of a column's largest entry); the forward's X by 2^(e_j - e), e the component's largest
-// e_j; the right-hand sides' entries per chunk.  Scales of K's rows taken anew in every chunk of the
-// adjoint cost a fifth of its issue slots (0.61 ms at 96^3, 16 right-hand sides).
+// Scales: K per column j (kscale[j] = 2^(15 - e_j), |K[j]| < 2^e_j, from the build; fp16 hi + lo leave
+// an error of max(2^-23 |K|, 2^-40 2^e_j)); the forward's X by 2^(e_j - e), e the component's largest
+// e_j; the right-hand sides' entries per chunk.  Each chunk enters the FP32 sums with all scales but
+// 2^(e_j - e) taken out, so that these overflow where the product would and not before; an X entry takes
+// its own power of two first, so that a small one against a small column keeps its bits.  Scales of K's rows
+// taken anew in every chunk of the adjoint cost a fifth of its issue slots (0.61 ms at 96^3, 16 right-hand
+// sides).
 #include <algorithm>
 
 #include "joint_tc.cuh"
@@ -44,7 +47,7 @@ __global__ void __launch_bounds__(288, 2)
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t done[2], ready[2];
   __shared__ uint32_t tmem_base;
-  __shared__ float bscale[4][P];            // 2^(e - kDataShift) of a chunk's right-hand sides
+  __shared__ float bscale[4][P];            // scales that a chunk's sums still carry, per right-hand side
   unsigned char* sa = smem;                 // [2 buffers][2 terms][128 rows][128 B]
   unsigned char* sb = sa + 4 * kRowTerm;    // [2 buffers][2 terms][N rows][128 B]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__(288, 2)
     for (int item = 0; item < items; ++item, c0 += per) {
       const int k = fk, row = fpos;
       const float* ks = kscale + (int64_t)k * 2 * Mp;
+      const int ke = log2_of(__ldg(kscale + (int64_t)G.q * 2 * Mp + k));  // e - 15
       float acc[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) acc[i] = 0.f;
@@ -185,6 +189,15 @@ __global__ void __launch_bounds__(288, 2)
       for (int ch = 0; ch < per; ++ch) {
         const int c = c0 + ch, d = c & 1;
         if (ch >= 2) fold(c - 2);  // also: the MMAs have read this buffer
+        const float xs = FWD ? __ldg(ks + Mp + ch * kSum + lane) : 1.f;  // 2^(e_j - e)
+        int be[I];  // xs |b| < 2^be, so that 2^(kDataShift - be) b is below 2^kDataShift / xs: finite
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+          const float m = absmax_nan(0.f, b[i].x, b[i].y);
+          if (FWD) bad = bad || !(m < INFINITY);
+          be[i] = exp_of(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(FWD ? m * xs : m))), -117);
+          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2_wide(be[i] - kDataShift + ke);
+        }
         unsigned char* ad = sa + (size_t)d * 2 * kRowTerm;
         if (FWD) {
           const int r = 32 * q4 + lane;
@@ -214,23 +227,12 @@ __global__ void __launch_bounds__(288, 2)
         }
         // the right-hand sides' rows (two a right-hand side): pair `lane` of the chunk in the rows' order
         const uint32_t kc = FWD ? lane / 4 : lane % 16 / 2, word = FWD ? lane % 4 : lane % 2 + lane / 16 * 2;
-        float xs = 1.f;  // 2^(e_j - e)
-        if (FWD) xs = __ldg(ks + Mp + ch * kSum + lane);
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-          float2 v = b[i];
-          if (FWD) {
-            bad = bad || !(absmax_nan(0.f, v.x, v.y) < INFINITY);
-            v.x *= xs;
-            v.y *= xs;
-          }
-          float m = absmax_nan(0.f, v.x, v.y);
-          for (int o = 16; o > 0; o >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
-          const int e = exp_of(m), n = 2 * (warp + 8 * i);
-          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2f(e - kDataShift);
-          const float sc = pow2f(kDataShift - e);
+          const int n = 2 * (warp + 8 * i);
+          const float sc = pow2f(kDataShift - be[i]);
           uint32_t h, l;
-          split2(v.x * sc, v.y * sc, h, l);
+          split2(FWD ? b[i].x * sc * xs : b[i].x * sc, FWD ? b[i].y * sc * xs : b[i].y * sc, h, l);
           const uint32_t hs = __byte_perm(h, 0, 0x1032), ls = __byte_perm(l, 0, 0x1032);
           unsigned char* o0 = sb + (size_t)d * 2 * kBTerm + tc::sw128_off(n, kc) + 4 * word;
           unsigned char* o1 = sb + (size_t)d * 2 * kBTerm + tc::sw128_off(n + 1, kc) + 4 * word;
@@ -253,17 +255,15 @@ __global__ void __launch_bounds__(288, 2)
       fold(c0 + per - 1);
       const int r = 32 * q4 + lane;
       if (FWD) {
-        // K was scaled by 2^(15 - e_j) and X by 2^(e_j - e): 2^(e - 15) is left
-        const float ko = __ldg(kscale + (int64_t)G.q * 2 * Mp + k);
         if (row + r < G.Cs[k])
 #pragma unroll
           for (int i = 0; i < P / 2; ++i) {
             const int s = s0 + half * (P / 2) + i;
-            if (s < p) out[(int64_t)s * G.Ct + G.toff[k] + row + r] = make_float2(acc[2 * i] * ko, acc[2 * i + 1] * ko);
+            if (s < p) out[(int64_t)s * G.Ct + G.toff[k] + row + r] = make_float2(acc[2 * i], acc[2 * i + 1]);
           }
       } else {
         const int j = blockIdx.y * kRows + r;
-        const float kj = j < G.M ? 1.f / __ldg(ks + j) : 0.f;  // 2^(e_j - 15)
+        const float kj = j < G.M ? __ldg(ks + Mp + j) : 0.f;  // 2^(e_j - e)
         if (j < G.M)
 #pragma unroll
           for (int i = 0; i < P / 2; ++i) {
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(128) core_exp_kernel(const __grid_constant__ J
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 4; ++w) m = max_nan(m, red[w]);
-    kscale[(int64_t)k * 2 * Mp + j] = m > 0.f ? (float)exp_of(m) : -1000.f;  // no entries: takes the largest e
+    kscale[(int64_t)k * 2 * Mp + j] = m > 0.f ? (float)exp_of(m, -106) : -1000.f;  // no entries: takes the largest e
   }
 }
 // the scales from the exponents: kscale[k][0][j] = 2^(15 - e_j), kscale[k][1][j] = 2^(e_j - e), and

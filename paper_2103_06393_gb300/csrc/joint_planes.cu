@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       asm volatile("bar.sync 1, 512;" ::: "memory");
 #pragma unroll
       for (int w = 0; w < kFwdWorkers / 32; ++w) m = max_nan(m, wmax[t & 1][w]);
-      const int e = exp_of(m, -117);  // 2^(kDataShift - e) stays finite; Y takes 2^-21 and 2^e in turn
+      const int e = exp_of(m, -117);  // 2^(kDataShift - e) stays finite; Y takes 2^-20 and 2^(e - 1) in turn
       const float sc = pow2f(kDataShift - e);
 #pragma unroll
       for (int u = 0; u < kQRegs; ++u)
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         }
       }
       if (t < lag) continue;
-      const float us = pow2f(eout);
+      const float us = pow2f(eout - 1);
       const int pl = (int)blockIdx.x + (t - lag) * (int)gridDim.x, s = pl / G.n3, i3 = pl - s * G.n3;
       float2* Yp = Y + ldy * s + (int64_t)k * ((int64_t)G.n1 * G.n2 * G.n3) +
                    (int64_t)G.n1 * (i20 + (int64_t)G.n2 * i3) + row0;
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             float2* y = y0 + (int64_t)G.n1 * 8 * c;
 #pragma unroll
             for (int w = 0; w < 8; ++w, y += G.n1)
-              if (live && 8 * c + w < left) __stcs(y, make_float2(v[2 * w] * 0x1p-21f * us, v[2 * w + 1] * 0x1p-21f * us));
+              if (live && 8 * c + w < left) __stcs(y, make_float2(v[2 * w] * 0x1p-20f * us, v[2 * w + 1] * 0x1p-20f * us));
           }
         }
         tc::fence_before();
@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
         wait(&done[d], (c >> 1) & 1);
         tc::fence_after();
         if (32 * q4 < rows) {
-          const float us = pow2f(rexp[c & 3][32 * q4 + lane] - kDataShift - kBasisShift);
+          const float us = pow2f(rexp[c & 3][32 * q4 + lane] - 2) * pow2f(2 - kDataShift - kBasisShift);
           const uint32_t t0 = tmem + (uint32_t)(d * N + half * NC) + ((uint32_t)(32 * q4) << 16);
 #pragma unroll
           for (int i = 0; i < I; ++i) {
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
           m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
           m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
           bad = bad || !(m < INFINITY);
-          const int e = exp_of(m), r = row0 + 32 * u;
+          const int e = exp_of(m, -117), r = row0 + 32 * u;  // 2^(kDataShift - e) stays finite
           if (c8 == 0) rexp[c & 3][r] = e;
           const float sc = pow2f(kDataShift - e);
           uint32_t h[4], l[4];

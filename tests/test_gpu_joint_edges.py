@@ -1,6 +1,7 @@
 """ZBC_AUTO at the edges of the joint form: handles that cannot take it (ranks above its bases' 64
-vectors) keep the forms they had, its workspaces (and the FP32 forward's) keep their place, and a device
-without room for it still runs the products."""
+vectors) keep the forms they had, its workspaces (and the FP32 forward's) keep their place, a device
+without room for it still runs the products, and vectors and columns of any size FP32 holds (the column
+sums run in FP32 up to 4 / 2 right-hand sides, forward / adjoint, and on the tensor cores from there on)."""
 import numpy as np
 import pytest
 
@@ -153,3 +154,45 @@ def test_products_without_room_for_the_joint_workspace():
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("p", [2, 6, 17])
+@pytest.mark.parametrize("scale,norm", [(1e-36, 1.0), (1.0, 1e-8), (1e35, 1e-8)])
+def test_scaled_vectors(p, scale, norm):
+    g, tens = _shared((40, 36, 20), 48, (12, 11, 10), (6, 5, 4), norm=norm)
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    X = _c64(inputs.cn01((48, p), seed=1) * scale)
+    Phi = _c64(inputs.cn01((3 * g.nv, p), seed=2) * scale)
+    assert _rel(_run(h, g, X, True), products.matvec(tens, g.shape, X)) < RTOL
+    assert _rel(_run(h, g, Phi, False), products.rmatvec(tens, g.shape, Phi)) < RTOL
+
+
+@pytest.mark.parametrize("p", [2, 6, 17])
+def test_small_column_against_a_small_entry(p):
+    """A column of 1e-18 times the others' norm, alone in X with an entry of 1e-21."""
+    g, tens = _shared((40, 36, 20), 48, (12, 11, 10), (6, 5, 4), norm=1e8)
+    tens[7] = [(_c64(G * 1e-18), U) for G, U in tens[7]]
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    X = np.zeros((48, p), np.complex128)
+    X[7] = _c64(inputs.cn01((p,), seed=1) * 1e-21)
+    Phi = _c64(inputs.cn01((3 * g.nv, p), seed=2))
+    assert _rel(_run(h, g, X, True), products.matvec(tens, g.shape, X)) < RTOL
+    Psi, ref = _run(h, g, Phi, False), products.rmatvec(tens, g.shape, Phi)
+    assert _rel(Psi, ref) < RTOL and _rel(Psi[7:8].T, ref[7:8].T) < RTOL
+
+
+@pytest.mark.parametrize("p", [2, 6, 17])
+def test_nan_is_reported_and_stays_in_its_column(p):
+    g, tens = _shared((40, 36, 20), 48, (12, 11, 10), (6, 5, 4))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    for fwd in (True, False):
+        A = zbc.colmajor(48 if fwd else 3 * g.nv, p, torch.complex64)
+        B = zbc.colmajor(3 * g.nv if fwd else 48, p, torch.complex64)
+        A.fill_(1.0)
+        A[1, 11] = float("nan")
+        (zbc.zbc_matvec if fwd else zbc.zbc_rmatvec)(h, A, B, zbc.AUTO)
+        with pytest.raises(zbc.ZbcError) as e:
+            zbc.zbc_product_status(h)
+        assert e.value.status == zbc.ZBC_ENAN
+        ok = torch.isfinite(torch.view_as_real(B)).flatten(1)
+        assert not ok[1].any() and ok[0].all() and ok[2:].all()
