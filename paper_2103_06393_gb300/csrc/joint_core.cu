@@ -28,6 +28,8 @@ namespace zbc {
 namespace {
 
 constexpr int kRows = 128, kSum = 32;
+constexpr int kFold = 32;  // chunks of the adjoint per FP32 chain: one over a slice's 300 chunks (96^3) made
+                           // more than half of its error
 constexpr uint32_t kRowTerm = kRows * 128u;  // one term of K's chunk
 
 __host__ __device__ inline int slices_of(int Cs, int split) { return ((Cs + kSum - 1) / kSum + split - 1) / split; }
@@ -43,7 +45,7 @@ __global__ void __launch_bounds__(288, 2)
                       const float2* __restrict__ R, int64_t ldr, int p, int split, float2* __restrict__ out,
                       int* __restrict__ err) {
   constexpr int N = 2 * P, I = P / 8;
-  constexpr uint32_t kBTerm = N * 128u, ncols = 2 * N < 32 ? 32 : 2 * N;
+  constexpr uint32_t kBTerm = N * 128u, ncols = FWD ? 2 * N : 4 * N;  // two accumulators, the adjoint's sums
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t done[2], ready[2];
   __shared__ uint32_t tmem_base;
@@ -92,8 +94,10 @@ __global__ void __launch_bounds__(288, 2)
           const uint64_t bh = tc::smem_desc_sw128(b0 + ks * 32), bl = tc::smem_desc_sw128(b0 + kBTerm + ks * 32);
           tc::mma<0>(tmem + d * N, al, bh, id, ks > 0);
           tc::mma<0>(tmem + d * N, ah, bl, id, 1);
-          tc::mma<0>(tmem + d * N, ah, bh, id, 1);
         }
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          tc::mma<0>(tmem + d * N, tc::smem_desc_sw128(a0 + ks * 32), tc::smem_desc_sw128(b0 + ks * 32), id, 1);
         tc::commit(&done[d]);
       }
     }
@@ -186,9 +190,26 @@ __global__ void __launch_bounds__(288, 2)
         }
         tc::fence_before();
       };
+      // adjoint: the sums so far wait in tensor memory, after the two accumulators (each thread its own)
+      auto put_by = [&](bool first) {
+        const uint32_t t0 = tmem + (uint32_t)(2 * N + half * P) + ((uint32_t)(32 * q4) << 16);
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+          uint32_t r[8];
+          if (!first) tmem_ld8(t0 + 8 * i, r);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            r[u] = __float_as_uint(first ? acc[8 * i + u] : acc[8 * i + u] + __uint_as_float(r[u]));
+            acc[8 * i + u] = 0.f;
+          }
+          tmem_st8(t0 + 8 * i, r);
+        }
+        tc::tmem_wait_st();
+      };
       for (int ch = 0; ch < per; ++ch) {
         const int c = c0 + ch, d = c & 1;
         if (ch >= 2) fold(c - 2);  // also: the MMAs have read this buffer
+        if (!FWD && ch % kFold == kFold - 1) put_by(ch < kFold);
         const float xs = FWD ? __ldg(ks + Mp + ch * kSum + lane) : 1.f;  // 2^(e_j - e)
         int be[I];  // xs |b| < 2^be, so that 2^(kDataShift - be) b is below 2^kDataShift / xs: finite
 #pragma unroll
@@ -196,7 +217,7 @@ __global__ void __launch_bounds__(288, 2)
           const float m = absmax_nan(0.f, b[i].x, b[i].y);
           if (FWD) bad = bad || !(m < INFINITY);
           be[i] = exp_of(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(FWD ? m * xs : m))), -117);
-          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2_wide(be[i] - kDataShift + ke);
+          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2_wide(be[i] - kDataShift + ke) * lo_first_gain(4);
         }
         unsigned char* ad = sa + (size_t)d * 2 * kRowTerm;
         if (FWD) {
@@ -262,6 +283,16 @@ __global__ void __launch_bounds__(288, 2)
             if (s < p) out[(int64_t)s * G.Ct + G.toff[k] + row + r] = make_float2(acc[2 * i], acc[2 * i + 1]);
           }
       } else {
+        if (per >= kFold) {
+          const uint32_t t0 = tmem + (uint32_t)(2 * N + half * P) + ((uint32_t)(32 * q4) << 16);
+#pragma unroll
+          for (int i = 0; i < I; ++i) {
+            uint32_t v[8];
+            tmem_ld8(t0 + 8 * i, v);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc[8 * i + u] += __uint_as_float(v[u]);
+          }
+        }
         const int j = blockIdx.y * kRows + r;
         const float kj = j < G.M ? __ldg(ks + Mp + j) : 0.f;  // 2^(e_j - e)
         if (j < G.M)

@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     __syncwarp();
   } else {
     const int q4 = warp & 3, grp = warp >> 2;  // accumulator rows; the groups share its columns
+    const float gain = mixed_gain(KB1 / 2, KB / 2);
     const float2* Qk = Q + G.qoff[k];
     float2 qr[kQRegs];
     uint32_t qoff[kQRegs];  // of the pair (x, y) in row 2 x; row 2 x + 1 lies 16 bytes further
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         }
       }
       if (t < lag) continue;
-      const float us = pow2f(eout - 1);
+      const float us = pow2f(eout - 1) * gain;
       const int pl = (int)blockIdx.x + (t - lag) * (int)gridDim.x, s = pl / G.n3, i3 = pl - s * G.n3;
       float2* Yp = Y + ldy * s + (int64_t)k * ((int64_t)G.n1 * G.n2 * G.n3) +
                    (int64_t)G.n1 * (i20 + (int64_t)G.n2 * i3) + row0;
@@ -360,8 +361,10 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
           const uint64_t bh = tc::smem_desc_sw128(b0 + ks * 32), bl = tc::smem_desc_sw128(b0 + kBTerm + ks * 32);
           tc::mma<0>(tmem + d * N, al, bh, id, ks > 0);
           tc::mma<0>(tmem + d * N, ah, bl, id, 1);
-          tc::mma<0>(tmem + d * N, ah, bh, id, 1);
         }
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          tc::mma<0>(tmem + d * N, tc::smem_desc_sw128(a0 + ks * 32), tc::smem_desc_sw128(b0 + ks * 32), id, 1);
         tc::commit(&done[d]);
       }
       // after giving up: the copies in flight land before the buffers are left
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
         wait(&done[d], (c >> 1) & 1);
         tc::fence_after();
         if (32 * q4 < rows) {
-          const float us = pow2f(rexp[c & 3][32 * q4 + lane] - 2) * pow2f(2 - kDataShift - kBasisShift);
+          const float us = pow2f(rexp[c & 3][32 * q4 + lane] - 2) * (pow2f(2 - kDataShift - kBasisShift) * lo_first_gain(4));
           const uint32_t t0 = tmem + (uint32_t)(d * N + half * NC) + ((uint32_t)(32 * q4) << 16);
 #pragma unroll
           for (int i = 0; i < I; ++i) {
@@ -482,6 +485,11 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
         for (int e = 0; e < kStage2 * R2p / 512; ++e)
           ((float4*)b2s)[tid + 256 * e] = __ldg(bsrc + j0 * R2p / 2 + tid + 256 * e);
         worker_barrier();
+        float2 qs[RC][RC];  // the stage's sums: chains of 32 terms
+#pragma unroll
+        for (int a = 0; a < RC; ++a)
+#pragma unroll
+          for (int b = 0; b < RC; ++b) qs[a][b] = make_float2(0.f, 0.f);
 #pragma unroll 2
         for (int j = 0; j < kStage2; j += 2) {
           float4 v[RC];
@@ -495,11 +503,18 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
             const float2 e0 = b2s[j * R2p + tx + 16 * b], e1 = b2s[(j + 1) * R2p + tx + 16 * b];
 #pragma unroll
             for (int a = 0; a < RC; ++a) {
-              qa[a][b] = cfma_conj(e0, make_float2(v[a].x, v[a].y), qa[a][b]);
-              qa[a][b] = cfma_conj(e1, make_float2(v[a].z, v[a].w), qa[a][b]);
+              qs[a][b] = cfma_conj(e0, make_float2(v[a].x, v[a].y), qs[a][b]);
+              qs[a][b] = cfma_conj(e1, make_float2(v[a].z, v[a].w), qs[a][b]);
             }
           }
         }
+#pragma unroll
+        for (int a = 0; a < RC; ++a)
+#pragma unroll
+          for (int b = 0; b < RC; ++b) {
+            qa[a][b].x += qs[a][b].x;
+            qa[a][b].y += qs[a][b].y;
+          }
       }
       worker_barrier();  // V is read before the next item overwrites the buffers
       if (t2 == nt2 - 1) {

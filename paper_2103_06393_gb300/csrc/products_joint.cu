@@ -17,6 +17,7 @@ namespace zbc {
 namespace {
 
 constexpr int kJc = 64;  // columns of X per shared-memory chunk of the forward core sum
+constexpr int kJf = 32;  // and per FP32 chain
 
 __device__ __forceinline__ bool finite2(float2 v) { return isfinite(v.x) && isfinite(v.y); }
 
@@ -35,9 +36,9 @@ __global__ void __launch_bounds__(128) joint_core_fwd_kernel(const __grid_consta
   const int j0 = blockIdx.y * per, j1 = min(G.M, j0 + per);
   const int64_t cs = G.Cs[k];
   const float2* Kp = K + G.koff[k] + (live ? c : 0);
-  float2 acc[2][P];
+  float2 sum[2][P];
 #pragma unroll
-  for (int s = 0; s < P; ++s) acc[0][s] = acc[1][s] = make_float2(0.f, 0.f);
+  for (int s = 0; s < P; ++s) sum[0][s] = sum[1][s] = make_float2(0.f, 0.f);
   bool bad = false;
   for (int jb = j0; jb < j1; jb += kJc) {
     const int nj = min(kJc, j1 - jb);
@@ -50,15 +51,28 @@ __global__ void __launch_bounds__(128) joint_core_fwd_kernel(const __grid_consta
       xs[jj][s] = v;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int jj = 0; jj < nj; ++jj) {
-      const float4 kv = __ldcs((const float4*)(Kp + (jb + jj) * cs));
+    for (int jh = 0; jh < nj; jh += kJf) {
+      float2 acc[2][P];  // chains of kJf terms
 #pragma unroll
-      for (int s = 0; s < P; ++s) {
-        const float2 x = xs[jj][s];
-        acc[0][s] = cfma(make_float2(kv.x, kv.y), x, acc[0][s]);
-        acc[1][s] = cfma(make_float2(kv.z, kv.w), x, acc[1][s]);
+      for (int s = 0; s < P; ++s) acc[0][s] = acc[1][s] = make_float2(0.f, 0.f);
+      const int je = min(nj, jh + kJf);
+#pragma unroll 4
+      for (int jj = jh; jj < je; ++jj) {
+        const float4 kv = __ldcs((const float4*)(Kp + (jb + jj) * cs));
+#pragma unroll
+        for (int s = 0; s < P; ++s) {
+          const float2 x = xs[jj][s];
+          acc[0][s] = cfma(make_float2(kv.x, kv.y), x, acc[0][s]);
+          acc[1][s] = cfma(make_float2(kv.z, kv.w), x, acc[1][s]);
+        }
       }
+#pragma unroll
+      for (int c2 = 0; c2 < 2; ++c2)
+#pragma unroll
+        for (int s = 0; s < P; ++s) {
+          sum[c2][s].x += acc[c2][s].x;
+          sum[c2][s].y += acc[c2][s].y;
+        }
     }
   }
   if (bad) atomicOr(err, kErrNonFinite);
@@ -67,7 +81,7 @@ __global__ void __launch_bounds__(128) joint_core_fwd_kernel(const __grid_consta
   for (int s = 0; s < P; ++s)
     if (s0 + s < p) {
       float2* o = T + ((int64_t)blockIdx.y * p + s0 + s) * G.Ct + G.toff[k] + c;
-      *(float4*)o = make_float4(acc[0][s].x, acc[0][s].y, acc[1][s].x, acc[1][s].y);
+      *(float4*)o = make_float4(sum[0][s].x, sum[0][s].y, sum[1][s].x, sum[1][s].y);
     }
 }
 
@@ -110,19 +124,19 @@ __global__ void __launch_bounds__(128) joint_mode3_fwd_kernel(const __grid_const
 }
 
 // F[s][toff + xy + RR z] = sum_i3 conj(B3[i3, z]) Q[s][qoff + i3 RR + xy]; entries up to Cs are zero
-__global__ void __launch_bounds__(128) joint_mode3_adj_kernel(const __grid_constant__ JointGeo G,
+__global__ void __launch_bounds__(128, 8) joint_mode3_adj_kernel(const __grid_constant__ JointGeo G,
                                                               const float2* __restrict__ basis, const float2* __restrict__ Q,
                                                               float2* __restrict__ F) {
-  constexpr int NZ = 8, NC = 64;
+  constexpr int NZ = 8, NC = 32;
   __shared__ float2 b3[NC][NZ];
   const int k = blockIdx.z % G.q, s = blockIdx.z / G.q, R3 = G.R[k][2];
   const int RR = G.R[k][0] * G.R[k][1], z0 = blockIdx.y * NZ;
   if ((int)blockIdx.x * 128 >= RR || z0 >= R3) return;
   const int xy = blockIdx.x * 128 + threadIdx.x;
   const float2* Qs = Q + (int64_t)s * G.Qt + G.qoff[k] + (xy < RR ? xy : 0);
-  float2 acc[NZ];
+  float2 sum[NZ];
 #pragma unroll
-  for (int z = 0; z < NZ; ++z) acc[z] = make_float2(0.f, 0.f);
+  for (int z = 0; z < NZ; ++z) sum[z] = make_float2(0.f, 0.f);
   for (int i0 = 0; i0 < G.n3; i0 += NC) {
     __syncthreads();
     for (int e = threadIdx.x; e < NC * NZ; e += 128) {
@@ -130,6 +144,9 @@ __global__ void __launch_bounds__(128) joint_mode3_adj_kernel(const __grid_const
       b3[i][z] = z0 + z < R3 && i0 + i < G.n3 ? basis[G.boff[k][2] + (int64_t)(z0 + z) * G.n3 + i0 + i] : make_float2(0.f, 0.f);
     }
     __syncthreads();
+    float2 acc[NZ];  // the chunk's sums: a chain of NC terms
+#pragma unroll
+    for (int z = 0; z < NZ; ++z) acc[z] = make_float2(0.f, 0.f);
     const int ni = min(NC, G.n3 - i0);
 #pragma unroll 8
     for (int i = 0; i < ni; ++i) {
@@ -137,12 +154,17 @@ __global__ void __launch_bounds__(128) joint_mode3_adj_kernel(const __grid_const
 #pragma unroll
       for (int z = 0; z < NZ; ++z) acc[z] = cfma_conj(b3[i][z], v, acc[z]);
     }
+#pragma unroll
+    for (int z = 0; z < NZ; ++z) {
+      sum[z].x += acc[z].x;
+      sum[z].y += acc[z].y;
+    }
   }
   float2* o = F + (int64_t)s * G.Ct + G.toff[k];
   if (xy < RR)
 #pragma unroll
     for (int z = 0; z < NZ; ++z)
-      if (z0 + z < R3) o[xy + (int64_t)RR * (z0 + z)] = acc[z];
+      if (z0 + z < R3) o[xy + (int64_t)RR * (z0 + z)] = sum[z];
   if (blockIdx.x == 0 && blockIdx.y == 0)
     for (int e = RR * R3 + threadIdx.x; e < G.Cs[k]; e += 128) o[e] = make_float2(0.f, 0.f);
 }

@@ -1,7 +1,8 @@
 """ZBC_AUTO at the edges of the joint form: handles that cannot take it (ranks above its bases' 64
 vectors) keep the forms they had, its workspaces (and the FP32 forward's) keep their place, a device
 without room for it still runs the products, and vectors and columns of any size FP32 holds (the column
-sums run in FP32 up to 4 / 2 right-hand sides, forward / adjoint, and on the tensor cores from there on)."""
+sums run in FP32 up to 4 / 2 right-hand sides, forward / adjoint, and on the tensor cores from there on),
+to FP32's accuracy."""
 import numpy as np
 import pytest
 
@@ -196,3 +197,19 @@ def test_nan_is_reported_and_stays_in_its_column(p):
         assert e.value.status == zbc.ZBC_ENAN
         ok = torch.isfinite(torch.view_as_real(B)).flatten(1)
         assert not ok[1].any() and ok[0].all() and ok[2:].all()
+
+
+@pytest.mark.parametrize("p", [2, 16])
+def test_accuracy(p):
+    """Factors in exact common bases, so that only the arithmetic errs.  Its FP32 chains have at most 64
+    terms, sqrt(64 / 2) 2^-24 / sqrt(3) = 2e-7 of a sum of random terms, in four passes of which each adds
+    less than that: 4e-7, and 1e-7 for operands in FP32.  Truncating accumulators would shift the mean by 4.3e-8
+    times half the sums they round, 1e-6 here; what is put back for them is a multiple of 2^-23 per pass."""
+    g, tens = _shared((96, 90, 64), 96, (56, 56, 48), (16, 16, 16))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    X = _c64(inputs.cn01((96, p), seed=1))
+    Phi = _c64(inputs.cn01((3 * g.nv, p), seed=2))
+    for A, ref, fwd in ((X, products.matvec, True), (Phi, products.rmatvec, False)):
+        got, ref = _run(h, g, A, fwd).astype(np.complex128), ref(tens, g.shape, A)
+        assert _rel(got, ref) < 5e-7
+        assert abs(np.vdot(ref, got).real / np.linalg.norm(ref) ** 2 - 1) < 1.5e-7
