@@ -483,7 +483,8 @@ int zbc_product_status(const zbc_handle* h, zbc_stream stream);
  * allows each consumer warp `polls` polls of the wait for its first stage (40,000,000 normally);
  * polls = 0 makes that wait give up at once, so the launch takes its abort path (the copies
  * already issued are still waited for, with the normal limit) and zbc_product_status reports
- * ZBC_ETIMEOUT.  Later launches use the normal limit.
+ * ZBC_ETIMEOUT.  A ZBC_AUTO product in the joint form takes the limit for its kernels' waits instead.
+ * Later launches use the normal limit.
  */
 int zbc_test_wait_limit(zbc_handle* h, uint32_t polls);
 

@@ -54,16 +54,21 @@ struct JointCache {
 // the plane products on the tensor cores (joint_planes.cu): Y from Q, and Q from Phi
 size_t joint_planes_bytes(const JointGeo& G);
 int joint_planes_build(const JointGeo& G, const float2* basis, unsigned char* bop, cudaStream_t st);
-int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st);
-int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err, cudaStream_t st);
+// (polls: tries of each bounded wait, about a microsecond each)
+constexpr uint32_t kJointPolls = 1000000;
+int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, uint32_t polls,
+                     cudaStream_t st);
+int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err, uint32_t polls,
+                     cudaStream_t st);
 
 // the column sums on the tensor cores (joint_core.cu): T from X, and partial Psi from F in `splits`
 // slices of `split` chunks of core entries
 size_t joint_core_bytes(const JointGeo& G);
 int joint_core_build(const JointGeo& G, const float2* K, float* kscale, bool* fits, cudaStream_t st);
-int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, cudaStream_t st);
+int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, uint32_t polls,
+                   cudaStream_t st);
 void joint_core_split(const JointGeo& G, int p, int* split, int* splits);
-int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, cudaStream_t st);
+int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, uint32_t polls, cudaStream_t st);
 
 // Builds h.joint (synchronises).  Returns ZBC_OK also when no small basis exists: see usable.
 int build_joint(Handle& h, cudaStream_t st);

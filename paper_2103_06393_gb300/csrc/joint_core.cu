@@ -43,7 +43,7 @@ template <bool FWD, int P>
 __global__ void __launch_bounds__(288, 2)
     joint_core_kernel(const __grid_constant__ JointGeo G, const float2* __restrict__ K, const float* __restrict__ kscale,
                       const float2* __restrict__ R, int64_t ldr, int p, int split, float2* __restrict__ out,
-                      int* __restrict__ err) {
+                      int* __restrict__ err, uint32_t polls) {
   constexpr int N = 2 * P, I = P / 8;
   constexpr uint32_t kBTerm = N * 128u, ncols = FWD ? 2 * N : 4 * N;  // two accumulators, the adjoint's sums
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -61,13 +61,7 @@ __global__ void __launch_bounds__(288, 2)
   if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
   __syncthreads();
   const uint32_t tmem = tmem_base;
-  bool ok = true;  // false after a wait gave up: no further waits
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok && !tc::mbar_wait_idle(bar, parity)) {
-      ok = false;
-      atomicOr(err, kErrTimeout);
-    }
-  };
+  Waits waits{err, polls};
   // forward: items are the 128-row tiles of all components, walked by blockIdx.x; adjoint: one item,
   // slice blockIdx.x of `split` chunks of one component (ksplit, first chunk ch0), for rows 128 blockIdx.y
   const int s0 = blockIdx.z * P, Mp = (G.M + kSum - 1) / kSum * kSum;
@@ -82,10 +76,11 @@ __global__ void __launch_bounds__(288, 2)
   if (warp == 8) {
     if (lane == 0) {
       constexpr uint32_t id = tc::instr_desc(128, N, 0);
-      for (int c = 0; c < items * per; ++c) {
+      int c = 0;
+      for (; c < items * per; ++c) {
         const int d = c & 1;
-        wait(&ready[d], (c >> 1) & 1);
-        if (!ok) break;
+        waits.one(&ready[d], (c >> 1) & 1);
+        if (!waits.ok) break;
         tc::fence_after();
         const uint32_t a0 = tc::smem_u32(sa) + d * 2 * kRowTerm, b0 = tc::smem_u32(sb) + d * 2 * kBTerm;
 #pragma unroll
@@ -100,6 +95,7 @@ __global__ void __launch_bounds__(288, 2)
           tc::mma<0>(tmem + d * N, tc::smem_desc_sw128(a0 + ks * 32), tc::smem_desc_sw128(b0 + ks * 32), id, 1);
         tc::commit(&done[d]);
       }
+      drain2(done, c);
     }
     __syncwarp();
   } else {
@@ -173,7 +169,7 @@ __global__ void __launch_bounds__(288, 2)
       for (int i = 0; i < P; ++i) acc[i] = 0.f;
       auto fold = [&](int c) {
         const int d = c & 1;
-        wait(&done[d], (c >> 1) & 1);
+        waits.warp(&done[d], (c >> 1) & 1);
         tc::fence_after();
         const uint32_t t0 = tmem + (uint32_t)(d * N + half * P) + ((uint32_t)(32 * q4) << 16);
 #pragma unroll
@@ -350,22 +346,24 @@ __global__ void __launch_bounds__(256) core_scale_kernel(const __grid_constant__
 int padded_m(const JointGeo& G) { return ceil_div(G.M, kSum) * kSum; }
 
 template <int P>
-int launch_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, cudaStream_t st) {
+int launch_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, uint32_t polls,
+               cudaStream_t st) {
   const JointGeo& G = jc.geo;
   ZBC_TRY((set_smem_limit<joint_core_kernel<true, P>>((int)core_smem<P>())));
   int tiles = 0;
   for (int k = 0; k < G.q; ++k) tiles += ceil_div(G.Cs[k], kRows);
   const int passes = ceil_div(p, P);
   joint_core_kernel<true, P><<<dim3(std::min(tiles, 2 * sm_count()), 1, passes), 288, core_smem<P>(), st>>>(
-      G, jc.K, jc.kscale, X, ldx, p, 0, T, err);
+      G, jc.K, jc.kscale, X, ldx, p, 0, T, err, polls);
   return ZBC_OK;
 }
 template <int P>
-int launch_adj(const JointCache& jc, const float2* F, int p, int split, int splits, float2* part, int* err, cudaStream_t st) {
+int launch_adj(const JointCache& jc, const float2* F, int p, int split, int splits, float2* part, int* err, uint32_t polls,
+               cudaStream_t st) {
   const JointGeo& G = jc.geo;
   ZBC_TRY((set_smem_limit<joint_core_kernel<false, P>>((int)core_smem<P>())));
   joint_core_kernel<false, P><<<dim3(splits, ceil_div(G.M, kRows), ceil_div(p, P)), 288, core_smem<P>(), st>>>(
-      G, jc.K, jc.kscale, F, G.Ct, p, split, part, err);
+      G, jc.K, jc.kscale, F, G.Ct, p, split, part, err, polls);
   return ZBC_OK;
 }
 
@@ -391,11 +389,12 @@ int joint_core_build(const JointGeo& G, const float2* K, float* kscale, bool* fi
   return ZBC_OK;
 }
 
-int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, cudaStream_t st) {
+int joint_core_fwd(const JointCache& jc, const float2* X, int64_t ldx, int p, float2* T, int* err, uint32_t polls,
+                   cudaStream_t st) {
   switch (rhs_tile(p)) {
-    case 8: ZBC_TRY(launch_fwd<8>(jc, X, ldx, p, T, err, st)); break;
-    case 16: ZBC_TRY(launch_fwd<16>(jc, X, ldx, p, T, err, st)); break;
-    default: ZBC_TRY(launch_fwd<32>(jc, X, ldx, p, T, err, st)); break;
+    case 8: ZBC_TRY(launch_fwd<8>(jc, X, ldx, p, T, err, polls, st)); break;
+    case 16: ZBC_TRY(launch_fwd<16>(jc, X, ldx, p, T, err, polls, st)); break;
+    default: ZBC_TRY(launch_fwd<32>(jc, X, ldx, p, T, err, polls, st)); break;
   }
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
@@ -412,13 +411,13 @@ void joint_core_split(const JointGeo& G, int p, int* split, int* splits) {
   for (int k = 0; k < G.q; ++k) *splits += slices_of(G.Cs[k], *split);
 }
 
-int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, cudaStream_t st) {
+int joint_core_adj(const JointCache& jc, const float2* F, int p, float2* part, int* err, uint32_t polls, cudaStream_t st) {
   int split, splits;
   joint_core_split(jc.geo, p, &split, &splits);
   switch (rhs_tile(p)) {
-    case 8: ZBC_TRY(launch_adj<8>(jc, F, p, split, splits, part, err, st)); break;
-    case 16: ZBC_TRY(launch_adj<16>(jc, F, p, split, splits, part, err, st)); break;
-    default: ZBC_TRY(launch_adj<32>(jc, F, p, split, splits, part, err, st)); break;
+    case 8: ZBC_TRY(launch_adj<8>(jc, F, p, split, splits, part, err, polls, st)); break;
+    case 16: ZBC_TRY(launch_adj<16>(jc, F, p, split, splits, part, err, polls, st)); break;
+    default: ZBC_TRY(launch_adj<32>(jc, F, p, split, splits, part, err, polls, st)); break;
   }
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());

@@ -52,7 +52,7 @@ constexpr int kQRegs = kJointRmax * kJointRmax / kFwdWorkers;
 __global__ void __launch_bounds__(kFwdThreads, 1)
     joint_planes_fwd_kernel(const __grid_constant__ JointGeo G, const __grid_constant__ FwdShape F,
                             const float2* __restrict__ basis, const float2* __restrict__ Q, int p, float2* __restrict__ Y,
-                            int64_t ldy, int* __restrict__ err) {
+                            int64_t ldy, int* __restrict__ err, uint32_t polls) {
   extern __shared__ __align__(128) unsigned char smem_f[];
   __shared__ __align__(8) uint64_t done[2], dfree[2], sready, qready, s1done;
   __shared__ uint32_t tmem_base;
@@ -108,13 +108,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
   const uint32_t tmem = tmem_base;
   const int planes = p * G.n3;
   const int mine = (planes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;  // grid x <= planes
-  bool ok = true;  // false after a wait gave up: no further waits, the barriers are still passed
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok && !tc::mbar_wait_idle(bar, parity)) {
-      ok = false;
-      atomicOr(err, kErrTimeout);
-    }
-  };
+  Waits waits{err, polls};
   if (warp == kFwdWorkers / 32) {
     if (lane == 0) {
       const uint32_t b1 = tc::smem_u32(sa), s0 = tc::smem_u32(ss), b2 = tc::smem_u32(sb2), q0 = tc::smem_u32(sq);
@@ -128,21 +122,22 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
           tc::mma<0>(d, ah, bh, id, 1);
         }
       };
+      int m1 = 0, n = 0;  // MMAs 1 issued, accumulators of MMA 2 used so far
       auto mma1 = [&](int t) {
-        wait(&qready, t & 1);
-        if (!ok) return;
+        waits.one(&qready, t & 1);
+        if (!waits.ok) return;
         tc::fence_after();
         chain(tmem, b2, b2term, q0, qterm, sbo1, KB1 / 2, tc::instr_desc(128, 2 * R1p, 0));
         tc::commit(&s1done);
+        ++m1;
       };
       mma1(0);
-      int n = 0;  // accumulators used so far
-      for (int t = 0; t < mine && ok; ++t) {
-        wait(&sready, t & 1);
+      for (int t = 0; t < mine && waits.ok; ++t) {
+        waits.one(&sready, t & 1);
         if (lag && t + 1 < mine) mma1(t + 1);
-        for (int b = 0; b < nblk && ok; ++b, ++n) {
-          wait(&dfree[n & 1], ((n >> 1) & 1) ^ 1);  // a fresh barrier's preceding phase counts as complete
-          if (!ok) break;
+        for (int b = 0; b < nblk && waits.ok; ++b, ++n) {
+          waits.one(&dfree[n & 1], ((n >> 1) & 1) ^ 1);  // a fresh barrier's preceding phase counts as complete
+          if (!waits.ok) break;
           tc::fence_after();
           chain(tmem + d2 + (uint32_t)((n & 1) * 2 * T2), b1 + (uint32_t)b * 2 * ablk, b == nblk - 1 ? alast : ablk,
                 s0 + (uint32_t)(t & lag) * 2 * sterm, sterm, sbo, KB / 2, tc::instr_desc(128, 2 * T2, 0));
@@ -150,6 +145,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         }
         if (!lag && t + 1 < mine) mma1(t + 1);
       }
+      drain1(&s1done, m1);
+      drain2(done, n);
     }
     __syncwarp();
   } else {
@@ -205,7 +202,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       if (t < mine) {
         // S's rows 2 i2, 2 i2 + 1 from D1's row i2: D1 = 2^(kDataShift + kBasisShift - e) S, so 2^-9 D1 < 2^15,
         // and D2 = 2^(21 - e) Y
-        wait(&s1done, t & 1);
+        waits.warp(&s1done, t & 1);
         tc::fence_after();
         const int r = 32 * q4 + lane;
         if (32 * q4 < T2) {
@@ -246,12 +243,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       const int left = min(T2, G.n2 - i20);
       for (int b = 0; b < nblk; ++b, ++n) {
         const int d = n & 1, i1 = b * 128 + 32 * q4;
-        wait(&done[d], (n >> 1) & 1);
+        waits.warp(&done[d], (n >> 1) & 1);
         tc::fence_after();
-        if (i1 < rows && ok) {
+        if (i1 < rows) {
           const uint32_t t0 = tmem + d2 + (uint32_t)(d * 2 * T2) + ((uint32_t)(32 * q4) << 16);
           float2* y0 = Yp + i1 + lane;
-          const bool live = i1 + lane < rows;
+          const bool live = i1 + lane < rows && waits.ok;
           for (int c = grp; c < T2 / 8; c += kFwdGroups) {
             float v[16];
             tc::tmem_ld16(t0 + 16 * c, v);
@@ -296,7 +293,7 @@ template <int I, bool VEC>
 __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     joint_planes_adj_kernel(const __grid_constant__ JointGeo G, const unsigned char* __restrict__ bop,
                             const float2* __restrict__ b2t, const float2* __restrict__ Phi, int64_t ldphi, int p,
-                            float2* __restrict__ Q, int* __restrict__ err) {
+                            float2* __restrict__ Q, int* __restrict__ err, uint32_t polls) {
   constexpr int NC = 8 * I, N = 2 * NC, RC = (NC + 15) / 16;  // Q: RC x RC entries a thread
   constexpr int R2p = 16 * RC;
   constexpr uint32_t kBTerm = N * 128u;
@@ -322,13 +319,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
   const int nch = (G.n1 + kChunk1 - 1) / kChunk1, nt2 = (G.n2 + kTile2 - 1) / kTile2;
   const int planes = G.n3 * p * G.q;  // plane = k + q (i3 + n3 s); a CTA's planes are blockIdx.x + g gridDim.x
   const int mine = (planes - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;  // grid <= planes
-  bool ok = true;  // false after a wait gave up: no further waits, the barriers are still passed
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok && !tc::mbar_wait_idle(bar, parity)) {
-      ok = false;
-      atomicOr(err, kErrTimeout);
-    }
-  };
+  Waits waits{err, polls};
   if (warp == 8) {
     if (lane == 0) {
       // chunk c of this CTA (all tiles of all its planes in order): its B block is copied once the MMAs
@@ -346,12 +337,12 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
       for (; c < total; ++c) {
         const int d = c & 1;
         const uint32_t par = (c >> 1) & 1;
-        if (c > 0) wait(&done[d ^ 1], ((c - 1) >> 1) & 1);
-        if (!ok) break;
+        if (c > 0) waits.one(&done[d ^ 1], ((c - 1) >> 1) & 1);
+        if (!waits.ok) break;
         if (c + 1 < total) copy_b(c + 1);
-        wait(&full[d], par);
-        wait(&ready[d], par);
-        if (!ok) break;
+        waits.one(&full[d], par);
+        waits.one(&ready[d], par);
+        if (!waits.ok) break;
         tc::fence_after();
         const uint32_t a0 = tc::smem_u32(sa) + d * 2 * kATerm, b0 = tc::smem_u32(sb) + d * 2 * kBTerm;
         constexpr uint32_t id = tc::instr_desc(128, N, 0);
@@ -367,11 +358,15 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
           tc::mma<0>(tmem + d * N, tc::smem_desc_sw128(a0 + ks * 32), tc::smem_desc_sw128(b0 + ks * 32), id, 1);
         tc::commit(&done[d]);
       }
+      drain2(done, c);
       // after giving up: the copies in flight land before the buffers are left
       for (int i = c; i < issued; ++i) tc::mbar_wait_idle(&full[i & 1], (i >> 1) & 1);
     }
     __syncwarp();
   } else {
+    // a limit known at compile time: 320 x 320 x 256, 8 right-hand sides (I = 3) 1.70 against 1.72 ms, but
+    // 194 against 188 us at I = 4 (160 x 160 x 128, 4)
+    if (I <= 3) waits.polls = kJointPolls;
     const int64_t nv = (int64_t)G.n1 * G.n2 * G.n3;
     const int row0 = warp * 4 + lane / 8, c8 = lane % 8;  // loader: rows row0 + 32 u, i1 = entry_of(c8, w)
     const int q4 = warp & 3, half = warp >> 2;            // accumulator rows and columns
@@ -424,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
       for (int c = 0; c < NC; ++c) acc[c] = 0.f;
       auto fold = [&](int c) {  // also: the MMAs have read chunk c's buffer
         const int d = c & 1;
-        wait(&done[d], (c >> 1) & 1);
+        waits.warp(&done[d], (c >> 1) & 1);
         tc::fence_after();
         if (32 * q4 < rows) {
           const float us = pow2f(rexp[c & 3][32 * q4 + lane] - 2) * (pow2f(2 - kDataShift - kBasisShift) * lo_first_gain(4));
@@ -581,13 +576,13 @@ __global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_const
 
 template <int I, bool VEC>
 int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
-                      int* err, cudaStream_t st) {
+                      int* err, uint32_t polls, cudaStream_t st) {
   const float2* b2t = (const float2*)(bop + bop_bytes(G));
   ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC>>((int)planes_adj_smem(8 * I))));
   const size_t sm = planes_adj_smem(8 * I);
   const int64_t planes = (int64_t)G.n3 * p * G.q;
   const int grid = (int)std::min<int64_t>(planes, (sm <= 112 * 1024 ? 2 : 1) * sm_count());
-  joint_planes_adj_kernel<I, VEC><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err);
+  joint_planes_adj_kernel<I, VEC><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err, polls);
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
@@ -595,16 +590,17 @@ int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2*
 
 template <int I>
 int planes_adj_vec(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
-                   int* err, cudaStream_t st) {
+                   int* err, uint32_t polls, cudaStream_t st) {
   // every column of every plane on 16 bytes, and no pair of entries across the end of one
   if (G.n1 % 2 == 0 && (p == 1 || ldphi % 2 == 0) && (uintptr_t)Phi % 16 == 0)
-    return launch_planes_adj<I, true>(G, bop, Phi, ldphi, p, Q, err, st);
-  return launch_planes_adj<I, false>(G, bop, Phi, ldphi, p, Q, err, st);
+    return launch_planes_adj<I, true>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  return launch_planes_adj<I, false>(G, bop, Phi, ldphi, p, Q, err, polls, st);
 }
 
 }  // namespace
 
-int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, cudaStream_t st) {
+int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, int64_t ldy, int* err, uint32_t polls,
+                     cudaStream_t st) {
   const JointGeo& G = jc.geo;
   constexpr size_t kLimit = 224 * 1024;
   // balanced tiles of i2 that leave tensor memory for D1 and two D2; where the operands do not fit
@@ -626,24 +622,24 @@ int joint_planes_fwd(const JointCache& jc, const float2* Q, int p, float2* Y, in
   ZBC_TRY(set_smem_limit<joint_planes_fwd_kernel>((int)kLimit));
   const int walkers = std::min(p * G.n3, std::max(1, sm_count() / (F.gy * F.nt2 * G.q)));
   joint_planes_fwd_kernel<<<dim3(walkers, F.gy * F.nt2, G.q), kFwdThreads, F.bytes(G.n1), st>>>(G, F, jc.basis, Q, p, Y, ldy,
-                                                                                            err);
+                                                                                            err, polls);
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
 }
 
-int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
+int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err, uint32_t polls,
                      cudaStream_t st) {
   const JointGeo& G = jc.geo;
   switch (adj_rows(G) / 8) {
-    case 1: return planes_adj_vec<1>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 2: return planes_adj_vec<2>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 3: return planes_adj_vec<3>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 4: return planes_adj_vec<4>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 5: return planes_adj_vec<5>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 6: return planes_adj_vec<6>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    case 7: return planes_adj_vec<7>(G, jc.bop, Phi, ldphi, p, Q, err, st);
-    default: return planes_adj_vec<8>(G, jc.bop, Phi, ldphi, p, Q, err, st);
+    case 1: return planes_adj_vec<1>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 2: return planes_adj_vec<2>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 3: return planes_adj_vec<3>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 4: return planes_adj_vec<4>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 5: return planes_adj_vec<5>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 6: return planes_adj_vec<6>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 7: return planes_adj_vec<7>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    default: return planes_adj_vec<8>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
   }
 }
 

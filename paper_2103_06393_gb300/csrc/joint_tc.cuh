@@ -93,10 +93,32 @@ __device__ __forceinline__ void warp_publish(uint64_t* bar) {
   if ((threadIdx.x & 31) == 0) mbar_arrive1(bar);
 }
 
-__host__ __device__ inline uint32_t tmem_cols(uint32_t need) {
-  uint32_t c = 32;
-  while (c < need) c *= 2;
-  return c;
+// The bounded waits of a kernel: once one gave up (after `polls` tries of about a microsecond) its thread waits no
+// more; the barriers are still passed, and the thread that issues the MMAs ends with drain2() / drain1().
+struct Waits {
+  int* err;
+  uint32_t polls;
+  bool ok = true;
+  __device__ void one(uint64_t* bar, uint32_t parity) {
+    if (ok && !tc::mbar_wait_idle(bar, parity, polls)) {
+      ok = false;
+      atomicOr(err, kErrTimeout);
+    }
+  }
+  // by all lanes of a warp, each of which may give up by itself: what needs the whole warp after it (tcgen05.ld)
+  // is run whatever `ok` says, and only what a lane does alone asks for it
+  __device__ void warp(uint64_t* bar, uint32_t parity) {
+    one(bar, parity);
+    __syncwarp();
+  }
+};
+// The n-th commit (from 1) to a pair of barriers, or to one, has completed: whatever was issued no longer reads
+// shared memory or writes tensor memory when the CTA gives them up.
+__device__ __forceinline__ void drain2(uint64_t* bar, int n) {
+  if (n > 0) tc::mbar_wait_idle(bar + ((n - 1) & 1), ((n - 1) >> 1) & 1);
+}
+__device__ __forceinline__ void drain1(uint64_t* bar, int n) {
+  if (n > 0) tc::mbar_wait_idle(bar, (n - 1) & 1);
 }
 
 }  // namespace

@@ -340,10 +340,18 @@ void joint_plan_work(JointCache* jc) {
   }
 }
 
+// tries of the product's bounded waits; a test limit applies to one product
+static uint32_t take_wait_limit(Handle& h) {
+  const uint32_t polls = std::min(h.test_first_wait, kJointPolls);
+  h.test_first_wait = kWaitPolls;
+  return polls;
+}
+
 int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int64_t ldy, cudaStream_t st) {
   const JointCache& jc = *h.joint;
   const JointGeo& G = jc.geo;
   int* err = (int*)h.work_err.ptr;
+  const uint32_t polls = take_wait_limit(h);
   ZBC_TRY(h.work_joint_fwd.ensure(joint_work_bytes(h, p, true)));
   int csmax = 0, rrmax = 0;
   for (int k = 0; k < G.q; ++k) {
@@ -358,14 +366,14 @@ int matvec_joint(Handle& h, const float2* X, int64_t ldx, int p, float2* Y, int6
     float2* Q = T + pl.telems;
     const float2* Xs = X + ldx * s0;
     switch (ps >= kTcFwd ? 0 : pl.P) {
-      case 0: ZBC_TRY(joint_core_fwd(jc, Xs, ldx, ps, T, err, st)); break;
+      case 0: ZBC_TRY(joint_core_fwd(jc, Xs, ldx, ps, T, err, polls, st)); break;
       case 1: launch_core_fwd<1>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
       case 2: launch_core_fwd<2>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
       default: launch_core_fwd<4>(G, jc.K, Xs, ldx, ps, JS, T, err, csmax, st); break;
     }
     joint_mode3_fwd_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(G.n3, kZ), ps * G.q), 128, 0, st>>>(G, jc.basis, T, ps, JS, Q);
     count_launch();
-    ZBC_TRY(joint_planes_fwd(jc, Q, ps, Y + ldy * s0, ldy, err, st));
+    ZBC_TRY(joint_planes_fwd(jc, Q, ps, Y + ldy * s0, ldy, err, polls, st));
   }
   return ZBC_OK;
 }
@@ -374,6 +382,7 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
   const JointCache& jc = *h.joint;
   const JointGeo& G = jc.geo;
   int* err = (int*)h.work_err.ptr;
+  const uint32_t polls = take_wait_limit(h);
   ZBC_TRY(h.work_joint_adj.ensure(joint_work_bytes(h, p, false)));
   int r3 = 0, rrmax = 0;
   for (int k = 0; k < G.q; ++k) {
@@ -388,10 +397,10 @@ int rmatvec_joint(Handle& h, const float2* Phi, int64_t ldphi, int p, float2* ou
     float2* F = Q + pl.qelems;
     float2* part = F + pl.felems;
     const float2* Ps = Phi + ldphi * s0;
-    ZBC_TRY(joint_planes_adj(jc, Ps, ldphi, ps, Q, err, st));
+    ZBC_TRY(joint_planes_adj(jc, Ps, ldphi, ps, Q, err, polls, st));
     joint_mode3_adj_kernel<<<dim3(ceil_div(rrmax, 128), ceil_div(r3, 8), ps * G.q), 128, 0, st>>>(G, jc.basis, Q, F);
     switch (ps >= kTcAdj ? 0 : pl.P) {
-      case 0: ZBC_TRY(joint_core_adj(jc, F, ps, part, err, st)); break;
+      case 0: ZBC_TRY(joint_core_adj(jc, F, ps, part, err, polls, st)); break;
       case 1: launch_core_adj<1>(G, jc.K, F, ps, chunk, splits, part, st); break;
       default: launch_core_adj<2>(G, jc.K, F, ps, chunk, splits, part, st); break;
     }

@@ -115,7 +115,8 @@ struct Handle {
   int8_t tune_adj_warps[kPClasses] = {0, 0, 0, 0, 0, 0, 0, 0};
   int8_t tune_adj_prec[kPClasses] = {-1, -1, -1, -1, -1, -1, -1, -1};
   // polls allowed to the first stage wait of each consumer warp of the next FP32 SIMT adjoint
-  // launch (zbc_test_wait_limit; reset after that launch); kWaitPolls otherwise
+  // launch, or to the waits of the next product in the joint form (zbc_test_wait_limit; reset after
+  // that launch or product); kWaitPolls otherwise
   uint32_t test_first_wait = kWaitPolls;
   ~Handle();
   int64_t nv() const { return (int64_t)n1 * n2 * n3; }

@@ -531,7 +531,8 @@ def zbc_tune(h: Handle, p: int, stream=None) -> dict:
 
 def zbc_test_wait_limit(h: Handle, polls: int):
     """Test hook: the next FP32 SIMT adjoint launch on h allows its consumers' first stage wait
-    `polls` polls (0: give up at once, so zbc_product_status reports ZBC_ETIMEOUT)."""
+    `polls` polls (0: give up at once, so zbc_product_status reports ZBC_ETIMEOUT); an AUTO product
+    in the joint form takes it for its kernels' waits."""
     _check(lib().zbc_test_wait_limit(h.ptr, int(polls)))
 
 

@@ -2,7 +2,7 @@
 vectors) keep the forms they had, its workspaces (and the FP32 forward's) keep their place, a device
 without room for it still runs the products, and vectors and columns of any size FP32 holds (the column
 sums run in FP32 up to 4 / 2 right-hand sides, forward / adjoint, and on the tensor cores from there on),
-to FP32's accuracy."""
+to FP32's accuracy; and its bounded waits, which end a product that cannot go on with a status."""
 import numpy as np
 import pytest
 
@@ -213,3 +213,18 @@ def test_accuracy(p):
         got, ref = _run(h, g, A, fwd).astype(np.complex128), ref(tens, g.shape, A)
         assert _rel(got, ref) < 5e-7
         assert abs(np.vdot(ref, got).real / np.linalg.norm(ref) ** 2 - 1) < 1.5e-7
+
+
+@pytest.mark.parametrize("p", [2, 9, 40])
+@pytest.mark.parametrize("fwd", [True, False])
+def test_a_wait_that_gives_up_is_reported_and_the_next_product_is_right(fwd, p):
+    g, tens = _shared((300, 36, 20), 150, (12, 11, 10), (6, 5, 4))  # several blocks of i1, tiles of rows
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    A = _c64(inputs.cn01((150 if fwd else 3 * g.nv, p), seed=1))
+    ref = (products.matvec if fwd else products.rmatvec)(tens, g.shape, A)
+    assert _rel(_run(h, g, A, fwd), ref) < RTOL
+    zbc.zbc_test_wait_limit(h, 0)
+    with pytest.raises(zbc.ZbcError) as e:
+        _run(h, g, A, fwd)
+    assert e.value.status == zbc.ZBC_ETIMEOUT
+    assert _rel(_run(h, g, A, fwd), ref) < RTOL  # the limit was for one product, and the word is clear
