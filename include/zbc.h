@@ -455,7 +455,9 @@ int zbc_rmatvec_noalloc(const zbc_handle* h, const void* Phi, int64_t ldphi, int
  * Each variant runs once untimed, then is timed over two calls, or over one when that call took
  * more than 1.5 times the best of its direction so far (the tensor-core forms are timed first).
  * Afterwards the per-handle operands of the forms that no tuned class selects (TC_MODE1's, TC_DC's,
- * TC2's) are freed; a later call of such a form builds them again (zbc_device_bytes shows both).
+ * TC2's, and the joint form's unless a ZBC_AUTO product of an untuned class has run it) are freed; a
+ * later call of such a form builds them again (zbc_device_bytes shows both; ZBC_AUTO does not build the
+ * joint form again for an untuned class as long as no tuned class selects it).
  * A CUDA graph captured before this call may hold pointers to those operands: tune first, then
  * capture.
  *   times_ms_host : optional float[10], the variants' times in the order above (ms per call;

@@ -38,6 +38,7 @@ constexpr int kJointPass = 64;  // right-hand sides that the products' workspace
 struct JointCache {
   bool usable = false;    // false: the factors share no small basis (the other forms are used)
   bool large = false;     // the products decompress more than 1e8 voxel ranks
+  bool untuned_use = false;  // products of untuned classes ran it: captured graphs may hold its operands
   bool no_room = false;   // unusable for want of device memory: zbc_tune tries again
   JointGeo geo;
   float2* basis = nullptr;

@@ -42,12 +42,22 @@ static bool joint_ready(Handle& h, int p, bool fwd, cudaStream_t st) {
   return s == ZBC_OK && h.joint->usable;
 }
 
-// The form of ZBC_AUTO: the tuned one; untuned, the joint form where the handle has it, else BF16X3
-// for a forward product of p >= 8 and FP32_SIMT.
+static bool tuned_to(const Handle& h, zbc_precision form) {
+  for (int i = 0; i < Handle::kPClasses; ++i)
+    if (h.tune_fwd_prec[i] == form || h.tune_adj_prec[i] == form) return true;
+  return false;
+}
+
+// The form of ZBC_AUTO: the tuned one; untuned, the joint form where the handle has it (it is not built
+// for an untuned class once tuning others has only found faster forms), else BF16X3 for a forward product
+// of p >= 8 and FP32_SIMT.
 static zbc_precision auto_form(Handle& h, int p, bool fwd, cudaStream_t st) {
-  const int tuned = fwd ? h.tune_fwd_prec[rhs_class(p)] : h.tune_adj_prec[rhs_class(p)];
+  const int cls = rhs_class(p), tuned = fwd ? h.tune_fwd_prec[cls] : h.tune_adj_prec[cls];
   if (tuned >= 0 && tuned != kFormJoint) return (zbc_precision)tuned;
-  if (joint_ready(h, p, fwd, st)) return kFormJoint;
+  if ((h.joint || !h.tuned || tuned_to(h, kFormJoint)) && joint_ready(h, p, fwd, st)) {
+    if (tuned < 0) h.joint->untuned_use = true;
+    return kFormJoint;
+  }
   return fwd && p >= 8 ? ZBC_BF16X3 : ZBC_FP32_SIMT;
 }
 
@@ -133,18 +143,18 @@ extern "C" int zbc_rmatvec(const zbc_handle* hh, const void* Phi, int64_t ldphi,
                       (cudaStream_t)stream);
 }
 
-// The per-handle operands of the forms that no tuned right-hand-side class selects (untuned
-// classes fall back to BF16X3 or FP32_SIMT, which need none of them) are freed; a later call of
-// such a form builds them again.  The decompression cache itself is kept.
+// The per-handle operands of the forms that no tuned right-hand-side class selects are freed; a later
+// call of such a form builds them again.  The decompression cache itself is kept, and the joint form's
+// operands once an untuned class has run it (untuned classes otherwise run BF16X3 or FP32_SIMT, which
+// need nothing else).
 static void release_unused_operands(Handle& h) {
   DecompCache* c = h.cache;
   if (!c) return;
-  bool m1f = false, m1a = false, dc = false, tc2 = false, joint = false;
+  bool m1f = false, m1a = false, dc = false, tc2 = false;
   for (int i = 0; i < Handle::kPClasses; ++i) {
     m1f = m1f || h.tune_fwd_prec[i] == ZBC_TC_MODE1;
     dc = dc || h.tune_fwd_prec[i] == ZBC_TC_DC;
     tc2 = tc2 || h.tune_fwd_prec[i] == ZBC_TC2;
-    joint = joint || h.tune_fwd_prec[i] == kFormJoint || h.tune_adj_prec[i] == kFormJoint;
     m1a = m1a || h.tune_adj_prec[i] == ZBC_TC_MODE1;
   }
   if (c->mode1 && !m1f) mode1_fwd_release(c->mode1);
@@ -157,7 +167,7 @@ static void release_unused_operands(Handle& h) {
     c->dc = nullptr;
   }
   if (!tc2) half_release(c);
-  if (!joint && h.joint && h.joint->usable) {
+  if (!tuned_to(h, kFormJoint) && h.joint && h.joint->usable && !h.joint->untuned_use) {
     joint_release(h.joint);
     h.joint = nullptr;
   }
@@ -258,6 +268,7 @@ extern "C" int zbc_tune(zbc_handle* hh, int p, zbc_stream stream, float* times_m
     return ZBC_EINVAL;
   }
   const int cls = rhs_class(p);
+  h.tuned = true;
   h.tune_fwd_prec[cls] = (int8_t)vars[bf].prec;
   h.tune_fwd_warps[cls] = (int8_t)vars[bf].warps;
   h.tune_adj_prec[cls] = (int8_t)vars[ba].prec;

@@ -110,6 +110,7 @@ struct Handle {
   int cache_r = 0;                 // largest r1 rounded up to 2 (cache row stride bound)
   // autotuned choices per right-hand-side class (zbc_tune; -1 / 0 = untuned)
   static constexpr int kPClasses = 8;
+  bool tuned = false;
   int8_t tune_fwd_prec[kPClasses] = {-1, -1, -1, -1, -1, -1, -1, -1};
   int8_t tune_fwd_warps[kPClasses] = {0, 0, 0, 0, 0, 0, 0, 0};
   int8_t tune_adj_warps[kPClasses] = {0, 0, 0, 0, 0, 0, 0, 0};

@@ -228,3 +228,35 @@ def test_a_wait_that_gives_up_is_reported_and_the_next_product_is_right(fwd, p):
         _run(h, g, A, fwd)
     assert e.value.status == zbc.ZBC_ETIMEOUT
     assert _rel(_run(h, g, A, fwd), ref) < RTOL  # the limit was for one product, and the word is clear
+
+
+def test_tuning_keeps_what_an_untuned_class_runs():
+    """A graph of an untuned class survives the tuning of another one, whichever form that selects."""
+    g, tens = _shared((24, 24, 24), 40, (10, 10, 10), (6, 6, 6))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    A = zbc.to_colmajor(inputs.cn01((40, 2), seed=1).astype(np.complex64))
+    Y, Z = (zbc.colmajor(3 * g.nv, 2, torch.complex64) for _ in range(2))
+    zbc.zbc_matvec(h, A, Y, zbc.AUTO)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        zbc.zbc_matvec(h, A, Z, zbc.AUTO)
+    held = h.device_bytes()["caches"]
+    for p in (1, 12, 64):
+        zbc.zbc_tune(h, p)
+        assert h.device_bytes()["caches"] >= held, p
+    graph.replay()
+    torch.cuda.synchronize()
+    zbc.zbc_product_status(h)
+    assert torch.equal(Y, Z)
+
+
+def test_untuned_class_after_tuning_without_the_joint_form():
+    """Tuned on its own, the handle drops the joint form if it lost, and an untuned class leaves it so."""
+    g, tens = _shared((24, 24, 24), 40, (10, 10, 10), (6, 6, 6))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    zbc.zbc_tune(h, 1)
+    held = h.device_bytes()["caches"]
+    X = _c64(inputs.cn01((40, 12), seed=1))
+    assert _rel(_run(h, g, X, True), products.matvec(tens, g.shape, X)) < RTOL
+    assert h.device_bytes()["caches"] == held
