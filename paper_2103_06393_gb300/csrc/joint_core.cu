@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(288, 2)
     for (int item = 0; item < items; ++item, c0 += per) {
       const int k = fk, row = fpos;
       const float* ks = kscale + (int64_t)k * 2 * Mp;
-      const int ke = log2_of(__ldg(kscale + (int64_t)G.q * 2 * Mp + k));  // e - 15
+      // 2^(e - 15) of the component, half of it, and what the accumulators' rounding takes off
+      const float kf = __ldg(kscale + (int64_t)G.q * 2 * Mp + k) * (0.5f * lo_first_gain(4));
       float acc[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) acc[i] = 0.f;
@@ -202,19 +203,10 @@ __global__ void __launch_bounds__(288, 2)
         }
         tc::tmem_wait_st();
       };
-      for (int ch = 0; ch < per; ++ch) {
+      auto chunk = [&](int ch) {
         const int c = c0 + ch, d = c & 1;
         if (ch >= 2) fold(c - 2);  // also: the MMAs have read this buffer
-        if (!FWD && ch % kFold == kFold - 1) put_by(ch < kFold);
-        const float xs = FWD ? __ldg(ks + Mp + ch * kSum + lane) : 1.f;  // 2^(e_j - e)
-        int be[I];  // xs |b| < 2^be, so that 2^(kDataShift - be) b is below 2^kDataShift / xs: finite
-#pragma unroll
-        for (int i = 0; i < I; ++i) {
-          const float m = absmax_nan(0.f, b[i].x, b[i].y);
-          if (FWD) bad = bad || !(m < INFINITY);
-          be[i] = exp_of(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(FWD ? m * xs : m))), -117);
-          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2_wide(be[i] - kDataShift + ke) * lo_first_gain(4);
-        }
+        const float xs = FWD ? __ldg(ks + Mp + ch * kSum + lane) : 1.f;  // 2^(e_j - e), used after K's split
         unsigned char* ad = sa + (size_t)d * 2 * kRowTerm;
         if (FWD) {
           const int r = 32 * q4 + lane;
@@ -247,7 +239,12 @@ __global__ void __launch_bounds__(288, 2)
 #pragma unroll
         for (int i = 0; i < I; ++i) {
           const int n = 2 * (warp + 8 * i);
-          const float sc = pow2f(kDataShift - be[i]);
+          // xs |b| < 2^e, so that 2^(kDataShift - e) b is below 2^kDataShift / xs: finite
+          const float m = absmax_nan(0.f, b[i].x, b[i].y);
+          if (FWD) bad = bad || !(m < INFINITY);
+          const int e = exp_of(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(FWD ? m * xs : m))), -117);
+          if (lane == 0) bscale[c & 3][warp + 8 * i] = pow2f(e - kDataShift + 1) * kf;
+          const float sc = pow2f(kDataShift - e);
           uint32_t h, l;
           split2(FWD ? b[i].x * sc * xs : b[i].x * sc, FWD ? b[i].y * sc * xs : b[i].y * sc, h, l);
           const uint32_t hs = __byte_perm(h, 0, 0x1032), ls = __byte_perm(l, 0, 0x1032);
@@ -267,7 +264,12 @@ __global__ void __launch_bounds__(288, 2)
           fetch(0);
         }
         warp_publish(&ready[d]);
-      }
+      };
+      int ch = 0;
+      if (!FWD)
+        for (; per - ch > kFold; put_by(ch == kFold))
+          for (int end = ch + kFold; ch < end; ++ch) chunk(ch);
+      for (; ch < per; ++ch) chunk(ch);
       if (per > 1) fold(c0 + per - 2);
       fold(c0 + per - 1);
       const int r = 32 * q4 + lane;
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__(288, 2)
             if (s < p) out[(int64_t)s * G.Ct + G.toff[k] + row + r] = make_float2(acc[2 * i], acc[2 * i + 1]);
           }
       } else {
-        if (per >= kFold) {
+        if (per > kFold) {
           const uint32_t t0 = tmem + (uint32_t)(2 * N + half * P) + ((uint32_t)(32 * q4) << 16);
 #pragma unroll
           for (int i = 0; i < I; ++i) {

@@ -29,12 +29,6 @@ __device__ __forceinline__ int exp_of(float m, int least) {
   return max(least, (int)(__float_as_uint(m) >> 23) - 126);
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }  // -126 .. 127
-__device__ __forceinline__ int log2_of(float pow2) { return (int)(__float_as_uint(pow2) >> 23) - 127; }
-// 2^e as the product of two normal floats: a denormal, 0 or infinite where 2^e is
-__device__ __forceinline__ float pow2_wide(int e) {
-  e = min(254, max(-252, e));
-  return pow2f(e >> 1) * pow2f(e - (e >> 1));
-}
 // order of a chunk's 32 summed entries in a 128-byte row: entry of word w of the 16-byte chunk c, so
 // that lane c's entries are two adjacent pairs and 8 lanes read 128 bytes without a gap
 __host__ __device__ constexpr int entry_of(int c, int w) { return 2 * c + (w & 1) + 16 * (w >> 1); }
