@@ -532,7 +532,7 @@ def roofline(inf, w, res, peaks, measured):
                                                    "tc2": "_tc2_kernel", "tc_dc": "_dc_kernel"}.get(name, "_tc_kernel")
     b1 = algorithmic_bytes(inf, w.grid.shape, res["p"])
     if name == "joint":  # bound by its vectors: Table III's flops are not what it computes
-        kern = "joint_planes_fwd_kernel" if dom_fwd else "joint_planes_adj_kernel"
+        kern = "joint form, the product's kernels together"
         gbs, peak = b1 / (dom_ms * 1e-3) / 1e9, peaks.get("hbm_gbs", 6800.0)
         return {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                 "peak_source": "measured copy bandwidth (MEASURED_PEAKS.json)", "kernel": kern, "kernel_ms": dom_ms,

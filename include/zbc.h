@@ -53,7 +53,9 @@ enum {
 typedef enum { ZBC_C64 = 0, ZBC_C128 = 1 } zbc_dtype;
 
 /* Arithmetic form of the product kernels.
- * FP32_SIMT : complex FP32 on CUDA cores (the plain form).
+ * FP32_SIMT : complex FP32 on CUDA cores (the plain form).  A forward whose tiles are fewer than the
+ *             SMs sums its columns in up to 8 slices; where their buffer does not fit, or would have
+ *             to grow during a stream capture, in one, which may change the last bits.
  * TF32X3    : tensor cores, tcgen05 kind::tf32, each operand split hi+lo, 3 products, FP32 accumulation.
  * BF16X3    : tensor cores, tcgen05 kind::f16 with bf16 operands split into 3 terms
  *             (hi+mid+lo), the 6 products above 2^-24, FP32 accumulation.
@@ -79,18 +81,21 @@ typedef enum { ZBC_C64 = 0, ZBC_C128 = 1 } zbc_dtype;
  *             same 1e-5 relative accuracy, but their last bits differ, so AUTO results depend on
  *             the tuning.
  * The joint form (AUTO only): where the factors of all stored columns share small orthonormal bases
- *             B_1, B_2, B_3 per component (each tensor represented to 1e-7 of its norm, below the
- *             rounding of its complex64 factors), Z_j = K_j x1 B_1 x2 B_2 x3 B_3 with cores K_j in
+ *             B_1, B_2, B_3 per component (each tensor represented to 1e-7 of its norm; its
+ *             complex64 factors are rounded to 6e-8), Z_j = K_j x1 B_1 x2 B_2 x3 B_3 with cores K_j in
  *             the bases, and the products sum over the columns' cores and pass between the cores
  *             and the grid once per right-hand side.  The bases and cores are built on the first
  *             AUTO or zbc_tune call (not during a stream capture) and kept with the handle, after the
  *             decompression cache and if they take at most half of the device memory then free;
  *             otherwise, and where a call's workspace does not fit, AUTO runs the other forms
- *             (zbc_tune looks again).  Its tensor-core operands are fp16 hi + lo (22 bits), its sums
- *             FP32.  Largest relative errors against 64 bits, beside FP32_SIMT's: 96^3, 1024 columns,
- *             16 right-hand sides 4.2e-7 / 3.5e-7 (forward / adjoint) against 9.0e-7 / 3.7e-7; 24^3,
- *             64 columns, 1 to 16 right-hand sides 2.3e-7 to 3.0e-7 / 3.1e-7 to 6.0e-7 against 1.5e-7
- *             to 2.7e-7 / 2.2e-7 to 3.6e-7.  A caller who wants plain FP32 asks for FP32_SIMT. */
+ *             (zbc_tune looks again).  That first call takes longer by the build (63 ms at 96^3 /
+ *             1024 columns, 5 ms at 1 mm / 128; the same again after an append): a caller with a
+ *             handful of products to do may name a form instead.
+ *             Its tensor-core operands are fp16 hi + lo (22 bits), its sums FP32.  Largest relative
+ *             errors against 64 bits, beside FP32_SIMT's: 96^3, 1024 columns, 16 right-hand sides
+ *             4.2e-7 / 3.5e-7 (forward / adjoint) against 9.0e-7 / 3.7e-7; 24^3, 64 columns, 1 to 16
+ *             right-hand sides 2.3e-7 to 3.0e-7 / 3.1e-7 to 6.0e-7 against 1.5e-7 to 2.7e-7 / 2.2e-7
+ *             to 3.6e-7.  A caller who wants plain FP32 asks for FP32_SIMT. */
 typedef enum {
   ZBC_FP32_SIMT = 0,
   ZBC_TF32X3 = 1,

@@ -8,7 +8,7 @@
 // so  Y^k = (sum_j K^{kj} X[j, :]) x1 B1 x2 B2 x3 B3  and the adjoint is its transpose: the sum
 // over the columns runs over R1 R2 R3 entries instead of n1 n2 n3 voxels, and the expansion to the
 // grid is done once per right-hand side instead of once per column.  This is the same operator to
-// the tolerance kJointEps, which is below the rounding of the complex64 tensors.
+// the tolerance kJointEps, of the size of the complex64 tensors' rounding.
 #pragma once
 
 #include "zbc_internal.cuh"

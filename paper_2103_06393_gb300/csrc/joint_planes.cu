@@ -3,9 +3,9 @@
 //   forward  Y[:, :, i3] = B1 S,  S = Q[i3] B2^T          (one write of Y)
 //   adjoint  Q[i3] = V conj(B2),  V = B1^H Phi[:, :, i3]  (one read of Phi)
 // The contraction with B1 touches every voxel R1 times and is a tcgen05 GEMM (kind::f16); the one
-// with B2 works on R1 rows and stays in FP32 on the CUDA cores.  Both operands are split into fp16
-// hi + lo (x = hi + lo to 2^-22) after scaling by powers of two and the three products hi hi,
-// hi lo, lo hi are summed in FP32.  In FP32 on the CUDA cores the same planes took 3.1 / 4.7 ms
+// with B2 works on R1 rows: a second GEMM before it in the forward, FP32 on the CUDA cores in the
+// adjoint.  Operands are split into fp16 hi + lo (x = hi + lo to 2^-22) after scaling by powers of two
+// and the three products hi hi, hi lo, lo hi are summed in FP32.  In FP32 on the CUDA cores the same planes took 3.1 / 4.7 ms
 // (320 x 320 x 256, 8 right-hand sides, R = 23-25: 57 % of the FP32 rate) against 0.74 ms that
 // writing or reading the 5 GB takes.
 //
@@ -280,16 +280,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
 // CUDA cores into Q, which stays in registers over the plane's tiles.
 constexpr int kTile2 = 128;   // i2 rows of a tile
 constexpr int kChunk1 = 32;   // i1 per chunk
-constexpr int kStage2 = 32;   // i2 per stage of B2
 constexpr uint32_t kATerm = kTile2 * 128u;
 
-inline size_t planes_adj_smem(int NC) {
+inline size_t planes_adj_smem(int NC, int kStage2) {
   return 4 * (size_t)kATerm + 2 * 2 * 2 * (size_t)NC * 128 + sizeof(float2) * kStage2 * ((NC + 15) / 16 * 16);
 }
 
 // NC = 8 I >= R1, R2 of every component.  VEC: Phi's columns start on 16 bytes, and a lane reads two
 // entries at a time (half the loads; the load unit was the busiest one).
-template <int I, bool VEC>
+// kStage2: i2 per stage of B2, and per FP32 chain of the contraction with it.
+template <int I, bool VEC, int kStage2>
 __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     joint_planes_adj_kernel(const __grid_constant__ JointGeo G, const unsigned char* __restrict__ bop,
                             const float2* __restrict__ b2t, const float2* __restrict__ Phi, int64_t ldphi, int p,
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
         for (int e = 0; e < kStage2 * R2p / 512; ++e)
           ((float4*)b2s)[tid + 256 * e] = __ldg(bsrc + j0 * R2p / 2 + tid + 256 * e);
         worker_barrier();
-        float2 qs[RC][RC];  // the stage's sums: chains of 32 terms
+        float2 qs[RC][RC];  // the stage's sums
         auto pair = [&](int j, bool first) {
           float4 v[RC];
 #pragma unroll
@@ -580,27 +580,39 @@ __global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_const
       i2 < G.n2 && y < G.R[k][1] ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i2] : make_float2(0.f, 0.f);
 }
 
-template <int I, bool VEC>
+template <int I, bool VEC, int kStage2>
 int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
                       int* err, uint32_t polls, cudaStream_t st) {
   const float2* b2t = (const float2*)(bop + bop_bytes(G));
-  ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC>>((int)planes_adj_smem(8 * I))));
-  const size_t sm = planes_adj_smem(8 * I);
+  ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC, kStage2>>((int)planes_adj_smem(8 * I, kStage2))));
+  const size_t sm = planes_adj_smem(8 * I, kStage2);
   const int64_t planes = (int64_t)G.n3 * p * G.q;
   const int grid = (int)std::min<int64_t>(planes, (sm <= 112 * 1024 ? 2 : 1) * sm_count());
-  joint_planes_adj_kernel<I, VEC><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err, polls);
+  joint_planes_adj_kernel<I, VEC, kStage2><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err, polls);
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
 }
 
-template <int I>
+template <int I, int kStage2>
 int planes_adj_vec(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
                    int* err, uint32_t polls, cudaStream_t st) {
   // every column of every plane on 16 bytes, and no pair of entries across the end of one
   if (G.n1 % 2 == 0 && (p == 1 || ldphi % 2 == 0) && (uintptr_t)Phi % 16 == 0)
-    return launch_planes_adj<I, true>(G, bop, Phi, ldphi, p, Q, err, polls, st);
-  return launch_planes_adj<I, false>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+    return launch_planes_adj<I, true, kStage2>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  return launch_planes_adj<I, false, kStage2>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+}
+
+template <int I>
+int planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
+               uint32_t polls, cudaStream_t st) {
+  // Stages of 64 i2 up to rank 24, where they hold no more padding than stages of 32: 1.68 against 1.70 ms for
+  // n2 = 320 (8 right-hand sides), 4.02 against 4.10 ms for 309 (32); but 187 against 160 us for 66 (29).  Above
+  // rank 24 a second CTA an SM, or the registers, would not fit.
+  if constexpr (I <= 3)
+    if (ceil_div(G.n2, 64) * 64 == ceil_div(G.n2, 32) * 32)
+      return planes_adj_vec<I, 64>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  return planes_adj_vec<I, 32>(G, bop, Phi, ldphi, p, Q, err, polls, st);
 }
 
 }  // namespace
@@ -638,14 +650,14 @@ int joint_planes_adj(const JointCache& jc, const float2* Phi, int64_t ldphi, int
                      cudaStream_t st) {
   const JointGeo& G = jc.geo;
   switch (adj_rows(G) / 8) {
-    case 1: return planes_adj_vec<1>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 2: return planes_adj_vec<2>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 3: return planes_adj_vec<3>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 4: return planes_adj_vec<4>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 5: return planes_adj_vec<5>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 6: return planes_adj_vec<6>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    case 7: return planes_adj_vec<7>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
-    default: return planes_adj_vec<8>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 1: return planes_adj<1>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 2: return planes_adj<2>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 3: return planes_adj<3>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 4: return planes_adj<4>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 5: return planes_adj<5>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 6: return planes_adj<6>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    case 7: return planes_adj<7>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
+    default: return planes_adj<8>(G, jc.bop, Phi, ldphi, p, Q, err, polls, st);
   }
 }
 

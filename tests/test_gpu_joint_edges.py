@@ -260,3 +260,13 @@ def test_untuned_class_after_tuning_without_the_joint_form():
     X = _c64(inputs.cn01((40, 12), seed=1))
     assert _rel(_run(h, g, X, True), products.matvec(tens, g.shape, X)) < RTOL
     assert h.device_bytes()["caches"] == held
+
+
+# the adjoint's stages of i2: of 64 where they hold no more padding than stages of 32, several a tile, several tiles
+@pytest.mark.parametrize("n2", [33, 64, 65, 100, 128, 187, 193, 256])
+@pytest.mark.parametrize("n1,r", [(24, 7), (25, 20)])
+def test_stages_of_the_adjoint_planes(n1, n2, r):
+    g, tens = _shared((n1, n2, 10), 40, (r, r, 8), (5, 5, 4))
+    h = zbc.zbc_create_from_host(g, 3, tens)
+    Phi = _c64(inputs.cn01((3 * g.nv, 3), seed=2))
+    assert _rel(_run(h, g, Phi, False), products.rmatvec(tens, g.shape, Phi)) < RTOL
