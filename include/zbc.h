@@ -86,7 +86,7 @@ typedef enum { ZBC_C64 = 0, ZBC_C128 = 1 } zbc_dtype;
  *             the bases, and the products sum over the columns' cores and pass between the cores
  *             and the grid once per right-hand side.  The bases and cores are built on the first
  *             AUTO or zbc_tune call (not during a stream capture) and kept with the handle, after the
- *             decompression cache and if they take at most half of the device memory then free;
+ *             decompression cache and if they leave a fifth of the device memory then free;
  *             otherwise, and where a call's workspace does not fit, AUTO runs the other forms
  *             (zbc_tune looks again).  That first call takes longer by the build (63 ms at 96^3 /
  *             1024 columns, 5 ms at 1 mm / 128; the same again after an append): a caller with a

@@ -413,11 +413,10 @@ static int build(Handle& h, JointCache* jc, cudaStream_t st) {
   // under half of W, less than the operands that tuning would otherwise leave
   jc->large = direct > 1e8;
   if (work > 0.5 * direct || 8.0 * kelems > (jc->large ? 2.0 : 0.5) * wbytes) return ZBC_OK;
-  // and at most half of what the device has free (W is built): the other forms' operands and the
-  // workspaces of later calls have to fit beside it
+  // and it leaves a quarter of its size free (W is built) for the workspaces of the products
   size_t mem_free = 0, mem_total = 0;
   ZBC_TRY_CUDA(cudaMemGetInfo(&mem_free, &mem_total));
-  if (sizeof(float2) * (size_t)kelems > mem_free / 2) return ZBC_ENOMEM;
+  if (sizeof(float2) * (size_t)kelems > mem_free / 5 * 4) return ZBC_ENOMEM;
   cudaError_t e = cudaMalloc(&jc->basis, sizeof(float2) * belems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->K, sizeof(float2) * kelems);
   if (e == cudaSuccess) e = cudaMalloc(&jc->bop, joint_planes_bytes(g));

@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(256) joint_sum_kernel(const float2* __restrict
 }
 
 // From this many right-hand sides on, the column sums run on the tensor cores (at least 8 a
-// pass).  160 x 160 x 128, 4096 columns: whole forward 0.92 ms in FP32 at 4 against 1.40 ms at 8, whole
-// adjoint 1.35 / 2.05 ms in FP32 at 2 / 4 against 1.37 ms at 8.
+// pass).  160 x 160 x 128, 4096 columns: whole forward 0.91 ms in FP32 at 4 against 1.11 ms at 8, whole
+// adjoint 1.33 / 2.05 ms in FP32 at 2 / 4 against 1.04 ms at 4 and 1.23 ms at 8.
 constexpr int kTcFwd = 5, kTcAdj = 3;
 
 int rhs_per_cta(int p) { return p <= 1 ? 1 : p <= 2 ? 2 : 4; }  // FP32 column sums
