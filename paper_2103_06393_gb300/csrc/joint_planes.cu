@@ -288,8 +288,9 @@ inline size_t planes_adj_smem(int NC, int kStage2) {
 
 // NC = 8 I >= R1, R2 of every component.  VEC: Phi's columns start on 16 bytes, and a lane reads two
 // entries at a time (half the loads; the load unit was the busiest one).
-// kStage2: i2 per stage of B2, and per FP32 chain of the contraction with it.
-template <int I, bool VEC, int kStage2>
+// kStage2: i2 per stage of B2, and per FP32 chain of the contraction with it; RAGGED: the last stage ends with
+// the tile's rows.
+template <int I, bool VEC, int kStage2, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
     joint_planes_adj_kernel(const __grid_constant__ JointGeo G, const unsigned char* __restrict__ bop,
                             const float2* __restrict__ b2t, const float2* __restrict__ Phi, int64_t ldphi, int p,
@@ -475,10 +476,11 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
             32 * q4 + lane < done_rows ? make_float2(acc[2 * c], acc[2 * c + 1]) : make_float2(0.f, 0.f);
       const float4* bsrc = (const float4*)(b2t + ((int64_t)k * nt2 + t2) * kTile2 * R2p);
       for (int j0 = 0; j0 < done_rows; j0 += kStage2) {
+        const int je = RAGGED ? min(kStage2, done_rows - j0) : kStage2;
         if (j0 > 0) worker_barrier();
 #pragma unroll
         for (int e = 0; e < kStage2 * R2p / 512; ++e)
-          ((float4*)b2s)[tid + 256 * e] = __ldg(bsrc + j0 * R2p / 2 + tid + 256 * e);
+          if (!RAGGED || e * (512 / R2p) < je) ((float4*)b2s)[tid + 256 * e] = __ldg(bsrc + j0 * R2p / 2 + tid + 256 * e);
         worker_barrier();
         float2 qs[RC][RC];  // the stage's sums
         auto pair = [&](int j, bool first) {
@@ -508,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, I <= 4 ? 2 : 1)
         else
           pair(0, true);
 #pragma unroll 2
-        for (int j = I <= 3 ? 0 : 2; j < kStage2; j += 2) pair(j, false);
+        for (int j = I <= 3 ? 0 : 2; j < je; j += 2) pair(j, false);  // rows past the tile's are zero
 #pragma unroll
         for (int a = 0; a < RC; ++a)
 #pragma unroll
@@ -580,39 +582,45 @@ __global__ void __launch_bounds__(256) transpose_basis_kernel(const __grid_const
       i2 < G.n2 && y < G.R[k][1] ? basis[G.boff[k][1] + (int64_t)y * G.n2 + i2] : make_float2(0.f, 0.f);
 }
 
-template <int I, bool VEC, int kStage2>
+template <int I, bool VEC, int kStage2, bool RAGGED>
 int launch_planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
                       int* err, uint32_t polls, cudaStream_t st) {
   const float2* b2t = (const float2*)(bop + bop_bytes(G));
-  ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC, kStage2>>((int)planes_adj_smem(8 * I, kStage2))));
+  ZBC_TRY((set_smem_limit<joint_planes_adj_kernel<I, VEC, kStage2, RAGGED>>((int)planes_adj_smem(8 * I, kStage2))));
   const size_t sm = planes_adj_smem(8 * I, kStage2);
   const int64_t planes = (int64_t)G.n3 * p * G.q;
   const int grid = (int)std::min<int64_t>(planes, (sm <= 112 * 1024 ? 2 : 1) * sm_count());
-  joint_planes_adj_kernel<I, VEC, kStage2><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err, polls);
+  joint_planes_adj_kernel<I, VEC, kStage2, RAGGED><<<grid, kThreads, sm, st>>>(G, bop, b2t, Phi, ldphi, p, Q, err, polls);
   count_launch();
   ZBC_TRY_CUDA(cudaGetLastError());
   return ZBC_OK;
 }
 
-template <int I, int kStage2>
+template <int I, int kStage2, bool RAGGED>
 int planes_adj_vec(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q,
                    int* err, uint32_t polls, cudaStream_t st) {
   // every column of every plane on 16 bytes, and no pair of entries across the end of one
   if (G.n1 % 2 == 0 && (p == 1 || ldphi % 2 == 0) && (uintptr_t)Phi % 16 == 0)
-    return launch_planes_adj<I, true, kStage2>(G, bop, Phi, ldphi, p, Q, err, polls, st);
-  return launch_planes_adj<I, false, kStage2>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+    return launch_planes_adj<I, true, kStage2, RAGGED>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  return launch_planes_adj<I, false, kStage2, RAGGED>(G, bop, Phi, ldphi, p, Q, err, polls, st);
 }
 
 template <int I>
 int planes_adj(const JointGeo& G, const unsigned char* bop, const float2* Phi, int64_t ldphi, int p, float2* Q, int* err,
                uint32_t polls, cudaStream_t st) {
-  // Stages of 64 i2 up to rank 24, where they hold no more padding than stages of 32: 1.68 against 1.70 ms for
-  // n2 = 320 (8 right-hand sides), 4.02 against 4.10 ms for 309 (32); but 187 against 160 us for 66 (29).  Above
-  // rank 24 a second CTA an SM, or the registers, would not fit.
-  if constexpr (I <= 3)
-    if (ceil_div(G.n2, 64) * 64 == ceil_div(G.n2, 32) * 32)
-      return planes_adj_vec<I, 64>(G, bop, Phi, ldphi, p, Q, err, polls, st);
-  return planes_adj_vec<I, 32>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  // Up to rank 24 stages of 64 i2 where they hold no more padding than stages of 32: 1.68 against 1.70 ms for
+  // n2 = 320 (8 right-hand sides), 4.02 against 4.10 ms for 309 (32).  Where stages of 32 would pad by a
+  // sixteenth or more, stages of 64 of which the last ends with its rows: 138 against 160 us for 66 (29), 379
+  // against 410 us for 74 (13), 78 against 83 us for 135 (11); the loop without a fixed length costs a few per
+  // cent, 1.49 against 1.46 ms for 93 (12), and one stage of 31 rows 235 against 229 us.  Above rank 24 a second
+  // CTA an SM, or the registers, would not fit.
+  if constexpr (I <= 3) {
+    const int rows32 = ceil_div(G.n2, 32) * 32;
+    if (ceil_div(G.n2, 64) * 64 == rows32)
+      return planes_adj_vec<I, 64, false>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+    if (G.n2 > 64 && (rows32 - G.n2) * 16 >= G.n2) return planes_adj_vec<I, 64, true>(G, bop, Phi, ldphi, p, Q, err, polls, st);
+  }
+  return planes_adj_vec<I, 32, false>(G, bop, Phi, ldphi, p, Q, err, polls, st);
 }
 
 }  // namespace

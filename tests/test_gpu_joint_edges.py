@@ -262,8 +262,9 @@ def test_untuned_class_after_tuning_without_the_joint_form():
     assert h.device_bytes()["caches"] == held
 
 
-# the adjoint's stages of i2: of 64 where they hold no more padding than stages of 32, several a tile, several tiles
-@pytest.mark.parametrize("n2", [33, 64, 65, 100, 128, 187, 193, 256])
+# the adjoint's stages of i2: of 64 where they hold no more padding than stages of 32, cut at the rows where they
+# hold more, several a tile, several tiles
+@pytest.mark.parametrize("n2", [31, 33, 64, 65, 67, 81, 96, 100, 128, 129, 159, 187, 193, 256])
 @pytest.mark.parametrize("n1,r", [(24, 7), (25, 20)])
 def test_stages_of_the_adjoint_planes(n1, n2, r):
     g, tens = _shared((n1, n2, 10), 40, (r, r, 8), (5, 5, 4))
